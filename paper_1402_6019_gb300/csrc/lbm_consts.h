@@ -43,7 +43,7 @@ inline double w_belt1(int q) {
 template <typename T>
 inline void fill_step_const(StepConst<T>& C, const lbm_params& p, int nx, int nz, int pitch, long long plane,
                             int ns, int zbc, const double rho_ref[2]) {
-    memset(&C, 0, sizeof C);
+    C = StepConst<T>{};
     C.nx = nx;
     C.nz = nz;
     C.pitch = pitch;
@@ -69,6 +69,13 @@ inline void fill_step_const(StepConst<T>& C, const lbm_params& p, int nx, int nz
             const double wa = p.weight_preset == LBM_WEIGHTS_CHEM09 ? w_belt1(q) : w_attr_paper(q);
             K[q] = wn * (p.G1[ps] * wa + p.G2[ps] * w_rep(q));
             C.sq[s][q] = (T)((q <= 2 ? 0.5 : 0.25) * K[q]);
+        }
+        if constexpr (sizeof(T) == 8) {
+            C.ex[s] = exp_fx_const(p.psi_form == LBM_PSI_EXP ? p.rho0[ps] : 1.0);
+            const double kf[5] = {K[1], K[2], 2.0 * K[4], K[5], 2.0 * K[8]};
+            const double sf[5] = {0.5 * K[1], 0.5 * K[2], K[4], 0.25 * K[5], K[8]};
+            coef_fx(C.kf[s], kf);
+            coef_fx(C.sf[s], sf);
         }
         for (int dz = -2; dz <= 2; ++dz)
             for (int dx = -2; dx <= 2; ++dx) {

@@ -9,6 +9,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "lbm_fixed.cuh"
+
 #if defined(__CUDACC__)
 #define LBM_HD __host__ __device__ __forceinline__
 #else
@@ -28,10 +30,20 @@ LBM_HD constexpr int opp(int l) { return l == 0 ? 0 : (l <= 4 ? (l + 1) % 4 + 1 
 // rest weights of D2Q9: 4/9, 1/9 (axis), 1/36 (diagonal)
 template <typename T> LBM_HD constexpr T wlb(int l) { return l == 0 ? T(4) / T(9) : (l <= 4 ? T(1) / T(9) : T(1) / T(36)); }
 
+// The FP64 step's fixed-point constants per species (lbm_fixed.cuh); the FP32 step has none.
+template <typename T>
+struct FixedConst {};
+template <>
+struct FixedConst<double> {
+    ExpFx ex[2];     // psi = 1 - exp(-rho / rho0)
+    CoefFx kf[2];    // K(1), K(2), 2 K(4), K(5), 2 K(8) of Eq. FORCE
+    CoefFx sf[2];    // sq(1), sq(2), 4 sq(4), sq(5), 4 sq(8) of Appendix A
+};
+
 // Per-step constants, passed to kernels by value (they live in the kernel-parameter
 // constant bank).  Force tables are indexed by the neighbour offset (dz + 2) * 5 + dx + 2.
 template <typename T>
-struct StepConst {
+struct StepConst : FixedConst<T> {
     int nx, nz, pitch, ns;
     int zbc;        // 0 periodic, 1 bounce-back walls
     int psi_form;   // 0 psi = 1 - exp(-rho/rho0), 1 psi = rho
@@ -58,6 +70,10 @@ LBM_HD float psi_of(const StepConst<float>& C, int s, float rho) {
 #endif
 }
 LBM_HD double psi_of(const StepConst<double>& C, int s, double rho) {
+#if defined(__CUDA_ARCH__)
+    // in integers (lbm_fixed.cuh): the FP64 pipe is the scarce one
+    if (C.psi_form == 0 && exp_fx_takes(rho)) return scaled_double((i64)(((u64)1 << 62) - exp_fx(rho, C.ex[s])), -62);
+#endif
     return C.psi_form == 1 ? rho : 1.0 - exp(-rho / C.rho0[s]);
 }
 
@@ -246,15 +262,28 @@ LBM_HD void collide(const StepConst<T>& C, T (&f)[NS][9], const T (&drho)[NS], c
         // even part e + c cu^2 and odd part d cu, axis (W = 1/9) and diagonal (W = 1/36) pairs
         const T e1 = base * T(1.0 / 9.0), c1 = b * T(0.5), d1 = b * T(1.0 / 3.0);
         const T e2 = base * T(1.0 / 36.0), c2 = b * T(0.125), d2 = b * T(1.0 / 12.0);
-        f[s][0] = f[s][0] * keep + base * T(4.0 / 9.0);
+        const T f0 = base * T(4.0 / 9.0);
         const T cu[4] = {ux, uz, ux + uz, uz - ux};  // pairs (1,3), (2,4), (5,7), (6,8)
+        // even part +- odd part = e + cu (c cu +- d): 4 operations a pair, 2 more to keep
+        // (1 - omega) f, which vanishes at tau = 1
+        if (keep == T(0)) {
+            f[s][0] = f0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const T even = k < 2 ? e1 + (c1 * cu[k]) * cu[k] : e2 + (c2 * cu[k]) * cu[k];
-            const T odd = (k < 2 ? d1 : d2) * cu[k];
-            const int lp = k < 2 ? k + 1 : k + 3;  // 1, 2, 5, 6
-            f[s][lp] = (f[s][lp] * keep + even) + odd;
-            f[s][opp(lp)] = (f[s][opp(lp)] * keep + even) - odd;
+            for (int k = 0; k < 4; ++k) {
+                const T e = k < 2 ? e1 : e2, c = (k < 2 ? c1 : c2) * cu[k], d = k < 2 ? d1 : d2;
+                const int lp = k < 2 ? k + 1 : k + 3;  // 1, 2, 5, 6
+                f[s][lp] = (c + d) * cu[k] + e;
+                f[s][opp(lp)] = (c - d) * cu[k] + e;
+            }
+        } else {
+            f[s][0] = f[s][0] * keep + f0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const T e = k < 2 ? e1 : e2, c = (k < 2 ? c1 : c2) * cu[k], d = k < 2 ? d1 : d2;
+                const int lp = k < 2 ? k + 1 : k + 3;
+                f[s][lp] = (c + d) * cu[k] + (f[s][lp] * keep + e);
+                f[s][opp(lp)] = (c - d) * cu[k] + (f[s][opp(lp)] * keep + e);
+            }
         }
     }
 }

@@ -205,6 +205,13 @@ __device__ __forceinline__ void gather_wall(const PullSmem<T, NS, ST, TW>& S, in
         }
 }
 
+// psi as the psi/rho tile holds it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) the bits of
+// psi on the 2^60 scale (lbm_fixed.cuh), whose window sums phase B forms in integers.
+__device__ __forceinline__ float psi_tile(const StepConst<float>& C, int s, float rho) { return psi_of(C, s, rho); }
+__device__ __forceinline__ double psi_tile(const StepConst<double>& C, int s, double rho) {
+    return C.psi_form == 1 ? rho : of_bits((u64)psi_fx(rho, C.ex[s]));
+}
+
 // rho and psi at psi/rho tile position (px, pz) for a position that is not a live site of the
 // tile: the ring, and the padding of ragged tiles.  With walls, rows beyond a wall take the
 // mirror image (or zero, Sec. IV's two readings of the ghost rows).  Positions that no live
@@ -245,7 +252,7 @@ __device__ __forceinline__ void side_density(PullSmem<T, NS, ST, TW>& S, int sl,
         for (int s = 0; s < NS; ++s) {
             const T rho = C.rho_ref[s] + sum[s];
             S.q[qb].rh[s][pz][px] = zero ? T(0) : rho;
-            S.q[qb].ps[s][pz][px] = zero ? T(0) : psi_of(C, s, rho);
+            S.q[qb].ps[s][pz][px] = zero ? T(0) : psi_tile(C, s, rho);
         }
     }
 }
@@ -432,7 +439,7 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
                     drho[s] = sum9(f[s]);
                     const T r = C.rho_ref[s] + drho[s];
                     S.q[qb].rh[s][tz + 2][tx + 2] = r;
-                    S.q[qb].ps[s][tz + 2][tx + 2] = psi_of(C, s, r);
+                    S.q[qb].ps[s][tz + 2][tx + 2] = psi_tile(C, s, r);
                 }
             }
         } else {
@@ -597,6 +604,18 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
                 for (int dz = 0; dz < 5; ++dz)
 #pragma unroll
                     for (int dx = 0; dx < 5; ++dx) p[dz][dx] = Q.ps[s2][tz + dz][tx + dx];
+                if constexpr (sizeof(T) == 8) {
+                    if (C.psi_form == 0) {
+                        i64 w[5][5];
+#pragma unroll
+                        for (int dz = 0; dz < 5; ++dz)
+#pragma unroll
+                            for (int dx = 0; dx < 5; ++dx) w[dz][dx] = (i64)bits_of(p[dz][dx]);
+                        intra_force_fx(C.kf[s2], w, scaled_double(w[2][2], -60), F[s2][0], F[s2][1]);
+                        if (MODE & M_OBS) intra_stress_fx(C.sf[s2], w, sxx, szz, sxz);
+                        continue;
+                    }
+                }
                 intra_force(C, s2, p, F[s2][0], F[s2][1]);
                 if (MODE & M_OBS) intra_stress(C, s2, p, sxx, szz, sxz);
             }
