@@ -80,9 +80,9 @@ struct lbm_ctx {
     int pull_grid[32][2][2] = {};                     // pull: resident CTAs per mode, depth and width (32, 64)
     void* rec = nullptr;                              // pull, M_RECORD pass: where the input state goes
     // pull: boxes in flight per CTA (1 or 2) for passes without [0] and with [1] observables; FP32
-    // defaults from measurements on GB300: FP32 depth 1 (3 CTAs per SM within 80 registers) with
-    // and without observables; FP64 depth 2
-    int stages[2] = {2, 2};
+    // default from measurements on GB300: depth 1 (3 CTAs per SM within 80 registers) with and
+    // without observables; FP64 has one depth, and the setting is only remembered
+    int stages[2] = {1, 1};
     // pull: tile width (32 or 64 columns) of the step passes without [0] and with [1] observables;
     // 64 only in FP32; chosen by lbm_autotune_tiles
     int width[2] = {32, 32};
@@ -91,6 +91,7 @@ struct lbm_ctx {
     InstGeom* inst_d = nullptr;
     std::vector<char> drive_set;  // lattice's drive set by lbm_set_instance_drive
     int ntz_all = 0;              // pull: tile rows of all lattices
+    int pull_pz = 8;              // pull: rows of a tile (8, or 4: pull_tile_rows)
     int prows = 0;                // pull: padded rows of a population plane
     double* host_out = nullptr; // pinned
     StepConst<float> c32{};
@@ -143,7 +144,7 @@ static int fail(lbm_ctx* c, int code, const char* fmt, ...) {
                         cudaGetErrorString(e_), __FILE__, __LINE__);                              \
     } while (0)
 
-static Batch batch(const lbm_ctx* c) { return Batch{c->inst_d, (int)c->inst.size(), c->ntz_all}; }
+static Batch batch(const lbm_ctx* c) { return Batch{c->inst_d, (int)c->inst.size(), c->ntz_all, c->nsm}; }
 
 // Device copy of the lattices' table (geometry and drives).
 static cudaError_t upload_inst(lbm_ctx* c) {
@@ -336,21 +337,26 @@ extern "C" int lbm_create(lbm_ctx** out, const lbm_desc* d) {
     }
     const int nx = d->nx, nz = d->nz, ns = d->n_species;
     c->esize = d->precision == LBM_FP64 ? sizeof(double) : sizeof(float);
-    if (d->precision == LBM_FP32) c->stages[0] = c->stages[1] = 1;
     c->kernel = d->kernel == LBM_KERNEL_AUTO ? LBM_KERNEL_PULL : d->kernel;
     c->pull = c->kernel == LBM_KERNEL_PULL;
     {  // the lattices: rows stacked in order, each with its own ghost rows in the planes
         const int ni = d->n_instances > 1 ? d->n_instances : 1;
         c->inst.assign(ni, InstGeom{});
         c->drive_set.assign(ni, 0);
-        int zrow = 0, prow = 0, trow = 0;
+        int zrow = 0, prow = 0, trow = 0, ntz8 = 0, ntz4 = 0;
+        for (int i = 0; i < ni; ++i) {
+            const int h = ni > 1 ? d->inst_nz[i] : nz;
+            ntz8 += (h + 7) / 8;
+            ntz4 += (h + 3) / 4;
+        }
+        c->pull_pz = pull_tile_rows((int)c->esize, nx, ntz8, ntz4, c->nsm);
         for (int i = 0; i < ni; ++i) {
             InstGeom& g = c->inst[i];
             g.nz = ni > 1 ? d->inst_nz[i] : nz;
             g.zrow0 = zrow;
             g.prow0 = prow;
             g.trow0 = trow;
-            g.ntz = (g.nz + 7) / 8;
+            g.ntz = (g.nz + c->pull_pz - 1) / c->pull_pz;
             zrow += g.nz;
             prow += g.nz + 2 * PULL_GZ;
             trow += g.ntz;
@@ -419,8 +425,9 @@ extern "C" int lbm_create(lbm_ctx** out, const lbm_desc* d) {
             return bail(fail(c, LBM_ECUDA, "cuTensorMapEncodeTiled failed for the two-pass field planes"));
     }
     if (c->pull) {
+        const int narrow = c->pull_pz == 4 ? 4 : 32;  // the shape of a 32-column tile
         for (int b = 0; b < 2; ++b) {
-            if (make_pop_tmap(c->pmap_in[b], c->f[b], (int)c->esize, ns, c->prows, c->pitch, c->plane, 32) != 0)
+            if (make_pop_tmap(c->pmap_in[b], c->f[b], (int)c->esize, ns, c->prows, c->pitch, c->plane, narrow) != 0)
                 return bail(fail(c, LBM_ECUDA, "cuTensorMapEncodeTiled failed for the population buffers"));
             if (d->precision == LBM_FP32 &&
                 make_pop_tmap(c->pmap_wide[b], c->f[b], (int)c->esize, ns, c->prows, c->pitch, c->plane, 64) != 0)
@@ -430,7 +437,7 @@ extern "C" int lbm_create(lbm_ctx** out, const lbm_desc* d) {
         const int modes[5] = {M_WRITE, M_WRITE | M_OBS | per, M_OBS | per, M_FIELDS, M_WRITE | M_RECORD};
         for (int m : modes)
             for (int st = 1; st <= 2; ++st) {
-                const int nb = d->precision == LBM_FP64 ? pull_blocks_per_sm<double>(ns, m, st, 32)
+                const int nb = d->precision == LBM_FP64 ? pull_blocks_per_sm<double>(ns, m, st, narrow)
                                                         : pull_blocks_per_sm<float>(ns, m, st, 32);
                 if (nb < 1) return bail(fail(c, LBM_ECUDA, "occupancy query of the pull kernel failed"));
                 c->pull_grid[m][st - 1][0] = nb * c->nsm;
@@ -605,7 +612,7 @@ static cudaError_t enqueue_pass(lbm_ctx* c, int cur, int mode, bool reduce, bool
         const void* tin = wide ? c->pmap_wide[cur] : c->pmap_in[cur];
         const int grid = c->pull_grid[pm][stg - 1][wide ? 1 : 0];
         if (c->d.precision == LBM_FP64)
-            e = launch_pull<double>(c->d.n_species, pm, stg, 32, tin, (double*)c->f[cur ^ 1], c->c64, O,
+            e = launch_pull<double>(c->d.n_species, pm, stg, c->pull_pz == 4 ? 4 : 32, tin, (double*)c->f[cur ^ 1], c->c64, O,
                                     Rd, c->sched, c->sched_set, B, grid, c->stream, (double*)c->rec);
         else
             e = launch_pull<float>(c->d.n_species, pm, stg, wide ? 64 : 32, tin, (float*)c->f[cur ^ 1], c->c32, O,

@@ -200,17 +200,24 @@ LBM_HD T feq_dev(int l, T drho, T rho, T ux, T uz) {
     return wlb<T>(l) * (drho + rho * (T(3) * cu + T(4.5) * cu * cu - T(1.5) * usq));
 }
 
-// Division and reciprocal: exact IEEE in FP64; in FP32 on the device the fast hardware
-// approximation (a few ulp), well inside the FP32 mode's error budget.
-LBM_HD double div_(double a, double b) { return a / b; }
-LBM_HD float div_(float a, float b) {
+// Reciprocal of a density.  FP64 on the device: within an ulp, in 3 FP64 instructions (rcp_fx; a
+// density outside its range is 0, NaN, Inf or over 1e30, which the step flags, or below 2^-1000).
+// FP32 on the device: the fast hardware approximation (a few ulp), well inside the FP32 mode's
+// error budget.
+LBM_HD double rcp_(double x) {
 #if defined(__CUDA_ARCH__)
-    return __fdividef(a, b);
+    return rcp_fx(x);
 #else
-    return a / b;
+    return 1.0 / x;
 #endif
 }
-
+LBM_HD float rcp_(float x) {
+#if defined(__CUDA_ARCH__)
+    return __fdividef(1.0f, x);
+#else
+    return 1.0f / x;
+#endif
+}
 // The nine equilibria of Sec. II as deviations from W_l rho_ref, using the pair structure of
 // D2Q9: l and its opposite share the even part W (drho + rho (9/2 cu^2 - 3/2 u^2)) and have
 // odd parts +-3 W rho cu.
@@ -231,6 +238,28 @@ LBM_HD void feq9_dev(T drho, T rho, T ux, T uz, T (&fe)[9]) {
     }
 }
 
+// The common velocity u' = sum_s omega_s j_s / sum_s omega_s rho_s: of one species j / rho, with the
+// reciprocal at hand.
+template <typename T, int NS>
+LBM_HD void common_velocity(const StepConst<T>& C, const T (&rho)[NS], const T (&ir)[NS], const T (&jx)[NS],
+                            const T (&jz)[NS], T& upx, T& upz) {
+    if constexpr (NS == 1) {
+        upx = jx[0] * ir[0];
+        upz = jz[0] * ir[0];
+    } else {
+        T nx_ = T(0), nz_ = T(0), den = T(0);
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            nx_ += C.omega[s] * jx[s];
+            nz_ += C.omega[s] * jz[s];
+            den += C.omega[s] * rho[s];
+        }
+        const T iden = rcp_(den);
+        upx = nx_ * iden;
+        upz = nz_ * iden;
+    }
+}
+
 // Shifted-velocity BGK collision of all species at one site (Eq. LB with u_eq = u' + tau F /
 // rho, u' the common velocity sum_s j_s/tau_s / sum_s rho_s/tau_s).  f is overwritten with the
 // post-collision values f + omega (feq - f) = (1 - omega) f + omega feq.  omega is folded into
@@ -241,15 +270,8 @@ LBM_HD void feq9_dev(T drho, T rho, T ux, T uz, T (&fe)[9]) {
 template <typename T, int NS>
 LBM_HD void collide(const StepConst<T>& C, T (&f)[NS][9], const T (&drho)[NS], const T (&rho)[NS],
                     const T (&ir)[NS], const T (&jx)[NS], const T (&jz)[NS], const T (&F)[NS][2]) {
-    T nx_ = T(0), nz_ = T(0), den = T(0);
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        nx_ += C.omega[s] * jx[s];
-        nz_ += C.omega[s] * jz[s];
-        den += C.omega[s] * rho[s];
-    }
-    const T iden = div_(T(1), den);
-    const T upx = nx_ * iden, upz = nz_ * iden;
+    T upx, upz;
+    common_velocity<T, NS>(C, rho, ir, jx, jz, upx, upz);
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
         const T om = C.omega[s], keep = T(1) - om;
@@ -310,21 +332,17 @@ LBM_HD void site_kinetics(const StepConst<T>& C, const T (&f)[NS][9], const T (&
     mx = T(0);
     mz = T(0);
     rtot = T(0);
-    T nx_ = T(0), nz_ = T(0), den = T(0);
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
         mx += jx[s] + T(0.5) * F[s][0];
         mz += jz[s] + T(0.5) * F[s][1];
         rtot += rho[s];
-        nx_ += C.omega[s] * jx[s];
-        nz_ += C.omega[s] * jz[s];
-        den += C.omega[s] * rho[s];
     }
-    const T irt = div_(T(1), rtot);
+    const T irt = NS == 1 ? ir[0] : rcp_(rtot);
     ux = mx * irt;
     uz = mz * irt;
-    const T iden = div_(T(1), den);
-    const T upx = nx_ * iden, upz = nz_ * iden;
+    T upx, upz;
+    common_velocity<T, NS>(C, rho, ir, jx, jz, upx, upz);
     pixz = T(0);
 #pragma unroll
     for (int s = 0; s < NS; ++s) {

@@ -55,7 +55,7 @@ struct InstGeom {
     int nz;       // rows of the lattice
     int zrow0;    // its row 0 among the compact rows of the batch
     int prow0;    // padded plane row of its row -PULL_GZ (its row z sits at prow0 + PULL_GZ + z)
-    int trow0;    // its first tile row in the pull kernel's numbering (tiles of PZ = 8 rows)
+    int trow0;    // its first tile row in the pull kernel's numbering (tiles of 8 rows, or 4: pull_tile_rows)
     int ntz;      // its tile rows
     float g_f;           // g in FP32 (set with g: the FP32 kernels issue no FP64 conversion)
     double g;            // body acceleration along x
@@ -91,11 +91,12 @@ inline void set_inst_drive(InstGeom& I, double g, double wb, double wt) {
     I.wall_u_f[1] = (float)wt;
 }
 // The lattices of a pull-kernel context, as the kernels see them: the device copy of the table,
-// its length, and the tile rows of all lattices together.
+// its length, the tile rows of all lattices together, and the device's SMs.
 struct Batch {
     const InstGeom* inst;
     int ninst;
     int ntz;
+    int nsm;  // SMs of the device
 };
 
 // The lattice holding compact row zg, or tile row tr (binary search over ascending starts).
@@ -168,16 +169,20 @@ struct Fold {
 constexpr int PULL_GX = 4, PULL_GZ = 3;
 
 // Pull-layout kernel: the TMA descriptor (CUtensorMap, 128 bytes at in_map) of one population
-// buffer f ([9 ns][prows][pitch] values) for loading the box of a tile of `width` (32 or 64)
-// columns and its 3-cell ring.  Returns 0 on success.
+// buffer f ([9 ns][prows][pitch] values) for loading the box of a tile of the given shape and its
+// 3-cell ring.  Returns 0 on success.  shape: 32 (32 x 8 sites), 64 (64 x 8, FP32) or 4 (32 x 4, FP64).
 int make_pop_tmap(void* in_map, const void* f, int esize, int ns, int prows, int pitch, long long plane,
-                  int width);
+                  int shape);
+// Rows of the pull kernel's tiles (4 or 8) for lattices of nx columns that have ntz8 tile rows of
+// 8 or ntz4 of 4, on nsm SMs.
+int pull_tile_rows(int precision_bytes, int nx, int ntz8, int ntz4, int nsm);
 // CTAs of the pull kernel resident per SM for a mode, a pipeline depth (stages = boxes in flight
-// per CTA, 1 or 2) and a tile width (32, or 64 for the FP32 step passes M_WRITE, M_WRITE | M_OBS,
-// M_PERIODIC | M_WRITE | M_OBS); sets the kernel's shared-memory limit on the current device; 0
-// on failure or for a width the mode is not built at.
+// per CTA, 1 or 2; FP64 has one depth, whatever stages says) and a tile shape (32 or, for the FP32
+// step passes M_WRITE, M_WRITE | M_OBS, M_PERIODIC | M_WRITE | M_OBS, 64; FP64: 32 or 4); sets the
+// kernel's shared-memory limit on the current device; 0 on failure or for a shape the mode is not
+// built at.
 template <typename T>
-int pull_blocks_per_sm(int ns, int mode, int stages, int width);
+int pull_blocks_per_sm(int ns, int mode, int stages, int shape);
 // One pass of the pull kernel: loads through tin (a buffer's in_map) and stores the new values
 // into fout, the other buffer (their periodic images too).  fold: a pending reduction run by the same launch.  sched: two
 // pairs of work-item counters (tiles, reduction items); consecutive launches of a context
@@ -185,7 +190,7 @@ int pull_blocks_per_sm(int ns, int mode, int stages, int width);
 // zeroes the other pair for the next.
 // grid_max: resident CTAs on the device.
 template <typename T>
-cudaError_t launch_pull(int ns, int mode, int stages, int width, const void* tin, T* fout,
+cudaError_t launch_pull(int ns, int mode, int stages, int shape, const void* tin, T* fout,
                         const StepConst<T>& C, const ObsPtrs& O, const Fold& fold, unsigned* sched, int set,
                         const Batch& B, int grid_max, cudaStream_t st, T* rec = nullptr);
 // One thread waits `cycles` clock cycles on a barrier nothing completes, then sets bit 1 of *flag.

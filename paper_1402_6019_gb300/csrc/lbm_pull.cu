@@ -12,7 +12,7 @@
 // periodic images of the lattice (rows only without walls); the kernel that writes a boundary
 // site also writes its images, so every tile's read is one in-bounds rectangle.
 //
-// Work.  A CTA of TW x PZ threads (one or two warps per tile row; Shape) loops over tiles.  The populations of
+// Work.  A CTA of W x PZ threads (one or two warps per tile row; Shape) loops over tiles.  The populations of
 // the tile and of a 3-cell ring around it (2 cells for the psi stencil of Eq. FORCE, 1 more for
 // the gather, x rounded to a 16-byte boundary) arrive in shared memory with one 3-D
 // cp.async.bulk.tensor load; each warp stores the new populations of its row of 32 sites straight
@@ -43,22 +43,27 @@ namespace lbm {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int PZ = 8;   // tile rows
-constexpr int BZ = PZ + 6;  // box rows: z0 - 3 .. z0 + PZ + 2 (padded z0 .. z0 + PZ + 5)
-constexpr int HH = PZ + 4;  // psi/rho tile rows: z0 - 2 .. z0 + PZ + 1
-// Tile shape: TW columns by PZ rows, one thread per site, TW = 32 (a warp per tile row) or 64 (two
-// warps per tile row).  Row sums are formed per warp, over 32 columns, and column sums over the
-// PZ rows, whatever the width: the partial sums, and so every result, do not depend on the shape.
-template <int TW>
+// Tile shape, a template parameter by its code: W columns by PZ rows, one thread per site.
+//   SHAPE_32 (32 x 8, a warp per tile row), SHAPE_64 (64 x 8, two warps per tile row);
+//   SHAPE_SHORT (32 x 4): FP64 lattices with too few tiles of 8 rows to give every SM its share.
+// Row sums are formed per warp, over 32 columns, and column sums over the PZ rows, whatever the
+// width: with 8 rows the partial sums, and so every result, do not depend on the shape.
+constexpr int SHAPE_32 = 32, SHAPE_64 = 64, SHAPE_SHORT = 4;
+template <int SHP>
 struct Shape {
-    static constexpr int NT = TW * PZ;               // threads
+    static constexpr int W = SHP == SHAPE_64 ? 64 : 32;
+    static constexpr int PZ = SHP == SHAPE_SHORT ? 4 : 8;
+    static constexpr int BZ = PZ + 6;  // box rows: z0 - 3 .. z0 + PZ + 2 (padded z0 .. z0 + PZ + 5)
+    static constexpr int HH = PZ + 4;  // psi/rho tile rows: z0 - 2 .. z0 + PZ + 1
+    static constexpr int NT = W * PZ;                // threads
     static constexpr int NW = NT / 32;               // warps
-    static constexpr int BX = TW + 8;                // box columns: x0 - 4 .. x0 + TW + 3
-    static constexpr int HW = TW + 4;                // psi/rho tile columns: x0 - 2 .. x0 + TW + 1
-    static constexpr int NRING = HW * HH - TW * PZ;  // psi/rho tile positions outside the tile
+    static constexpr int BX = W + 8;                 // box columns: x0 - 4 .. x0 + W + 3
+    static constexpr int HW = W + 4;                 // psi/rho tile columns: x0 - 2 .. x0 + W + 1
+    static constexpr int NRING = HW * HH - W * PZ;   // psi/rho tile positions outside the tile
     static constexpr int RPW = NRING / NW;           // ring positions per warp
-    static_assert(NRING % NW == 0 && RPW <= 32, "the ring shared evenly over the warps");
-    static_assert(NT % RB_THREADS == 0, "a CTA runs the reduction's work items");
+    static constexpr int RR = (RPW + 31) / 32;       // rounds a warp takes for them
+    static_assert(NRING % NW == 0 && RPW <= 64, "the ring shared evenly over the warps");
+    static_assert(NT % RB_THREADS == 0 || RB_THREADS % NT == 0, "a CTA runs the reduction's work items");
 };
 // ST (template parameter): boxes in flight per CTA.  Width 32: 2, tiles loaded two ahead, 2 CTAs
 // per SM in FP32; 1, one ahead, 3 CTAs per SM with fewer registers each.  Width 64: one CTA of 16
@@ -70,15 +75,15 @@ template <typename T, int NS>
 constexpr bool kPair = sizeof(T) == 4 && NS == 2;
 
 // psi and rho of the tile and its 2-cell ring: per species, or (species A, B) pairs
-template <typename T, int NS, int TW, bool PAIR = kPair<T, NS>>
+template <typename T, int NS, int SHP, bool PAIR = kPair<T, NS>>
 struct PsiTile {
-    T ps[NS][HH][Shape<TW>::HW];
-    T rh[NS][HH][Shape<TW>::HW];
+    T ps[NS][Shape<SHP>::HH][Shape<SHP>::HW];
+    T rh[NS][Shape<SHP>::HH][Shape<SHP>::HW];
 };
-template <int TW>
-struct PsiTile<float, 2, TW, true> {
-    f2 ps[HH][Shape<TW>::HW];
-    f2 rh[HH][Shape<TW>::HW];
+template <int SHP>
+struct PsiTile<float, 2, SHP, true> {
+    f2 ps[Shape<SHP>::HH][Shape<SHP>::HW];
+    f2 rh[Shape<SHP>::HH][Shape<SHP>::HW];
 };
 
 // Per-iteration ring of the tiles to work on: iteration k works on the tile described by
@@ -99,16 +104,21 @@ struct TileInfo {
     T g, wall[2];   // its lattice's drive
 };
 
-template <typename T, int NS, int ST, int TW>
+template <typename T, int NS, int ST, int SHP>
 struct PullSmem {
-    T box[ST][9 * NS][BZ][Shape<TW>::BX];  // TMA destinations (column bx = x - x0 + 4, row bz = z - z0 + 3)
-    PsiTile<T, NS, TW> q[2];    // by iteration parity: tile k + 1 fills one while tile k reads the other
-    T colsum[2][PZ][NQC][TW];   // by iteration parity: summed over the tile's rows one tile later
-    typename Red<T>::A wsc[Shape<TW>::NW][NSC];  // folded reduction: per-warp scalars
+    using SH = Shape<SHP>;
+    // psi / rho tiles: two by iteration parity, so that tile k + 1 fills one while tile k reads the
+    // other; one in FP64, which then fits two CTAs on an SM (the FP64 pipe needs the warps: 8 per SM
+    // kept it 67 % busy) at the price of a second barrier per tile
+    static constexpr int QB = sizeof(T) == 8 ? 1 : 2;
+    T box[ST][9 * NS][SH::BZ][SH::BX];  // TMA destinations (column bx = x - x0 + 4, row bz = z - z0 + 3)
+    PsiTile<T, NS, SHP> q[QB];
+    T colsum[2][SH::PZ][NQC][SH::W];    // by iteration parity: summed over the tile's rows one tile later
+    typename Red<T>::A wsc[SH::NW > RB_THREADS / 32 ? SH::NW : RB_THREADS / 32][NSC];  // folded reduction: per-warp scalars
     alignas(8) unsigned long long bar[ST];
     TileInfo<T> ti[NTQ];
     int fold_item;  // the reduction work item thread 0 drew for the CTA
-    unsigned short ring[Shape<TW>::NT];  // observing builds: ring position of thread tid, rpz << 8 | rpx
+    unsigned short ring[SH::NT];  // observing builds: ring position of thread tid, rpz << 8 | rpx
 };
 
 // Tile t of the work order; rot > 0 (one periodic lattice): the order starts rot tiles in, at
@@ -117,7 +127,7 @@ struct PullSmem {
 // rows in the opposite direction -- rows 0, ntz - 1, ntz - 2, ..., 1 when periodic (the image rows
 // still first), ntz - 1 .. 0 between walls -- so that a launch starts on the rows the launch
 // before wrote last, which may still be in L2.
-template <typename T, int TW>
+template <typename T, int SHP>
 __device__ __forceinline__ void describe(TileInfo<T>& D, int t, int ntiles, const InstGeom* __restrict__ inst,
                                          int ninst, int ntx, int rot, int rev) {
     D.t = t;
@@ -132,8 +142,8 @@ __device__ __forceinline__ void describe(TileInfo<T>& D, int t, int ntiles, cons
         tl = tl < ntiles - rot ? tl + rot : tl - (ntiles - rot);
     }
     const int j = tl / ntx;
-    D.x0 = (tl - j * ntx) * TW;
-    D.z0 = j * PZ;
+    D.x0 = (tl - j * ntx) * Shape<SHP>::W;
+    D.z0 = j * Shape<SHP>::PZ;
     D.jg = I.trow0 + j;
     D.lnz = I.nz;
     D.zrow0 = I.zrow0;
@@ -145,9 +155,9 @@ __device__ __forceinline__ void describe(TileInfo<T>& D, int t, int ntiles, cons
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
-template <typename T, int NS, int ST, int TW>
-__device__ __forceinline__ void issue_load(PullSmem<T, NS, ST, TW>& S, const CUtensorMap* map, int x, int z, int sl) {
-    constexpr unsigned bytes = (unsigned)(sizeof(T) * 9 * NS * BZ * Shape<TW>::BX);
+template <typename T, int NS, int ST, int SHP>
+__device__ __forceinline__ void issue_load(PullSmem<T, NS, ST, SHP>& S, const CUtensorMap* map, int x, int z, int sl) {
+    constexpr unsigned bytes = (unsigned)(sizeof(T) * 9 * NS * Shape<SHP>::BZ * Shape<SHP>::BX);
     const unsigned bar = smem_u32(&S.bar[sl]);
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
     asm volatile(
@@ -186,15 +196,15 @@ __global__ void k_wait_selftest(int* flag, long long limit) {
 // Post-streaming populations at box position (bx, bz): the gather of the pull layout.  lo / hi:
 // the site is the bottom / top row next to a wall, where populations coming from beyond the
 // wall are the site's own reflected values.
-template <typename T, int NS, int ST, int TW>
-__device__ __forceinline__ void gather(const PullSmem<T, NS, ST, TW>& S, int sl, int bx, int bz, T (&f)[NS][9]) {
+template <typename T, int NS, int ST, int SHP>
+__device__ __forceinline__ void gather(const PullSmem<T, NS, ST, SHP>& S, int sl, int bx, int bz, T (&f)[NS][9]) {
 #pragma unroll
     for (int s = 0; s < NS; ++s)
 #pragma unroll
         for (int l = 0; l < 9; ++l) f[s][l] = S.box[sl][s * 9 + l][bz - cz(l)][bx - cx(l)];
 }
-template <typename T, int NS, int ST, int TW>
-__device__ __forceinline__ void gather_wall(const PullSmem<T, NS, ST, TW>& S, int sl, int bx, int bz, bool lo, bool hi,
+template <typename T, int NS, int ST, int SHP>
+__device__ __forceinline__ void gather_wall(const PullSmem<T, NS, ST, SHP>& S, int sl, int bx, int bz, bool lo, bool hi,
                                             T (&f)[NS][9]) {
 #pragma unroll
     for (int s = 0; s < NS; ++s)
@@ -206,7 +216,7 @@ __device__ __forceinline__ void gather_wall(const PullSmem<T, NS, ST, TW>& S, in
 }
 
 // psi as the psi/rho tile holds it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) the bits of
-// psi on the 2^60 scale (lbm_fixed.cuh), whose window sums phase B forms in integers.
+// psi on the 2^56 scale (lbm_fixed.cuh), whose window sums phase B forms in integers.
 __device__ __forceinline__ float psi_tile(const StepConst<float>& C, int s, float rho) { return psi_of(C, s, rho); }
 __device__ __forceinline__ double psi_tile(const StepConst<double>& C, int s, double rho) {
     return C.psi_form == 1 ? rho : of_bits((u64)psi_fx(rho, C.ex[s]));
@@ -216,9 +226,10 @@ __device__ __forceinline__ double psi_tile(const StepConst<double>& C, int s, do
 // tile: the ring, and the padding of ragged tiles.  With walls, rows beyond a wall take the
 // mirror image (or zero, Sec. IV's two readings of the ghost rows).  Positions that no live
 // site reads (far padding of ragged tiles) are set to zero.
-template <typename T, int NS, int ST, int TW>
-__device__ __forceinline__ void side_density(PullSmem<T, NS, ST, TW>& S, int sl, int qb, const StepConst<T>& C,
-                                             const PairConst& K, int px, int pz, int z0, int nz, bool WALL) {
+// side_sum returns false for those, else the sums of the populations there.
+template <typename T, int NS, int ST, int SHP>
+__device__ __forceinline__ bool side_sum(PullSmem<T, NS, ST, SHP>& S, int sl, const StepConst<T>& C, int px, int pz,
+                                         int z0, int nz, bool WALL, T (&sum)[NS]) {
     const int Z = z0 - 2 + pz;
     int Zs = Z;
     bool zero = false;
@@ -229,20 +240,26 @@ __device__ __forceinline__ void side_density(PullSmem<T, NS, ST, TW>& S, int sl,
             Zs = mirror_index(Z, nz);
     }
     const int bz = Zs - z0 + 3, bx = px + 2;
-    if (bz < 1 || bz > BZ - 2) zero = true;
-    T sum[NS];
+    if (bz < 1 || bz > Shape<SHP>::BZ - 2) zero = true;
 #pragma unroll
     for (int s = 0; s < NS; ++s) sum[s] = T(0);
     if (!zero) {
         T g[NS][9];
         const bool lo = WALL && Zs == 0, hi = WALL && Zs == nz - 1;
         if (WALL && (lo || hi))
-            gather_wall<T, NS, ST, TW>(S, sl, bx, bz, lo, hi, g);
+            gather_wall<T, NS, ST, SHP>(S, sl, bx, bz, lo, hi, g);
         else
-            gather<T, NS, ST, TW>(S, sl, bx, bz, g);
+            gather<T, NS, ST, SHP>(S, sl, bx, bz, g);
 #pragma unroll
         for (int s = 0; s < NS; ++s) sum[s] = sum9(g[s]);
     }
+    return !zero;
+}
+template <typename T, int NS, int ST, int SHP>
+__device__ __forceinline__ void side_density(PullSmem<T, NS, ST, SHP>& S, int sl, int qb, const StepConst<T>& C,
+                                             const PairConst& K, int px, int pz, int z0, int nz, bool WALL) {
+    T sum[NS];
+    const bool zero = !side_sum<T, NS, ST, SHP>(S, sl, C, px, pz, z0, nz, WALL, sum);
     if constexpr (kPair<T, NS>) {
         const f2 rho = add2(K.rho_ref, p2(sum[0], sum[1]));
         S.q[qb].rh[pz][px] = zero ? sp(0.f) : rho;
@@ -293,10 +310,10 @@ __device__ __noinline__ void write_images(const StepConst<T>& C, T* __restrict__
 // Ring position (psi/rho tile coordinates) of lane `lane` < RPW of warp `warp`: every warp has the
 // same phase-A work (22 positions per warp at width 32, 19 at width 64); in ring order the top two
 // rows, the bottom two rows, then two columns on each side of the tile rows.
-template <int TW>
+template <int SHP>
 __device__ __forceinline__ void ring_position(int lane, int warp, int& rpx, int& rpz) {
-    constexpr int HW = Shape<TW>::HW;
-    const int k = warp * Shape<TW>::RPW + lane;
+    constexpr int HW = Shape<SHP>::HW, HH = Shape<SHP>::HH;
+    const int k = warp * Shape<SHP>::RPW + lane;
     if (k < 2 * HW) {
         rpz = k / HW;
         rpx = k % HW;
@@ -311,8 +328,9 @@ __device__ __forceinline__ void ring_position(int lane, int warp, int& rpx, int&
     }
 }
 
-template <typename T, int NS, int MODE, int ST, int TW>
-__global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 ? (ST == 2 ? 2 : 3) : 1))
+template <typename T, int NS, int MODE, int ST, int SHP>
+__global__ void __launch_bounds__(Shape<SHP>::NT,
+                                  SHP == SHAPE_64 ? 1 : (sizeof(T) == 4 ? (ST == 2 ? 2 : 3) : 2))
     k_pull(const __grid_constant__ CUtensorMap tin, T* __restrict__ fout,
            const StepConst<T> C, const PairConst K, const ObsPtrs O, const Fold Rd, unsigned* __restrict__ ctr,
            unsigned* __restrict__ ctr_next, const InstGeom* __restrict__ inst, int ninst, int ntx, int ntz,
@@ -320,9 +338,10 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
     // walls in z: never in the periodic build, else as the step constants say
     const bool WALL = (MODE & M_PERIODIC) ? false : C.zbc != 0;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    using SH = Shape<TW>;
-    PullSmem<T, NS, ST, TW>& S = *reinterpret_cast<PullSmem<T, NS, ST, TW>*>(smem_raw);
-    const int tx = threadIdx.x, tz = threadIdx.y, tid = tz * TW + tx;
+    using SH = Shape<SHP>;
+    constexpr int PZ = SH::PZ, TW = SH::W, QB = PullSmem<T, NS, ST, SHP>::QB;
+    PullSmem<T, NS, ST, SHP>& S = *reinterpret_cast<PullSmem<T, NS, ST, SHP>*>(smem_raw);
+    const int tx = threadIdx.x, tz = threadIdx.y, tid = tz * Shape<SHP>::W + tx;
     const int nx = C.nx, nz = C.nz;
     const int ntiles = ntx * ntz;  // nz: rows of all lattices; ntz: their tile rows
     // tiles 0 .. nstat - 1 are owned by CTA (tile mod grid), the rest come from ctr[0]
@@ -337,8 +356,8 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
     // registers are short), the others keep it in registers
     const bool ring = (tid & 31) < SH::RPW;
     int rpx0 = 0, rpz0 = 0;
-    if (ring) ring_position<TW>(tid & 31, tid >> 5, rpx0, rpz0);
-    if constexpr ((MODE & M_OBS) != 0) S.ring[tid] = (unsigned short)(rpz0 << 8 | rpx0);
+    if (ring) ring_position<SHP>(tid & 31, tid >> 5, rpx0, rpz0);
+    if constexpr ((MODE & M_OBS) != 0 && sizeof(T) == 4) S.ring[tid] = (unsigned short)(rpz0 << 8 | rpx0);
     // thread 0 draws tiles one ahead of their loads, so the counter's latency is hidden;
     // ntiles: nothing more to draw
     int upcoming = ntiles;
@@ -351,8 +370,11 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&tin) : "memory");
         for (int sl = 0; sl < ST; ++sl) {
             const int t = (int)blockIdx.x + sl * (int)gridDim.x;
-            if (t < nstat) describe<T, TW>(S.ti[sl], t, ntiles, inst, ninst, ntx, rot, rev);
+            if (t < nstat) describe<T, SHP>(S.ti[sl], t, ntiles, inst, ninst, ntx, rot, rev);
         }
+    }
+    if constexpr (sizeof(T) == 8) {  // the exponential's table into L1 meanwhile
+        if (tid < 8) asm volatile("prefetch.global.L1 [%0];\n" ::"l"(exp2_table_dev + 16 * tid));
     }
     // Programmatic dependent launch: the next step's CTAs may be scheduled as soon as this grid's
     // CTAs start retiring; every thread of a grid waits for the previous grid's completion (and
@@ -372,7 +394,7 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
             if (!more) break;  // the slots after the CTA's first non-tile item stay unused
             const int t = (int)blockIdx.x + sl * (int)gridDim.x;
             if (t >= nstat)
-                describe<T, TW>(S.ti[sl], min(nstat + (int)atomicAdd(ctr, 1u), ntiles), ntiles, inst, ninst, ntx,
+                describe<T, SHP>(S.ti[sl], min(nstat + (int)atomicAdd(ctr, 1u), ntiles), ntiles, inst, ninst, ntx,
                                 rot, rev);
             more = S.ti[sl].t < ntiles;
             if (more && sl == 0) issue_load(S, &tin, S.ti[0].x0, S.ti[0].prow0 + S.ti[0].z0, 0);
@@ -388,11 +410,11 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
     int prev_x = -1, prev_jg = 0;
     int k = 0;
     for (;; ++k) {
-        const int sl = k % ST, qb = k & 1;
+        const int sl = k % ST, qb = k & 1, qi = qb & (QB - 1);
         const TileInfo<T> D = S.ti[k % NTQ];
         if (D.t >= ntiles) break;
         if (tid == 0)  // publish the tile of iteration k + ST, one barrier ahead of its readers
-            describe<T, TW>(S.ti[(k + ST) % NTQ], upcoming, ntiles, inst, ninst, ntx, rot, rev);
+            describe<T, SHP>(S.ti[(k + ST) % NTQ], upcoming, ntiles, inst, ninst, ntx, rot, rev);
         // this tile: first column and row (rows of its lattice), tile row among all lattices; its
         // lattice: rows, first compact row, first padded row (the observing builds read them again
         // from shared memory after the tile barrier, so that they hold no registers across it)
@@ -413,9 +435,9 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
         if (live) {
             const bool lo = WALL && z == 0, hi = WALL && z == lnz - 1;
             if (WALL && (lo || hi))
-                gather_wall<T, NS, ST, TW>(S, sl, tx + 4, tz + 3, lo, hi, f);
+                gather_wall<T, NS, ST, SHP>(S, sl, tx + 4, tz + 3, lo, hi, f);
             else
-                gather<T, NS, ST, TW>(S, sl, tx + 4, tz + 3, f);
+                gather<T, NS, ST, SHP>(S, sl, tx + 4, tz + 3, f);
             if constexpr ((MODE & M_RECORD) != 0) {  // the input state, as plain values (one lattice)
                 const long long n = (long long)nx * nz, i = (long long)z * nx + x;
 #pragma unroll
@@ -431,30 +453,74 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
                 drho[0] = d.x;
                 drho[NS - 1] = d.y;
                 const f2 r = add2(K.rho_ref, d);
-                S.q[qb].rh[tz + 2][tx + 2] = r;
-                S.q[qb].ps[tz + 2][tx + 2] = psi2(C, K, r);
+                S.q[qi].rh[tz + 2][tx + 2] = r;
+                S.q[qi].ps[tz + 2][tx + 2] = psi2(C, K, r);
             } else {
 #pragma unroll
                 for (int s = 0; s < NS; ++s) {
                     drho[s] = sum9(f[s]);
-                    const T r = C.rho_ref[s] + drho[s];
-                    S.q[qb].rh[s][tz + 2][tx + 2] = r;
-                    S.q[qb].ps[s][tz + 2][tx + 2] = psi_tile(C, s, r);
+                    if constexpr (sizeof(T) == 4) {
+                        const T r = C.rho_ref[s] + drho[s];
+                        S.q[qi].rh[s][tz + 2][tx + 2] = r;
+                        S.q[qi].ps[s][tz + 2][tx + 2] = psi_tile(C, s, r);
+                    }
                 }
             }
-        } else {
-            side_density<T, NS, ST, TW>(S, sl, qb, C, K, tx + 2, tz + 2, z0, lnz, WALL);
+        } else if constexpr (sizeof(T) == 4) {
+            side_density<T, NS, ST, SHP>(S, sl, qi, C, K, tx + 2, tz + 2, z0, lnz, WALL);
         }
-        if (ring) {
+        if constexpr (sizeof(T) == 8) {
+            // the thread's own position and its ring positions: their sums first, then their psi
+            // side by side, so that the exponentials' dependent integer chains overlap
+            T sum[SH::RR + 1][NS];
+            int px[SH::RR + 1], pz[SH::RR + 1];
+            bool in[SH::RR + 1], has[SH::RR + 1];
+            px[0] = tx + 2;
+            pz[0] = tz + 2;
+            in[0] = has[0] = true;
+            if (live) {
+#pragma unroll
+                for (int s = 0; s < NS; ++s) sum[0][s] = drho[s];
+            } else {
+                has[0] = side_sum<T, NS, ST, SHP>(S, sl, C, px[0], pz[0], z0, lnz, WALL, sum[0]);
+            }
+#pragma unroll
+            for (int r = 0; r < SH::RR; ++r) {
+                const int i = (tid & 31) + 32 * r;
+                in[r + 1] = i < SH::RPW;
+                has[r + 1] = false;
+                px[r + 1] = pz[r + 1] = 0;
+#pragma unroll
+                for (int s = 0; s < NS; ++s) sum[r + 1][s] = T(0);
+                if (in[r + 1]) {
+                    ring_position<SHP>(i, tid >> 5, px[r + 1], pz[r + 1]);
+                    has[r + 1] = side_sum<T, NS, ST, SHP>(S, sl, C, px[r + 1], pz[r + 1], z0, lnz, WALL, sum[r + 1]);
+                }
+            }
+            T ps[SH::RR + 1][NS];
+#pragma unroll
+            for (int r = 0; r <= SH::RR; ++r)
+#pragma unroll
+                for (int s = 0; s < NS; ++s) ps[r][s] = psi_tile(C, s, C.rho_ref[s] + sum[r][s]);
+#pragma unroll
+            for (int r = 0; r <= SH::RR; ++r)
+                if (in[r]) {
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        S.q[qi].rh[s][pz[r]][px[r]] = has[r] ? C.rho_ref[s] + sum[r][s] : T(0);
+                        S.q[qi].ps[s][pz[r]][px[r]] = has[r] ? ps[r][s] : T(0);
+                    }
+                }
+        } else if (ring) {
             int rpx = rpx0, rpz = rpz0;
             if constexpr ((MODE & M_OBS) != 0) {
                 const unsigned rp = S.ring[tid];
                 rpx = (int)(rp & 255u);
                 rpz = (int)(rp >> 8);
             }
-            side_density<T, NS, ST, TW>(S, sl, qb, C, K, rpx, rpz, z0, lnz, WALL);
+            side_density<T, NS, ST, SHP>(S, sl, qi, C, K, rpx, rpz, z0, lnz, WALL);
         }
-        // the only CTA barrier of a tile: psi / rho of the tile and ring complete, box sl read
+        // the CTA barrier of a tile (in FP64 a second one ends it): psi / rho of the tile and ring complete, box sl read
         // by all, the previous tile's column sums written
         if (__syncthreads_or(!ok)) {
             failed = true;
@@ -499,7 +565,7 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
         }
 
         // ---- phase B: interaction, collision, new stored values, observables ----
-        const PsiTile<T, NS, TW>& Q = S.q[qb];
+        const PsiTile<T, NS, SHP>& Q = S.q[qi];
         T rowq[NQR];
 #pragma unroll
         for (int q = 0; q < NQR; ++q) rowq[q] = T(0);
@@ -611,7 +677,7 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
                         for (int dz = 0; dz < 5; ++dz)
 #pragma unroll
                             for (int dx = 0; dx < 5; ++dx) w[dz][dx] = (i64)bits_of(p[dz][dx]);
-                        intra_force_fx(C.kf[s2], w, scaled_double(w[2][2], -60), F[s2][0], F[s2][1]);
+                        intra_force_fx(C.kf[s2], w, scaled_double(w[2][2], -56), F[s2][0], F[s2][1]);
                         if (MODE & M_OBS) intra_stress_fx(C.sf[s2], w, sxx, szz, sxz);
                         continue;
                     }
@@ -637,7 +703,7 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
                 for (int s2 = 0; s2 < NS; ++s2) {
                     rho[s2] = C.rho_ref[s2] + drho[s2];
                     if (!(rho[s2] > T(0)) || !(rho[s2] < T(1e30))) bad = 1;
-                    ir[s2] = div_(T(1), rho[s2]);
+                    ir[s2] = rcp_(rho[s2]);
                     momentum9(f[s2], jx[s2], jz[s2]);
                     F[s2][0] += rho[s2] * S.ti[k % NTQ].g;
                 }
@@ -776,6 +842,7 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
             S.colsum[qb][tz][QC_PS][tx] = cps;
             S.colsum[qb][tz][QC_PXX][tx] = cpx;
         }
+        if constexpr (QB == 1) __syncthreads();  // the one psi / rho tile is read by all
     }
     if ((MODE & M_OBS) && !failed) {
         // the last tile's per-column sums
@@ -794,7 +861,7 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
             __syncthreads();
             const int b = S.fold_item;
             if (b >= nfold) break;  // uniform: every thread read the same item
-            reduce_block<T, (TW > 32)>(b, Rd.part_row, Rd.part_col, O.flag, Rd.nxpart, Rd.nzpart, nx, nz, C.zbc, nrb, Rd.out,
+            reduce_block<T, SH::NW>(b, Rd.part_row, Rd.part_col, O.flag, Rd.nxpart, Rd.nzpart, nx, nz, C.zbc, nrb, Rd.out,
                             Rd.avg, Rd.bpart, Rd.bavg, Rd.accumulate, T(Rd.inx), T(Rd.inz), S.wsc,
                             ninst > 1 ? inst : nullptr, ninst);  // ends with a CTA barrier
         }
@@ -810,24 +877,25 @@ __global__ void __launch_bounds__(Shape<TW>::NT, TW == 64 ? 1 : (sizeof(T) == 4 
     }
 }
 
-template <typename T, int NS, int MODE, int ST, int TW>
+template <typename T, int NS, int MODE, int ST, int SHP>
 int pull_occupancy() {
-    const size_t smem = sizeof(PullSmem<T, NS, ST, TW>);
-    if (cudaFuncSetAttribute(k_pull<T, NS, MODE, ST, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    const size_t smem = sizeof(PullSmem<T, NS, ST, SHP>);
+    // a short tile's launch may ask for 116 KB (launch_mode)
+    if (cudaFuncSetAttribute(k_pull<T, NS, MODE, ST, SHP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             SHP == SHAPE_SHORT ? 116 * 1024 : (int)smem) != cudaSuccess)
         return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pull<T, NS, MODE, ST, TW>, Shape<TW>::NT, smem) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pull<T, NS, MODE, ST, SHP>, Shape<SHP>::NT, smem) !=
         cudaSuccess)
         return 0;
     return nb;
 }
 
-template <typename T, int NS, int MODE, int ST, int TW>
+template <typename T, int NS, int MODE, int ST, int SHP>
 cudaError_t launch_mode(const void* tin, T* fout, const StepConst<T>& C, const ObsPtrs& O,
                         const Fold& Rd, unsigned* sched, int set, const Batch& B, int grid_max, cudaStream_t st,
                         T* rec) {
-    const int ntx = (C.nx + TW - 1) / TW;
+    const int ntx = (C.nx + Shape<SHP>::W - 1) / Shape<SHP>::W;
     const long long ntiles = (long long)ntx * B.ntz;
     int grid = (int)(ntiles < grid_max ? ntiles : grid_max);
     if (Rd.enabled && grid < 1) grid = 1;
@@ -835,17 +903,22 @@ cudaError_t launch_mode(const void* tin, T* fout, const StepConst<T>& C, const O
     if constexpr (kPair<T, NS>) fill_pair_const(K, C);
     // launched with programmatic stream serialisation: it may start while the kernel before it
     // on the stream drains, and waits for it in its prologue (griddepcontrol.wait)
+    constexpr size_t ONE_PER_SM = 116 * 1024;
+    static_assert(SHP != SHAPE_SHORT || sizeof(PullSmem<T, NS, ST, SHP>) <= ONE_PER_SM, "shared memory of a short tile");
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(TW, PZ);
-    cfg.dynamicSmemBytes = sizeof(PullSmem<T, NS, ST, TW>);
+    cfg.blockDim = dim3(Shape<SHP>::W, Shape<SHP>::PZ);
+    cfg.dynamicSmemBytes = sizeof(PullSmem<T, NS, ST, SHP>);
+    // no more short tiles than SMs: one CTA per SM (it asks for over half the shared memory), or a
+    // launch that starts while the last one drains doubles up on the SMs that are free first
+    if (SHP == SHAPE_SHORT && ntiles <= B.nsm) cfg.dynamicSmemBytes = ONE_PER_SM;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_pull<T, NS, MODE, ST, TW>, *static_cast<const CUtensorMap*>(tin), fout, C, K,
+    return cudaLaunchKernelEx(&cfg, k_pull<T, NS, MODE, ST, SHP>, *static_cast<const CUtensorMap*>(tin), fout, C, K,
                               O, Rd, sched + 2 * set, sched + 2 * (set ^ 1), B.inst, B.ninst, ntx, B.ntz, rec,
                               set & 1);
 }
@@ -856,13 +929,13 @@ bool wide_pass(int mode) {
     return sizeof(T) == 4 && (mode == M_WRITE || mode == (M_WRITE | M_OBS) || mode == (M_PERIODIC | M_WRITE | M_OBS));
 }
 
-template <typename T, int NS, int ST, int TW>
+template <typename T, int NS, int ST, int SHP>
 cudaError_t launch_ns(int mode, const void* tin, T* fout, const StepConst<T>& C,
                       const ObsPtrs& O, const Fold& Rd, unsigned* sched, int set, const Batch& B, int grid_max,
                       cudaStream_t st, T* rec) {
 #define LBM_PULL_CASE(m) \
-    case m: return launch_mode<T, NS, m, ST, TW>(tin, fout, C, O, Rd, sched, set, B, grid_max, st, rec);
-    if constexpr (TW == 32) {
+    case m: return launch_mode<T, NS, m, ST, SHP>(tin, fout, C, O, Rd, sched, set, B, grid_max, st, rec);
+    if constexpr (SHP != SHAPE_64) {
         switch (mode) {
             LBM_PULL_CASE(M_WRITE)
             LBM_PULL_CASE(M_WRITE | M_OBS)
@@ -918,11 +991,11 @@ __global__ void k_images(int ns, T* __restrict__ f, const StepConst<T> C, const 
 
 }  // namespace
 
-template <typename T, int NS, int ST, int TW>
+template <typename T, int NS, int ST, int SHP>
 int blocks_per_sm_ns(int mode) {
 #define LBM_PULL_CASE(m) \
-    case m: return pull_occupancy<T, NS, m, ST, TW>();
-    if constexpr (TW == 32) {
+    case m: return pull_occupancy<T, NS, m, ST, SHP>();
+    if constexpr (SHP != SHAPE_64) {
         switch (mode) {
             LBM_PULL_CASE(M_WRITE)
             LBM_PULL_CASE(M_WRITE | M_OBS)
@@ -946,39 +1019,53 @@ int blocks_per_sm_ns(int mode) {
 #undef LBM_PULL_CASE
 }
 
-template <typename T, int ST, int TW>
+template <typename T, int ST, int SHP>
 int blocks_per_sm(int ns, int mode) {
-    return ns == 1 ? blocks_per_sm_ns<T, 1, ST, TW>(mode) : blocks_per_sm_ns<T, 2, ST, TW>(mode);
+    return ns == 1 ? blocks_per_sm_ns<T, 1, ST, SHP>(mode) : blocks_per_sm_ns<T, 2, ST, SHP>(mode);
 }
 
 template <typename T>
-int pull_blocks_per_sm(int ns, int mode, int stages, int width) {
-    if (width == 64) {
-        if (!wide_pass<T>(mode)) return 0;
-        return stages == 1 ? blocks_per_sm<T, 1, 64>(ns, mode) : blocks_per_sm<T, 2, 64>(ns, mode);
+int pull_blocks_per_sm(int ns, int mode, int stages, int shape) {
+    if constexpr (sizeof(T) == 8) {
+        return shape == SHAPE_SHORT ? blocks_per_sm<T, 1, SHAPE_SHORT>(ns, mode) : blocks_per_sm<T, 1, SHAPE_32>(ns, mode);
+    } else {
+        if (shape == SHAPE_64) {
+            if (!wide_pass<T>(mode)) return 0;
+            return stages == 1 ? blocks_per_sm<T, 1, SHAPE_64>(ns, mode) : blocks_per_sm<T, 2, SHAPE_64>(ns, mode);
+        }
+        return stages == 1 ? blocks_per_sm<T, 1, SHAPE_32>(ns, mode) : blocks_per_sm<T, 2, SHAPE_32>(ns, mode);
     }
-    return stages == 1 ? blocks_per_sm<T, 1, 32>(ns, mode) : blocks_per_sm<T, 2, 32>(ns, mode);
+}
+
+// FP64 lattices take tiles of 4 rows where tiles of 8 leave SMs without work.  The step is bound by
+// the FP64 pipe of the SM with the most sites, ceil(tiles / SMs) tiles; a tile of 4 rows forms its
+// ring's densities in two rounds per warp instead of one, about 10 % more FP64 work per site.
+int pull_tile_rows(int precision_bytes, int nx, int ntz8, int ntz4, int nsm) {
+    if (precision_bytes == 4) return 8;
+    const long long ntx = (nx + 31) / 32;
+    const long long most8 = (ntx * ntz8 + nsm - 1) / nsm * 8, most4 = (ntx * ntz4 + nsm - 1) / nsm * 4;
+    return most4 * 11 < most8 * 10 ? 4 : 8;
 }
 
 template <typename T>
-cudaError_t launch_pull(int ns, int mode, int stages, int width, const void* tin, T* fout,
+cudaError_t launch_pull(int ns, int mode, int stages, int shape, const void* tin, T* fout,
                         const StepConst<T>& C, const ObsPtrs& O, const Fold& fold, unsigned* sched, int set,
                         const Batch& B, int grid_max, cudaStream_t st, T* rec) {
     if (set & ~1) return cudaErrorInvalidValue;
     if (grid_max < 1) return cudaErrorInvalidConfiguration;
-    if (width == 64) {
-        if (!wide_pass<T>(mode)) return cudaErrorInvalidValue;
-        if (stages == 1)
-            return ns == 1 ? launch_ns<T, 1, 1, 64>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec)
-                           : launch_ns<T, 2, 1, 64>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec);
-        return ns == 1 ? launch_ns<T, 1, 2, 64>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec)
-                       : launch_ns<T, 2, 2, 64>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec);
+#define LBM_PULL_NS(depth, shp)                                                                                   \
+    (ns == 1 ? launch_ns<T, 1, depth, shp>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec)         \
+             : launch_ns<T, 2, depth, shp>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec))
+    if constexpr (sizeof(T) == 8) {  // one depth
+        return shape == SHAPE_SHORT ? LBM_PULL_NS(1, SHAPE_SHORT) : LBM_PULL_NS(1, SHAPE_32);
+    } else {
+        if (shape == SHAPE_64) {
+            if (!wide_pass<T>(mode)) return cudaErrorInvalidValue;
+            return stages == 1 ? LBM_PULL_NS(1, SHAPE_64) : LBM_PULL_NS(2, SHAPE_64);
+        }
+        return stages == 1 ? LBM_PULL_NS(1, SHAPE_32) : LBM_PULL_NS(2, SHAPE_32);
     }
-    if (stages == 1)
-        return ns == 1 ? launch_ns<T, 1, 1, 32>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec)
-                       : launch_ns<T, 2, 1, 32>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec);
-    return ns == 1 ? launch_ns<T, 1, 2, 32>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec)
-                   : launch_ns<T, 2, 2, 32>(mode, tin, fout, C, O, fold, sched, set, B, grid_max, st, rec);
+#undef LBM_PULL_NS
 }
 
 cudaError_t launch_wait_selftest(int* flag, long long cycles, cudaStream_t st) {
@@ -992,14 +1079,16 @@ cudaError_t launch_pull_images(int ns, T* f, const StepConst<T>& C, const Batch&
     return cudaGetLastError();
 }
 
-int make_pop_tmap(void* in_map, const void* f, int esize, int ns, int prows, int pitch, long long plane, int width) {
+int make_pop_tmap(void* in_map, const void* f, int esize, int ns, int prows, int pitch, long long plane, int shape) {
     const auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(tensor_map_encoder());
     if (!encode) return 1;
     // the whole padded plane (prows rows), boxes of a tile and its 3-cell ring
     const cuuint64_t dims[3] = {(cuuint64_t)pitch, (cuuint64_t)prows, (cuuint64_t)(9 * ns)};
     const cuuint64_t strides[2] = {(cuuint64_t)pitch * esize, (cuuint64_t)plane * esize};
-    if (width != 32 && width != 64) return 3;
-    const cuuint32_t box[3] = {(cuuint32_t)(width + 8), (cuuint32_t)BZ, (cuuint32_t)(9 * ns)};
+    if (shape != SHAPE_32 && shape != SHAPE_64 && shape != SHAPE_SHORT) return 3;
+    const cuuint32_t box[3] = {(cuuint32_t)(shape == SHAPE_64 ? Shape<SHAPE_64>::BX : Shape<SHAPE_32>::BX),
+                               (cuuint32_t)(shape == SHAPE_SHORT ? Shape<SHAPE_SHORT>::BZ : Shape<SHAPE_32>::BZ),
+                               (cuuint32_t)(9 * ns)};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUtensorMapDataType dt = esize == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
     const CUresult r = encode(static_cast<CUtensorMap*>(in_map), dt, 3, const_cast<void*>(f), dims, strides, box, estr,

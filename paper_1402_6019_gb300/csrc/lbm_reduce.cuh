@@ -62,9 +62,9 @@ template <> struct Red<float> {
     __device__ static bool nonzero(A a) { return a.x != 0.f || a.y != 0.f; }
 };
 
-// Work item blk, run by a block of RB_THREADS threads (all of which call this), or with WIDE by a
-// block of a multiple of them, whose warps past the first RB_THREADS / 32 take part in the
-// barriers only.  One warp per
+// Work item blk, run by a block of NWARP warps (all of which call this): RB_THREADS / 32, or more
+// (the warps past the first RB_THREADS / 32 take part in the barriers only), or fewer (each takes
+// several of the item's rows or columns in turn).  One warp per
 // row: the row's totals over its column groups, its profile entries (x-averages), its fluidity (Eq. fluidity: shear rate = central difference of ux_z, one-sided
 // at wall rows, wrapped when periodic, over the shear stress), its wall momenta and, when
 // sampling, its time sums.  One warp per column: the z-averages of P_xx - P_zz and P_xx.  Each
@@ -79,7 +79,7 @@ template <> struct Red<float> {
 // block partials use the accumulators above.  Fixed summation order: repeatable results.
 // inst / ninst: the lattices of a stacked batch (rows of different lattices are not neighbours);
 // null for a single lattice of nz rows.
-template <typename PT, bool WIDE = false>
+template <typename PT, int NWARP = RB_THREADS / 32>
 __device__ __forceinline__ void reduce_block(int blk, const void* part_row, const void* part_col, const int* flag,
                                              int nxpart, int nzpart, int nx, int nz, int zbc, int nrowblocks,
                                              void* __restrict__ out, void* __restrict__ avg,
@@ -89,13 +89,14 @@ __device__ __forceinline__ void reduce_block(int blk, const void* part_row, cons
     using R = Red<PT>;
     using A = typename R::A;
     constexpr int WPB = RB_THREADS / 32;
-    const int t = (int)(threadIdx.y * blockDim.x + threadIdx.x), lane = t & 31, warp = t >> 5;
+    const int t = (int)(threadIdx.y * blockDim.x + threadIdx.x), lane = t & 31, warp0 = t >> 5;
     const PT* const prow = static_cast<const PT*>(part_row);
     const PT* const pcol = static_cast<const PT*>(part_col);
     const long long iux = O_PROF, irz = O_PROF + nz, isx = O_PROF + 3LL * nz, ifl = O_PROF + 4LL * nz,
                     ips = O_PROF + 5LL * nz, ipx = ips + nx, imx = ipx + nx, imz = imx + nz, iwb = imz + nz,
                     iwt = iwb + nz;
-    for (int k = lane; k < NSC; k += 32) wsc[warp][k] = R::zero();
+    for (int w = warp0; w < (NWARP < WPB ? WPB : warp0 + 1); w += NWARP)
+        for (int k = lane; k < NSC; k += 32) wsc[w][k] = R::zero();
     if (blk == 0 && t == 0) {  // the step kernels' flag of a bad density
         const bool bad = (flag[0] & 1) != 0;
         R::put(out, O_BAD, R::from(bad ? PT(1) : PT(0)));
@@ -104,9 +105,9 @@ __device__ __forceinline__ void reduce_block(int blk, const void* part_row, cons
         else if (accumulate && bad)
             R::put(avg, O_BAD, R::from(PT(1)));
     }
-    if (WIDE && warp >= WPB) {
-        // idle in this work item
-    } else if (blk < nrowblocks) {
+    // row or column `warp` of the item
+    auto line = [&](const int warp) {
+    if (blk < nrowblocks) {
         const int z = blk * WPB + warp;
         if (z < nz) {
             // this row's lattice: its first compact row and height
@@ -216,6 +217,14 @@ __device__ __forceinline__ void reduce_block(int blk, const void* part_row, cons
                 if (accumulate) R::put(avg, oi, R::add(old, val));
             }
         }
+    }
+    };
+    if constexpr (NWARP == WPB) {
+        line(warp0);
+    } else if constexpr (NWARP > WPB) {
+        if (warp0 < WPB) line(warp0);
+    } else {
+        for (int w = warp0; w < WPB; w += NWARP) line(w);
     }
     __syncthreads();
     A bsum = R::zero();

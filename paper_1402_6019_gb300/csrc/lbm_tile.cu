@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(TPX* TZ, (sizeof(T) == 4 ? 1024 : 512) / (TPX 
         for (int s = 0; s < NS; ++s) {
             rho[s] = C.rho_ref[s] + drho[s];
             if (!(rho[s] > T(0)) || !(rho[s] < T(1e30))) bad = 1;
-            ir[s] = div_(T(1), rho[s]);
+            ir[s] = rcp_(rho[s]);
             momentum9(f[s], jx[s], jz[s]);
             F[s][0] += rho[s] * C.g;
         }

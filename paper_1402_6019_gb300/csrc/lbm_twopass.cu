@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(TPX* TPZ) k_twopass(const T* __restrict__ fin,
             drho[s] = sum9(f[s]);
             rho[s] = C.rho_ref[s] + drho[s];
             if (!(rho[s] > T(0)) || !(rho[s] < T(1e30))) bad = 1;
-            ir[s] = div_(T(1), rho[s]);
+            ir[s] = rcp_(rho[s]);
             momentum9(f[s], jx[s], jz[s]);
             F[s][0] += rho[s] * C.g;
         }

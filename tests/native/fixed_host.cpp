@@ -22,11 +22,13 @@ extern "C" {
 double fixed_psi(double rho, double rho0, double* out) {
     const ExpFx K = exp_fx_const(rho0);
     const i64 v = psi_fx(rho, K);
-    out[0] = scaled_double(v, -60);
+    out[0] = scaled_double(v, -56);
     out[1] = 1.0 - exp(-rho / rho0);
-    const long double got = (long double)v * 0x1p-60L;
+    const long double got = (long double)v * 0x1p-56L;
     return (double)(fabsl(got - psi_l(rho, rho0)) * 0x1p56L);
 }
+
+double fixed_rcp(double x) { return rcp_fx(x); }
 
 double fixed_scaled(long long v, int e) { return scaled_double(v, e); }
 
@@ -45,7 +47,7 @@ void fixed_site(const lbm_params* p, int s, const double* rho25, double* F, doub
         d[k / 5][k % 5] = psi_of(C, s, rho25[k]);
         l[k / 5][k % 5] = psi_l(rho25[k], p->rho0[s]);
     }
-    intra_force_fx(C.kf[s], w, scaled_double(w[2][2], -60), F[0], F[1]);
+    intra_force_fx(C.kf[s], w, scaled_double(w[2][2], -56), F[0], F[1]);
     S[0] = S[1] = S[2] = S64[0] = S64[1] = S64[2] = 0.0;
     intra_stress_fx(C.sf[s], w, S[0], S[1], S[2]);
     intra_force(C, s, d, F64[0], F64[1]);

@@ -26,6 +26,8 @@ def fixed(tmp_path_factory):
     dp = ctypes.POINTER(ctypes.c_double)
     lib.fixed_psi.argtypes = [ctypes.c_double, ctypes.c_double, dp]
     lib.fixed_psi.restype = ctypes.c_double
+    lib.fixed_rcp.argtypes = [ctypes.c_double]
+    lib.fixed_rcp.restype = ctypes.c_double
     lib.fixed_scaled.argtypes = [ctypes.c_longlong, ctypes.c_int]
     lib.fixed_scaled.restype = ctypes.c_double
     lib.fixed_site.argtypes = [ctypes.POINTER(L.lbm_params), ctypes.c_int] + [dp] * 7
@@ -61,6 +63,19 @@ def test_psi_of_an_invalid_density_is_zero(fixed):
     assert out[0] == 1.0
 
 
+def test_reciprocal_is_within_an_ulp(fixed):
+    """Against exact rationals: error below 2^-53 of the value (the last rounding) plus 2^-62 (the
+    iteration's remainder and its own roundings), over mantissas and exponents, at powers of two
+    and their neighbours."""
+    rng = np.random.default_rng(5)
+    xs = list(rng.uniform(1e-3, 8.0, 5000)) + list(2.0 ** rng.uniform(-900, 900, 2000))
+    for e in range(-40, 41):
+        xs += [2.0 ** e, math.nextafter(2.0 ** e, 0.0), math.nextafter(2.0 ** e, 9e99), -(2.0 ** e) * 1.7]
+    for x in xs:
+        want = 1 / Fraction(x)
+        assert abs(Fraction(fixed.fixed_rcp(x)) - want) <= abs(want) * (Fraction(1, 2 ** 53) + Fraction(1, 2 ** 62)), x
+
+
 def test_scaled_double_rounds_to_nearest(fixed):
     rng = np.random.default_rng(4)
     for v in [0, 1, -1, 2 ** 62, -2 ** 62, 2 ** 53 + 1, 2 ** 62 - 1, -(2 ** 63 - 1)] + \
@@ -90,3 +105,24 @@ def test_force_and_stress_are_no_further_off_than_fp64(fixed, preset, params):
         err[0] += (np.concatenate([F, S]) - want) ** 2
         err[1] += (np.concatenate([F64, S64]) - want) ** 2
     assert np.all(err[0] <= err[1]), np.sqrt(err / 3000)
+
+
+def test_force_is_exactly_odd(fixed):
+    """A window turned by 180 degrees gives exactly the reversed force, a uniform one exactly none:
+    the rounding of the fixed-point products has no preferred direction."""
+    p = L.lbm_params()
+    p.weight_norm = W.FILM_PARAMS["weight_norm"]
+    for k in range(2):
+        p.tau[k], p.G1[k], p.G2[k], p.rho0[k] = 1.0, -20.4, 16.0, 1.0
+    rng = np.random.default_rng(13)
+    scratch = [np.zeros(3) for _ in range(5)]
+
+    def force(rho):
+        F = np.zeros(2)
+        fixed.fixed_site(ctypes.byref(p), 0, _p(np.ascontiguousarray(rho)), _p(F), *[_p(a) for a in scratch])
+        return F
+
+    for _ in range(500):
+        rho = 0.05 + 1.4 * rng.random(25)
+        assert np.array_equal(force(rho), -force(rho[::-1]))
+        assert np.array_equal(force(np.full(25, rho[0])), np.zeros(2))
