@@ -121,6 +121,10 @@ __device__ __forceinline__ double sadd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ float sfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double sfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// 1 / x of a density
+__device__ __forceinline__ float rcp3(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rcp3(double x) { return lbm::rcp_fx(x); }
+
 // ---- geometry and constants ----------------------------------------------------------------
 
 constexpr int GX = 4, GY = 2, GZ = 2;         // ghosts of the psi / rho volumes
@@ -134,8 +138,19 @@ constexpr int NSHAPE = 4;
 constexpr int SHAPE_TY[NSHAPE] = {4, 2, 8, 4};
 constexpr int SHAPE_TZ[NSHAPE] = {2, 4, 1, 4};
 
+// FP64: the pseudopotential and Eq. FORCE's sums in fixed point (lbm_fixed.cuh).  psi is held on the
+// 2^55 scale: a shell's sum reaches 16 (|c|^2 = 6), all seven 47.
+constexpr int PSI3_BITS = 55;
 template <typename T>
-struct Step3 {
+struct Fixed3 {};
+template <>
+struct Fixed3<double> {
+    lbm::ExpFx ex[2];
+    lbm::CoefFx<7> kf[2];  // K_s(1, 2, 3, 4, 5, 6, 8)
+};
+
+template <typename T>
+struct Step3 : Fixed3<T> {
     int nx, ny, nz, ns, zbc, psi_form;
     int pitch;            // population row length (nx rounded up to 32)
     int gpitch;           // sites per row of a volume (nx + 2 GX rounded up to 4)
@@ -148,15 +163,13 @@ struct Step3 {
     T kc[3];              // weight_norm G_AB w_cross(q), q = 1, 2 (zero for one species)
 };
 
-template <typename T>
-__device__ __forceinline__ T psi3(const Step3<T>& C, int s, T rho);
-template <>
-__device__ __forceinline__ float psi3<float>(const Step3<float>& C, int s, float rho) {
+// psi as the volumes hold it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) the bits of psi on
+// the 2^PSI3_BITS scale.
+__device__ __forceinline__ float psi3(const Step3<float>& C, int s, float rho) {
     return C.psi_form == 1 ? rho : 1.0f - __expf(-rho * C.inv_rho0[s]);
 }
-template <>
-__device__ __forceinline__ double psi3<double>(const Step3<double>& C, int s, double rho) {
-    return C.psi_form == 1 ? rho : 1.0 - exp(-rho / C.rho0[s]);
+__device__ __forceinline__ double psi3(const Step3<double>& C, int s, double rho) {
+    return C.psi_form == 1 ? rho : lbm::of_bits((lbm::u64)((lbm::psi_fx(rho, C.ex[s]) + 1) >> (56 - PSI3_BITS)));
 }
 
 __device__ __forceinline__ int wrap3(int i, int n) {
@@ -251,7 +264,7 @@ __global__ void __launch_bounds__(128, TOT || sizeof(T) == 8 ? 8 : 16)
                     }
                 }
                 rho[s] = C.rho_ref[s] + a;
-                psi[s] = psi3<T>(C, s, rho[s]);
+                psi[s] = psi3(C, s, rho[s]);
                 if constexpr (TOT) {
                     if (s == 0)
                         mass0 += (double)a;
@@ -357,6 +370,43 @@ __device__ __forceinline__ V addc(V acc, V d) {
     return acc;
 }
 
+// Eq. FORCE of one species from psi on the 2^PSI3_BITS scale: the 46 antipodal differences gathered
+// shell by shell in integers (exact), the seven shells' weighted sums rounded once (DotFx), the
+// product with psi(x) in FP64.  The FP64 form takes about 170 FP64 instructions a species, this 3.
+template <typename PSF>
+__device__ __forceinline__ double3 force3_fx(const lbm::CoefFx<7>& K, const PSF& ps) {
+    using lbm::i64;
+    lbm::DotFx tx, ty, tz;
+#define LBM3_ACC(dx, dy, dz)                                    \
+    {                                                           \
+        const i64 d_ = ps(dx, dy, dz) - ps(-(dx), -(dy), -(dz)); \
+        sx += (dx) * d_;                                        \
+        sy += (dy) * d_;                                        \
+        sz += (dz) * d_;                                        \
+    }
+#define LBM3_SHELL(k, LIST)          \
+    {                                \
+        i64 sx = 0, sy = 0, sz = 0;  \
+        LIST(LBM3_ACC)               \
+        tx.add(K, k, sx);            \
+        ty.add(K, k, sy);            \
+        tz.add(K, k, sz);            \
+    }
+    LBM3_SHELL(0, LBM3_SHELL1)
+    LBM3_SHELL(1, LBM3_SHELL2)
+    LBM3_SHELL(2, LBM3_SHELL3)
+    LBM3_SHELL(3, LBM3_SHELL4)
+    LBM3_SHELL(4, LBM3_SHELL5)
+    LBM3_SHELL(5, LBM3_SHELL6)
+    LBM3_SHELL(6, LBM3_SHELL8)
+#undef LBM3_SHELL
+#undef LBM3_ACC
+    const double m = -lbm::scaled_double(ps(0, 0, 0), -PSI3_BITS);
+    const int e = K.e - 2 - PSI3_BITS;
+    return make_double3(__dmul_rn(m, lbm::scaled_double(tx.sum(), e)), __dmul_rn(m, lbm::scaled_double(ty.sum(), e)),
+                        __dmul_rn(m, lbm::scaled_double(tz.sum(), e)));
+}
+
 // Eq. FORCE over the 46 antipodal link pairs, shell by shell, both species at once, and the cross
 // repulsion of Sec. IV over the first belt: F[s][axis] of the site whose psi and rho pairs at the
 // offset (dx, dy, dz) are ps(dx, dy, dz) and rh(dx, dy, dz).
@@ -366,6 +416,20 @@ __device__ __forceinline__ void force3(const Step3<T>& C, const PSF& ps, const R
 #define PS(dx, dy, dz) ps(dx, dy, dz)
 #define RH(dx, dy, dz) rh(dx, dy, dz)
     const V zero = vsplat(T(0));
+    V Fx, Fy, Fz;
+    bool fixed = false;
+    if constexpr (sizeof(T) == 8) fixed = C.psi_form == 0;  // uniform
+    if (fixed) {
+        if constexpr (sizeof(T) == 8) {
+            double3 f0 = force3_fx(C.kf[0], [&](int dx, int dy, int dz) { return (lbm::i64)lbm::bits_of(PS(dx, dy, dz).x); });
+            Fx.x = f0.x, Fy.x = f0.y, Fz.x = f0.z;
+            Fx.y = Fy.y = Fz.y = 0.0;
+            if constexpr (NS == 2) {
+                f0 = force3_fx(C.kf[1], [&](int dx, int dy, int dz) { return (lbm::i64)lbm::bits_of(PS(dx, dy, dz).y); });
+                Fx.y = f0.x, Fy.y = f0.y, Fz.y = f0.z;
+            }
+        }
+    } else {
     V ax = zero, ay = zero, az = zero;
 #define LBM3_ACC(dx, dy, dz)                                \
     {                                                       \
@@ -394,26 +458,19 @@ __device__ __forceinline__ void force3(const Step3<T>& C, const PSF& ps, const R
     LBM3_SHELL(8, LBM3_SHELL8)
 #undef LBM3_SHELL
 #undef LBM3_ACC
-    const V p0 = PS(0, 0, 0), r0 = RH(0, 0, 0);
-    const V mp = vsub(zero, p0);
-    V Fx = vmul(mp, ax), Fy = vmul(mp, ay), Fz = vmul(mp, az);
-    if constexpr (NS == 2) {
-        // cross repulsion: F_s += -G_AB rho_s(x) sum_l w(|c|^2) rho_s'(x + c_l) c_l over the first belt
-        V bx1 = zero, by1 = zero, bz1 = zero, bx2 = zero, by2 = zero, bz2 = zero;
-#define LBM3_XACC(dx, dy, dz, SX, SY, SZ)                      \
-    {                                                          \
-        const V d_ = vsub(RH(dx, dy, dz), RH(-(dx), -(dy), -(dz)));  \
-        SX = addc<dx>(SX, d_);                                 \
-        SY = addc<dy>(SY, d_);                                 \
-        SZ = addc<dz>(SZ, d_);                                 \
+    const V mp = vsub(zero, PS(0, 0, 0));
+    Fx = vmul(mp, ax), Fy = vmul(mp, ay), Fz = vmul(mp, az);
     }
-#define LBM3_X1(dx, dy, dz) LBM3_XACC(dx, dy, dz, bx1, by1, bz1)
-#define LBM3_X2(dx, dy, dz) LBM3_XACC(dx, dy, dz, bx2, by2, bz2)
-        LBM3_SHELL1(LBM3_X1)
-        LBM3_SHELL2(LBM3_X2)
-#undef LBM3_X1
-#undef LBM3_X2
-#undef LBM3_XACC
+    if constexpr (NS == 2) {
+        const V r0 = RH(0, 0, 0);
+        // cross repulsion: F_s += -G_AB rho_s(x) sum_l w(|c|^2) rho_s'(x + c_l) c_l over the first belt
+#define LBM3_X(dx, dy, dz) vsub(RH(dx, dy, dz), RH(-(dx), -(dy), -(dz)))
+        const V bx1 = LBM3_X(1, 0, 0), by1 = LBM3_X(0, 1, 0), bz1 = LBM3_X(0, 0, 1);
+        const V xyp = LBM3_X(1, 1, 0), xym = LBM3_X(1, -1, 0), xzp = LBM3_X(1, 0, 1), xzm = LBM3_X(1, 0, -1),
+                yzp = LBM3_X(0, 1, 1), yzm = LBM3_X(0, 1, -1);
+#undef LBM3_X
+        const V bx2 = vadd(vadd(xyp, xym), vadd(xzp, xzm)), by2 = vadd(vsub(xyp, xym), vadd(yzp, yzm)),
+                bz2 = vadd(vsub(xzp, xzm), vsub(yzp, yzm));
         const V k1 = vsplat(C.kc[1]), k2 = vsplat(C.kc[2]);
         const V cx_ = vfma(k2, bx2, vmul(k1, bx1)), cy_ = vfma(k2, by2, vmul(k1, by1)),
                 cz_ = vfma(k2, bz2, vmul(k1, bz1));
@@ -460,7 +517,7 @@ __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T
         drho[s] = a;
         rho[s] = sadd(C.rho_ref[s], a);
         if (!(rho[s] > T(0)) || !(rho[s] < T(1e30))) bad = true;
-        ir[s] = T(1) / rho[s];
+        ir[s] = rcp3(rho[s]);
         jx[s] = mx;
         jy[s] = my;
         jz[s] = mz;
@@ -475,7 +532,7 @@ __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T
         nzu = sfma(C.omega[s], jz[s], nzu);
         den = sfma(C.omega[s], rho[s], den);
     }
-    const T iden = T(1) / den;
+    const T iden = rcp3(den);
     const T upx = smul(nxu, iden), upy = smul(nyu, iden), upz = smul(nzu, iden);
 
     if constexpr ((MODE & K3_FIELDS) != 0) {
@@ -590,19 +647,25 @@ __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T
                 const T u15 = smul(T(1.5), sfma(ux, ux, sfma(uy, uy, smul(uz, uz))));
                 const T b = smul(om, rho[s]);
                 const T base = sadd(smul(om, drho[s]), -smul(b, u15));  // omega (drho - 3/2 rho u^2)
-                push(s, 0, sfma(keep, f[s][0], smul(w19<T>(0), base)));
+                // even part +- odd part = e + cu (4.5 w b cu +- 3 w b), per weight class; the kept
+                // part (1 - omega) f vanishes at tau = 1
+                const T wa = w19<T>(1), we = w19<T>(7);
+                const T ea = smul(wa, base), ee = smul(we, base);
+                const T ca = smul(T(4.5) * wa, b), ce = smul(T(4.5) * we, b);
+                const T da = smul(T(3) * wa, b), de = smul(T(3) * we, b);
+                const bool relaxed = keep == T(0);
+                const T g0 = smul(w19<T>(0), base);
+                push(s, 0, relaxed ? g0 : sfma(keep, f[s][0], g0));
 #pragma unroll
                 for (int l = 1; l < 19; l += 2) {  // l and its opposite l + 1
                     // starting from the first, +1, component (no add of zero)
                     T cu = c3x(l) ? ux : (c3y(l) ? uy : uz);
                     if (c3x(l) && c3y(l)) cu = sadd(cu, c3y(l) > 0 ? uy : -uy);
                     if ((c3x(l) || c3y(l)) && c3z(l)) cu = sadd(cu, c3z(l) > 0 ? uz : -uz);
-                    const T w = w19<T>(l);
-                    const T wb = smul(w, b);
-                    const T even = sfma(smul(T(4.5), wb), smul(cu, cu), smul(w, base));
-                    const T odd = smul(smul(T(3), wb), cu);
-                    push(s, l, sadd(sfma(keep, f[s][l], even), odd));
-                    push(s, l + 1, sadd(sfma(keep, f[s][l + 1], even), -odd));
+                    const T e = l < 7 ? ea : ee, c = l < 7 ? ca : ce, d = l < 7 ? da : de;
+                    const T ep = relaxed ? e : sfma(keep, f[s][l], e), em = relaxed ? e : sfma(keep, f[s][l + 1], e);
+                    push(s, l, sfma(sfma(c, cu, d), cu, ep));
+                    push(s, l + 1, sfma(sfma(c, cu, -d), cu, em));
                 }
             }
         }
@@ -639,13 +702,15 @@ __global__ void __launch_bounds__(TX* TY* TZ, TX* TY* TZ > 256 ? 1 : (sizeof(T) 
     }
     // own populations from HBM while the box is on its way
     const long long i = ((long long)z * C.ny + y) * C.pitch + x;
+    // (FP64, short of registers, loads them after the force: its other warps cover the wait)
     T f[NS][19];
-    if (live) {
+    const auto load = [&]() {
 #pragma unroll
         for (int s = 0; s < NS; ++s)
 #pragma unroll
             for (int l = 0; l < 19; ++l) f[s][l] = fin[(s * 19 + l) * C.plane + i];
-    }
+    };
+    if (sizeof(T) == 4 && live) load();
     __syncthreads();  // the barrier is initialised before anyone waits on it
     bool ok = true;
     {
@@ -691,6 +756,7 @@ __global__ void __launch_bounds__(TX* TY* TZ, TX* TY* TZ > 256 ? 1 : (sizeof(T) 
     force3<T, NS>(
         C, [&](int dx, int dy, int dz) { return S.box[0][bz + dz][by + dy][bx + dx]; },
         [&](int dx, int dy, int dz) { return S.box[1][bz + dz][by + dy][bx + dx]; }, F);
+    if (sizeof(T) == 8) load();
     site3<T, NS, MODE>(C, f, F, x, y, z, i, fout, flag, fields);
 }
 
@@ -840,6 +906,11 @@ static void fill_step3(const lbm3_ctx* c, Step3<T>& C) {
         C.rho_ref[s] = on ? (T)c->rho_ref[s] : T(0);
         for (int q = 0; q < 9; ++q)
             C.kq[s][q] = on ? (T)(wn * (c->p.G1[ps] * w_att3(q) + c->p.G2[ps] * w_rep3(q))) : T(0);
+        if constexpr (sizeof(T) == 8) {
+            C.ex[s] = lbm::exp_fx_const(c->p.psi_form == LBM_PSI_EXP ? c->p.rho0[ps] : 1.0);
+            const double k[7] = {C.kq[s][1], C.kq[s][2], C.kq[s][3], C.kq[s][4], C.kq[s][5], C.kq[s][6], C.kq[s][8]};
+            lbm::coef_fx(C.kf[s], k);
+        }
     }
     for (int q = 0; q < 3; ++q) C.kc[q] = c->d.n_species == 2 ? (T)(wn * c->p.G_AB * w_cross3(q)) : T(0);
 }

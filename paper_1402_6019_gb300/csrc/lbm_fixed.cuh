@@ -225,23 +225,23 @@ LBM_FX i64 psi_fx(double rho, const ExpFx& K) {
 
 // ---- forces and stresses --------------------------------------------------------------------
 
-// Coefficients c_k = v[k] 2^(e - 62), |v[k]| <= 2^62, and c_k = (h[k] 2^29 + l[k]) 2^(e - 58) in two
+// N coefficients c_k = v[k] 2^(e - 62), |v[k]| <= 2^62, and c_k = (h[k] 2^29 + l[k]) 2^(e - 58) in two
 // limbs, 0 <= l < 2^29, |h| <= 2^29.
+template <int N>
 struct CoefFx {
-    i64 v[5];
-    double c[3];  // c_1, c_3, c_4 themselves
-    int h[5], l[5];
+    i64 v[N];
+    double c[N];  // the coefficients themselves
+    int h[N], l[N];
     int e, pad;
 };
-inline void coef_fx(CoefFx& F, const double* c) {
-    F.c[0] = c[1];
-    F.c[1] = c[3];
-    F.c[2] = c[4];
+template <int N>
+inline void coef_fx(CoefFx<N>& F, const double* c) {
     double top = 0.0;
-    for (int k = 0; k < 5; ++k) top = fabs(c[k]) > top ? fabs(c[k]) : top;
+    for (int k = 0; k < N; ++k) top = fabs(c[k]) > top ? fabs(c[k]) : top;
     int e = 0;
     if (top > 0.0) (void)frexp(top, &e);  // top < 2^e
-    for (int k = 0; k < 5; ++k) {
+    for (int k = 0; k < N; ++k) {
+        F.c[k] = c[k];
         F.v[k] = (i64)ldexp(c[k], 62 - e);
         const i64 u = (i64)rint(ldexp(c[k], 58 - e));
         F.h[k] = (int)(u >> 29);
@@ -251,13 +251,15 @@ inline void coef_fx(CoefFx& F, const double* c) {
     F.pad = 0;
 }
 
-// sum_k c_k S_k of five sums |S_k| <= 6 2^56, exact in three accumulators of 29-bit limb products (each
-// a 32 x 32 -> 64 multiply-add; at most 5 (2^58.6 + 2^58)), rounded once to the nearest on the
-// scale 2^(58 - e).  Rounding every product down instead would push each site the same way, a drift
-// that adds up over the steps; this is odd in S.
-struct Dot5 {
+// sum_k c_k S_k of a few sums |S_k| < 2^60, exact in three accumulators of 29-bit limb products (each a
+// 32 x 32 -> 64 multiply-add), rounded once to the nearest: sum() 2^(e - 56) times the scale of S.
+// Rounding every product down instead would push each site the same way, a drift that adds up over
+// the steps; this is odd in S.  Room: with |c_k| <= 2^e and sum_k |S_k| <= 2^60.6 no accumulator
+// passes 2^62.7.
+struct DotFx {
     i64 hh = 0, mid = 0, ll = 0;
-    LBM_FX void add(const CoefFx& K, int k, i64 S) {
+    template <int N>
+    LBM_FX void add(const CoefFx<N>& K, int k, i64 S) {
         const int sh = (int)(S >> 29), sl = (int)(S & ((1 << 29) - 1));
         hh += (i64)sh * K.h[k];
         mid += (i64)sh * K.l[k];
@@ -269,15 +271,15 @@ struct Dot5 {
 
 // Eq. FORCE of one species from the 5 x 5 window p of psi on the 2^56 scale: intra_force of
 // lbm_core.cuh with every sum exact.  K: K(1), K(2), 2 K(4), K(5), 2 K(8).  psi0: psi at the site.
-// Every shell sum is at most 6 and their weighted sum at most 12 2^e, which fits.  40 multiply-adds
+// The shell sums are at most 1, 2, 1, 6 and 2, and their weighted sum at most 12 2^e, which fits.  40 multiply-adds
 // and about 30 adds in integers and 4 FP64 instructions replace 34 FP64 ones.
-LBM_FX void intra_force_fx(const CoefFx& K, const i64 (&p)[5][5], double psi0, double& fx, double& fz) {
+LBM_FX void intra_force_fx(const CoefFx<5>& K, const i64 (&p)[5][5], double psi0, double& fx, double& fz) {
 #define LBM_Q(dx, dz) p[(dz) + 2][(dx) + 2]
     const i64 d11 = LBM_Q(1, 1) - LBM_Q(-1, -1), e11 = LBM_Q(-1, 1) - LBM_Q(1, -1);
     const i64 d21 = LBM_Q(2, 1) - LBM_Q(-2, -1), e21 = LBM_Q(-2, 1) - LBM_Q(2, -1);
     const i64 d12 = LBM_Q(1, 2) - LBM_Q(-1, -2), e12 = LBM_Q(-1, 2) - LBM_Q(1, -2);
     const i64 d22 = LBM_Q(2, 2) - LBM_Q(-2, -2), e22 = LBM_Q(-2, 2) - LBM_Q(2, -2);
-    Dot5 x, z;
+    DotFx x, z;
     x.add(K, 0, LBM_Q(1, 0) - LBM_Q(-1, 0));
     z.add(K, 0, LBM_Q(0, 1) - LBM_Q(0, -1));
     x.add(K, 1, d11 - e11);
@@ -298,7 +300,7 @@ LBM_FX void intra_force_fx(const CoefFx& K, const i64 (&p)[5][5], double psi0, d
 // formed on the 2^58 scale; the shells' sums (at most 40 in shell 5) meet on the 2^57 scale, the
 // weighted sums (at most 2 + 4 + 4 + 40 + 8) on the 2^55 scale.  33 products in integers and 6 FP64
 // instructions replace about 65 FP64 ones.
-LBM_FX void intra_stress_fx(const CoefFx& Q, const i64 (&p)[5][5], double& sxx, double& szz, double& sxz) {
+LBM_FX void intra_stress_fx(const CoefFx<5>& Q, const i64 (&p)[5][5], double& sxx, double& szz, double& sxz) {
 #define LBM_P(dx, dz) (p[(dz) + 2][(dx) + 2] << 4)           // 2^60
 #define LBM_M(a, b) (i64)mulhi_u((u64)(a) << 2, (u64)(b))    // 2^62 x 2^k -> 2^(k - 2), nothing negative
     const i64 p0 = p[2][2] << 6;                             // 2^62
@@ -329,7 +331,7 @@ LBM_FX void intra_stress_fx(const CoefFx& Q, const i64 (&p)[5][5], double& sxx, 
     sxx += scaled_double(mulhi_s(Q.v[0], x1) + mulhi_s(Q.v[2], x4) + mulhi_s(Q.v[3], x5) + both, Q.e - 55);
     szz += scaled_double(mulhi_s(Q.v[0], z1) + mulhi_s(Q.v[2], z4) + mulhi_s(Q.v[3], z5) + both, Q.e - 55);
     // xz, a difference of nearly equal sums, is small: weighted in FP64, whose rounding follows its size
-    sxz += (Q.c[0] * scaled_double(u2, -57) + Q.c[1] * scaled_double(w5, -57)) + Q.c[2] * scaled_double(u8, -57);
+    sxz += (Q.c[1] * scaled_double(u2, -57) + Q.c[3] * scaled_double(w5, -57)) + Q.c[4] * scaled_double(u8, -57);
 #undef LBM_P
 #undef LBM_M
 }
