@@ -109,7 +109,8 @@ int lbm3_profile(lbm3_ctx *c, int enable);
 int lbm3_profile_read(lbm3_ctx *c, double *ms, long long *steps);
 
 /* Tile shapes of the collide pass: 0 = 32 x 4 x 2 sites (the default), 1 = 32 x 2 x 4,
-   2 = 32 x 8 x 1 (256 threads each), 3 = 32 x 4 x 4 (512 threads).  The shape changes which
+   2 = 32 x 8 x 1 (256 threads each), 3 = 32 x 4 x 4 (512 threads); in FP64 0 = 16 x 8 x 1,
+   1 = 16 x 4 x 2, 2 = 16 x 2 x 4 (128 threads), 3 = 16 x 8 x 2 (256).  The shape changes which
    CTA does which sites and how much of the psi / rho halo each reads, not the arithmetic:
    results are bit-identical.  lbm3_autotune times `steps` (1 .. 10000) steps of each shape on
    the context's own lattice, keeps the fastest, and puts the state and step counter back as

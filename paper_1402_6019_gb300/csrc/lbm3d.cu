@@ -128,15 +128,29 @@ __device__ __forceinline__ double rcp3(double x) { return lbm::rcp_fx(x); }
 // ---- geometry and constants ----------------------------------------------------------------
 
 constexpr int GX = 4, GY = 2, GZ = 2;         // ghosts of the psi / rho volumes
-constexpr int TX = 32;                        // tile width: one warp per tile row
-constexpr int BX = TX + 2 * GX;               // box width (x from x0 - 4: 16-byte aligned)
 constexpr long long WAIT_LIMIT = 2000000000LL;  // clock cycles of the bounded wait (~1 s)
-// The tile shapes (TY x TZ rows of 32 sites, one thread per site) lbm3_autotune chooses from:
-// the halo box of a tile is (TY + 4) x (TZ + 4) rows, so flatter tiles read more halo from L2
-// per site and taller ones hold fewer CTAs per SM.
+// The tile shapes (TY x TZ rows of TX sites, one thread per site) lbm3_autotune chooses from: the
+// halo box of a tile is (TY + 4) x (TZ + 4) rows (x from x0 - 4: 16-byte aligned), so flatter tiles
+// read more halo from L2 per site and taller ones hold fewer CTAs per SM.
+//  * FP32: rows of 32 (a warp), 256 threads (shape 3: 512).
+//  * FP64: rows of 16, two to a warp, 128 threads (shape 3: 256).  The pass is bound by the FP64
+//    pipe, which a warp holds for 16 cycles an instruction however few of its sites are inside the
+//    lattice, so a row's last tile should waste few: at nx = 65 rows of 16 keep 81 % of the lanes
+//    at work, rows of 32 68 %; and the smaller CTAs leave a smaller last wave.
 constexpr int NSHAPE = 4;
-constexpr int SHAPE_TY[NSHAPE] = {4, 2, 8, 4};
-constexpr int SHAPE_TZ[NSHAPE] = {2, 4, 1, 4};
+template <typename T>
+struct Tile3 {
+    static constexpr int TX = sizeof(T) == 4 ? 32 : 16;
+    static constexpr int BX = TX + 2 * GX;  // box width
+    static constexpr int ty(int shape) {
+        constexpr int f[NSHAPE] = {4, 2, 8, 4}, d[NSHAPE] = {8, 4, 2, 8};
+        return sizeof(T) == 4 ? f[shape] : d[shape];
+    }
+    static constexpr int tz(int shape) {
+        constexpr int f[NSHAPE] = {2, 4, 1, 4}, d[NSHAPE] = {1, 2, 4, 2};
+        return sizeof(T) == 4 ? f[shape] : d[shape];
+    }
+};
 
 // FP64: the pseudopotential and Eq. FORCE's sums in fixed point (lbm_fixed.cuh).  psi is held on the
 // 2^55 scale: a shell's sum reaches 16 (|c|^2 = 6), all seven 47.
@@ -248,20 +262,17 @@ __global__ void __launch_bounds__(128, TOT || sizeof(T) == 8 ? 8 : 16)
             if (x >= C.nx) continue;
             const long long i = ((long long)z * C.ny + y) * C.pitch + x;
             T rho[2] = {T(0), T(0)}, psi[2] = {T(0), T(0)};
-            T mx = T(0), my = T(0), mz = T(0);
+            T d[9];  // TOT: f_l - f_opp(l) of the nine pairs, the species added
 #pragma unroll
             for (int s = 0; s < 2; ++s) {  // unrolled, so that the per-species values stay in registers
                 if (s >= C.ns) break;
-                T a = T(0);
+                T a = f[(s * 19) * C.plane + i];
 #pragma unroll
-                for (int l = 0; l < 19; ++l) {
-                    const T v = f[(s * 19 + l) * C.plane + i];
+                for (int l = 1; l < 19; l += 2) {
+                    const T u = f[(s * 19 + l) * C.plane + i], v = f[(s * 19 + l + 1) * C.plane + i];
+                    a += u;
                     a += v;
-                    if constexpr (TOT) {
-                        if (c3x(l)) mx += c3x(l) > 0 ? v : -v;
-                        if (c3y(l)) my += c3y(l) > 0 ? v : -v;
-                        if (c3z(l)) mz += c3z(l) > 0 ? v : -v;
-                    }
+                    if constexpr (TOT) d[l / 2] = s == 0 ? u - v : d[l / 2] + (u - v);
                 }
                 rho[s] = C.rho_ref[s] + a;
                 psi[s] = psi3(C, s, rho[s]);
@@ -273,9 +284,10 @@ __global__ void __launch_bounds__(128, TOT || sizeof(T) == 8 ? 8 : 16)
                 }
             }
             if constexpr (TOT) {
-                momx += (double)mx;
-                momy += (double)my;
-                momz += (double)mz;
+                // velocities 1, 3, 5 along x, y, z, then (1,1,0), (1,-1,0), (1,0,1), (1,0,-1), (0,1,1), (0,1,-1)
+                momx += (double)(d[0] + ((d[3] + d[4]) + (d[5] + d[6])));
+                momy += (double)(d[1] + ((d[3] - d[4]) + (d[7] + d[8])));
+                momz += (double)(d[2] + ((d[5] - d[6]) + (d[7] - d[8])));
             }
             V pv, rv;
             pv.x = psi[0];
@@ -340,7 +352,7 @@ enum { K3_WRITE = 1, K3_FIELDS = 2 };
 
 template <typename T, int TY, int TZ>
 struct Smem3 {
-    static constexpr int BY = TY + 2 * GY, BZ = TZ + 2 * GZ;
+    static constexpr int BX = Tile3<T>::BX, BY = TY + 2 * GY, BZ = TZ + 2 * GZ;
     typename PairOf<T>::V box[2][BZ][BY][BX];  // psi, rho pairs of the tile and its halo
     alignas(8) unsigned long long bar;
 };
@@ -675,10 +687,11 @@ __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T
 // FP32 tiles of 256 threads: 3 CTAs per SM (80 registers, 16 bytes of spills), measured faster than
 // 2 CTAs at 110 registers without spills -- the kernel waits on memory and more warps hide it.
 template <typename T, int MODE, int NS, int TY, int TZ>
-__global__ void __launch_bounds__(TX* TY* TZ, TX* TY* TZ > 256 ? 1 : (sizeof(T) == 4 ? 3 : 2))
+__global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
+                                  Tile3<T>::TX* TY* TZ > 256 ? 1 : (sizeof(T) == 4 ? 3 : 512 / (Tile3<T>::TX * TY * TZ)))
     k3_step(const __grid_constant__ CUtensorMap vmap, const T* __restrict__ fin, T* __restrict__ fout,
             const Step3<T> C, int* __restrict__ flag, double* __restrict__ fields) {
-    using V = typename PairOf<T>::V;
+    constexpr int TX = Tile3<T>::TX;
     extern __shared__ __align__(1024) unsigned char smem3[];
     Smem3<T, TY, TZ>& S = *reinterpret_cast<Smem3<T, TY, TZ>*>(smem3);
     const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
@@ -786,6 +799,7 @@ cudaError_t launch_step3(const CUtensorMap& map, const T* fin, T* fout, const St
         if (e != cudaSuccess) return e;
         attr = true;
     }
+    constexpr int TX = Tile3<T>::TX;
     const dim3 grid((C.nx + TX - 1) / TX, (C.ny + TY - 1) / TY, (C.nz + TZ - 1) / TZ);
     return launch_pdl(k3_step<T, MODE, NS, TY, TZ>, grid, dim3(TX, TY, TZ), smem, st, map, fin, fout, C, flag, fields);
 }
@@ -794,10 +808,10 @@ template <typename T, int MODE, int NS>
 cudaError_t launch_shape(int shape, const CUtensorMap& map, const T* fin, T* fout, const Step3<T>& C, int* flag,
                          double* fields, cudaStream_t st) {
     switch (shape) {
-        case 0: return launch_step3<T, MODE, NS, SHAPE_TY[0], SHAPE_TZ[0]>(map, fin, fout, C, flag, fields, st);
-        case 1: return launch_step3<T, MODE, NS, SHAPE_TY[1], SHAPE_TZ[1]>(map, fin, fout, C, flag, fields, st);
-        case 2: return launch_step3<T, MODE, NS, SHAPE_TY[2], SHAPE_TZ[2]>(map, fin, fout, C, flag, fields, st);
-        case 3: return launch_step3<T, MODE, NS, SHAPE_TY[3], SHAPE_TZ[3]>(map, fin, fout, C, flag, fields, st);
+        case 0: return launch_step3<T, MODE, NS, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, st);
+        case 1: return launch_step3<T, MODE, NS, Tile3<T>::ty(1), Tile3<T>::tz(1)>(map, fin, fout, C, flag, fields, st);
+        case 2: return launch_step3<T, MODE, NS, Tile3<T>::ty(2), Tile3<T>::tz(2)>(map, fin, fout, C, flag, fields, st);
+        case 3: return launch_step3<T, MODE, NS, Tile3<T>::ty(3), Tile3<T>::tz(3)>(map, fin, fout, C, flag, fields, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -809,8 +823,8 @@ cudaError_t launch_step3_any(int mode, int ns, int shape, const CUtensorMap& map
     if (mode == K3_WRITE)
         return ns == 2 ? launch_shape<T, K3_WRITE, 2>(shape, map, fin, fout, C, flag, fields, st)
                        : launch_shape<T, K3_WRITE, 1>(shape, map, fin, fout, C, flag, fields, st);
-    return ns == 2 ? launch_step3<T, K3_FIELDS, 2, SHAPE_TY[0], SHAPE_TZ[0]>(map, fin, fout, C, flag, fields, st)
-                   : launch_step3<T, K3_FIELDS, 1, SHAPE_TY[0], SHAPE_TZ[0]>(map, fin, fout, C, flag, fields, st);
+    return ns == 2 ? launch_step3<T, K3_FIELDS, 2, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, st)
+                   : launch_step3<T, K3_FIELDS, 1, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, st);
 }
 
 }  // namespace lbm3
@@ -964,8 +978,11 @@ static int make_vol_map(lbm3_ctx* c, int shape) {
                                 (cuuint64_t)(c->d.nz + 2 * GZ), 2};
     const cuuint64_t strides[3] = {(cuuint64_t)2 * c->gpitch * es, (cuuint64_t)2 * c->gpitch * (c->d.ny + 2 * GY) * es,
                                    (cuuint64_t)2 * c->gvol * es};
-    const cuuint32_t box[4] = {(cuuint32_t)(2 * BX), (cuuint32_t)(SHAPE_TY[shape] + 2 * GY),
-                               (cuuint32_t)(SHAPE_TZ[shape] + 2 * GZ), 2};
+    const bool f32 = c->esize == 4;
+    const int bx = f32 ? Tile3<float>::BX : Tile3<double>::BX;
+    const int ty = f32 ? Tile3<float>::ty(shape) : Tile3<double>::ty(shape);
+    const int tz = f32 ? Tile3<float>::tz(shape) : Tile3<double>::tz(shape);
+    const cuuint32_t box[4] = {(cuuint32_t)(2 * bx), (cuuint32_t)(ty + 2 * GY), (cuuint32_t)(tz + 2 * GZ), 2};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const CUresult r = encode(reinterpret_cast<CUtensorMap*>(c->map[shape]),
                               c->esize == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4,
@@ -1023,10 +1040,14 @@ extern "C" int lbm3_create(lbm3_ctx** out, const lbm3_desc* d) {
     CKC3(cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
     int nsm = 0;
     CKC3(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, d->device));
-    {  // the density pass with totals: about 8 CTAs per SM, each looping over its rows
-        const int gx = (nx + 127) / 128, target = 8 * nsm;
-        const int gy = std::max(1, std::min(ny, target / gx));
-        const int gz = std::max(1, std::min(nz, target / (gx * gy)));
+    {  // the density pass with totals: about 8 CTAs per SM, each looping over as many rows (not one
+       // over two and the next over one), or a CTA per row segment while there are few
+        const int gx = (nx + 127) / 128, target = (long long)gx * ny * nz <= 16 * nsm ? 16 * nsm : 8 * nsm;
+        int gy = std::max(1, std::min(ny, target / gx));
+        int gz = std::max(1, std::min(nz, target / (gx * gy)));
+        const int py = (ny + gy - 1) / gy, pz = (nz + gz - 1) / gz;
+        gy = (ny + py - 1) / py;
+        gz = (nz + pz - 1) / pz;
         c->tot_grid[0] = gx;
         c->tot_grid[1] = gy;
         c->tot_grid[2] = gz;
