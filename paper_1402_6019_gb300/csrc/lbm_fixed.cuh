@@ -84,6 +84,17 @@ LBM_FX double scaled_double(i64 v, int e) {
     return of_bits(b | (v < 0 ? (u64)1 << 63 : (u64)0));
 }
 
+// A float as a double by its bits: the conversion instruction takes the FP64 pipe 16 cycles a warp.
+LBM_FX double widen_fx(float v) {
+#if defined(__CUDA_ARCH__)
+    const unsigned b = __float_as_uint(v);
+    const unsigned e = b & 0x7f800000u;
+    if (e != 0u && e != 0x7f800000u)  // normal: the exponent rebiased, the mantissa moved up
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+#endif
+    return (double)v;
+}
+
 // 1 / x for a normal x with |x| in 2^-1000 .. 2^1000: a seed from the FP32 reciprocal of the mantissa
 // (relative error below 2^-21), then one step of the third-order (Halley) iteration
 // y (1 + d + d^2), d = 1 - x y, whose remainder d^3 is below 2^-63: 3 FP64 instructions, the error

@@ -69,17 +69,39 @@ __device__ __forceinline__ long long pull_src(const StepConst<T>& C, int x, int 
     return (long long)(prow0 + zs + PULL_GZ) * C.pitch + (x - cx(l) + PULL_GX);
 }
 
+// W_l rho_ref of each species' rest, axis and diagonal populations, and as two floats hi + lo.
+struct ExportBase {
+    double base[6];
+    float hi[6], lo[6];
+};
+
+// A stored value and its base W_l rho_ref added and rounded to O.  FP32 to FP32 stays off the FP64
+// pipe, which its two conversions and the add kept busy for three quarters of the export: the base is
+// split into two floats and added with its rounding error (two_sum), so the sum is the FP64 one
+// rounded (but for a tie in 2^-24 of the cases).
+template <typename T, typename O>
+__device__ __forceinline__ O plain_value(T v, double base, float hi, float lo) {
+    if constexpr (sizeof(T) == 4 && sizeof(O) == 4) {
+        const float2 s = two_sum(hi, v);
+        return s.x + (s.y + lo);
+    } else if constexpr (sizeof(T) == 4) {
+        return (O)(widen_fx(v) + base);
+    } else {
+        return (O)((double)v + base);
+    }
+}
+
 // The post-streaming populations as plain values, [ns][9][nz][nx]: the stored value of (x, l) in
 // the push layout, the gather of the pull layout.  Blocks of 32 x 8 sites of one population
 // (blockIdx.z = s * 9 + l).
 template <typename T, typename O>
 __global__ void __launch_bounds__(256) k_export(int ns, const T* __restrict__ f, O* __restrict__ out,
-                                                const StepConst<T> C, const InstGeom* __restrict__ inst, int ninst) {
+                                                const StepConst<T> C, const __grid_constant__ ExportBase B,
+                                                const InstGeom* __restrict__ inst, int ninst) {
     const long long n = (long long)C.nx * C.nz;
     const int s = blockIdx.z / 9, l = blockIdx.z % 9;
     const int x = blockIdx.x * 32 + threadIdx.x, zg = blockIdx.y * 8 + threadIdx.y;
     if (x >= C.nx || zg >= C.nz) return;
-    const double base = wlb<double>(l) * (double)C.rho_ref[s];
     long long o = (long long)zg * C.pitch + x;
     int ls = l;
     if (inst) {
@@ -90,7 +112,9 @@ __global__ void __launch_bounds__(256) k_export(int ns, const T* __restrict__ f,
             o = pull_src(C, x, zg, C.nz, 0, l, ls);
         }
     }
-    out[(s * 9 + l) * n + (long long)zg * C.nx + x] = (O)((double)f[(s * 9 + ls) * C.plane + o] + base);
+    const int k = s * 3 + (l == 0 ? 0 : (l <= 4 ? 1 : 2));
+    out[(s * 9 + l) * n + (long long)zg * C.nx + x] =
+        plain_value<T, O>(f[(s * 9 + ls) * C.plane + o], B.base[k], B.hi[k], B.lo[k]);
 }
 
 // The inverse of k_export: plain FP64 post-streaming values in, stored values out.
@@ -239,7 +263,14 @@ cudaError_t launch_init(int ns, T* f, const double* rho, const double* u, const 
 template <typename T, typename O>
 cudaError_t launch_export(int ns, const T* f, O* out, const StepConst<T>& C, const Batch* B, cudaStream_t st) {
     const dim3 grid((C.nx + 31) / 32, (C.nz + 7) / 8, 9 * ns);
-    k_export<T, O><<<grid, dim3(32, 8), 0, st>>>(ns, f, out, C, B ? B->inst : nullptr, B ? B->ninst : 0);
+    ExportBase E;
+    for (int k = 0; k < 6; ++k) {
+        const int l[3] = {0, 1, 5};
+        E.base[k] = wlb<double>(l[k % 3]) * (double)C.rho_ref[k / 3];
+        E.hi[k] = (float)E.base[k];
+        E.lo[k] = (float)(E.base[k] - (double)E.hi[k]);
+    }
+    k_export<T, O><<<grid, dim3(32, 8), 0, st>>>(ns, f, out, C, E, B ? B->inst : nullptr, B ? B->ninst : 0);
     return cudaGetLastError();
 }
 
