@@ -18,6 +18,15 @@
 // once plus the 16 B of the volumes written and read, 488 B; the method's own is 304 B
 // (each population read and written once).  Populations are SoA f[s][l][z][y][x] (rows padded
 // to 32), FP32 deviations f - W_l rho_ref,s or plain FP64.
+//
+// Full relaxation (FP32, tau = 1 for every species) needs no populations: the collision leaves
+// f*_l = feq_l(rho_s, u_s), so the density and velocity after it (4 numbers per species, held as 5)
+// are the whole state, and a step only needs the density and momentum of what streams in.
+//  * k3_stream evaluates, at every site, the 19 equilibria that stream in from the neighbours'
+//    moments, and writes their density and momentum (and the psi / rho volumes);
+//  * k3_step in its K3_RELAX form takes the force from the volumes and writes the new density and velocity.
+// About 170 B per site-update, and half the instructions.  Populations are formed where they are asked
+// for (k3_expand).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <stdarg.h>
@@ -120,6 +129,10 @@ __device__ __forceinline__ float sadd(float a, float b) { return __fadd_rn(a, b)
 __device__ __forceinline__ double sadd(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ float sfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double sfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// v as FP64: of an FP32 value by its bits (the conversion instruction runs on the FP64 pipe).
+__device__ __forceinline__ double wide3(float v) { return lbm::widen_fx(v); }
+__device__ __forceinline__ double wide3(double v) { return v; }
 
 // 1 / x of a density
 __device__ __forceinline__ float rcp3(float x) { return 1.0f / x; }
@@ -249,9 +262,12 @@ __device__ __forceinline__ int ghost_list(int v, int n, int g, bool mirror, int*
 // FP64 pipe is the scarce one), in a fixed order.
 // 16 CTAs per SM for the plain FP32 pass (32 registers, as it ran fastest); 8 with the totals,
 // whose FP64 accumulators need up to 64 registers, and in FP64, so that neither spills
-template <typename T, bool TOT>
-__global__ void __launch_bounds__(128, TOT || sizeof(T) == 8 ? 8 : 16)
-    k3_density(const T* __restrict__ f, T* __restrict__ vol, const Step3<T> C, double* __restrict__ part) {
+// dn, jt (FP32, full relaxation, from populations; else null): the densities' deviations and the
+// momentum (three planes) for K3_RELAX.
+template <typename T, bool TOT, bool MOM = false>
+__global__ void __launch_bounds__(128, TOT || MOM || sizeof(T) == 8 ? 8 : 16)
+    k3_density(const T* __restrict__ f, T* __restrict__ vol, const Step3<T> C, double* __restrict__ part,
+               float2* __restrict__ dn = nullptr, float* __restrict__ jt = nullptr) {
     using V = typename PairOf<T>::V;
     pdl_enter();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -262,7 +278,8 @@ __global__ void __launch_bounds__(128, TOT || sizeof(T) == 8 ? 8 : 16)
             if (x >= C.nx) continue;
             const long long i = ((long long)z * C.ny + y) * C.pitch + x;
             T rho[2] = {T(0), T(0)}, psi[2] = {T(0), T(0)};
-            T d[9];  // TOT: f_l - f_opp(l) of the nine pairs, the species added
+            float2 dev = make_float2(0.f, 0.f);
+            T d[9];  // TOT, MOM: f_l - f_opp(l) of the nine pairs, the species added
 #pragma unroll
             for (int s = 0; s < 2; ++s) {  // unrolled, so that the per-species values stay in registers
                 if (s >= C.ns) break;
@@ -272,7 +289,7 @@ __global__ void __launch_bounds__(128, TOT || sizeof(T) == 8 ? 8 : 16)
                     const T u = f[(s * 19 + l) * C.plane + i], v = f[(s * 19 + l + 1) * C.plane + i];
                     a += u;
                     a += v;
-                    if constexpr (TOT) d[l / 2] = s == 0 ? u - v : d[l / 2] + (u - v);
+                    if constexpr (TOT || MOM) d[l / 2] = s == 0 ? u - v : d[l / 2] + (u - v);
                 }
                 rho[s] = C.rho_ref[s] + a;
                 psi[s] = psi3(C, s, rho[s]);
@@ -282,12 +299,24 @@ __global__ void __launch_bounds__(128, TOT || sizeof(T) == 8 ? 8 : 16)
                     else
                         mass1 += (double)a;
                 }
+                if constexpr (MOM) (s == 0 ? dev.x : dev.y) = a;
             }
-            if constexpr (TOT) {
+            if constexpr (TOT || MOM) {
                 // velocities 1, 3, 5 along x, y, z, then (1,1,0), (1,-1,0), (1,0,1), (1,0,-1), (0,1,1), (0,1,-1)
-                momx += (double)(d[0] + ((d[3] + d[4]) + (d[5] + d[6])));
-                momy += (double)(d[1] + ((d[3] - d[4]) + (d[7] + d[8])));
-                momz += (double)(d[2] + ((d[5] - d[6]) + (d[7] - d[8])));
+                const T mx = d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
+                const T my = d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
+                const T mz = d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
+                if constexpr (TOT) {
+                    momx += (double)mx;
+                    momy += (double)my;
+                    momz += (double)mz;
+                }
+                if constexpr (MOM) {
+                    dn[i] = dev;
+                    jt[i] = mx;
+                    jt[C.plane + i] = my;
+                    jt[2 * C.plane + i] = mz;
+                }
             }
             V pv, rv;
             pv.x = psi[0];
@@ -348,7 +377,8 @@ __global__ void __launch_bounds__(256)
 
 // ---- k3_step -----------------------------------------------------------------------------
 
-enum { K3_WRITE = 1, K3_FIELDS = 2 };
+// K3_RELAX (FP32, tau = 1): the pass over moments
+enum { K3_WRITE = 1, K3_FIELDS = 2, K3_RELAX = 4 };
 
 template <typename T, int TY, int TZ>
 struct Smem3 {
@@ -560,7 +590,7 @@ __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T
             fields[s * n + k] = (double)rho[s];
 #pragma unroll
             for (int l = 0; l < 19; ++l)
-                fields[(NS + 3 + s * 19 + l) * n + k] = (double)f[s][l] + w19<double>(l) * (double)C.rho_ref[s];
+                fields[(NS + 3 + s * 19 + l) * n + k] = wide3(f[s][l]) + w19<double>(l) * (double)C.rho_ref[s];
         }
         fields[(NS + 0) * n + k] = (double)(mxs / rt);
         fields[(NS + 1) * n + k] = (double)(mys / rt);
@@ -684,13 +714,313 @@ __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T
     }
 }
 
+// ---- full relaxation: the state as moments ------------------------------------------------------
+
+// The state after a fully relaxed collision, as (A, B) pairs of FP32 in the layout of a population
+// plane: the density deviation d (from rho_ref), the velocity u of the species' equilibrium, and
+// base = d - 3/2 rho u.u, which its populations share:
+//   f*_l - w_l rho_ref = w_l (base + rho c.u (3 + 9/2 c.u)).
+// d has two copies (k3_stream reads the neighbours' old one while it writes the new).  jt holds the
+// streamed-in lattice momentum, the species added (R5's common velocity needs no more at tau = 1).
+// With one species the B half is zero.
+struct Mom3 {
+    float2* d[2];
+    float2 *base, *ux, *uy, *uz;
+    float *jx, *jy, *jz;
+};
+
+// cu: c.u, or with sg = -1 its negative: (-cu) (3 - 9/2 cu) = cu (9/2 cu - 3) to the bit.
+__device__ __forceinline__ float2 relaxed_pop(float w, float2 base, float2 rho, float2 cu, int sg) {
+    return vmul(vsplat(w), vfma(vmul(rho, cu), vfma(vsplat(4.5f), cu, vsplat(sg > 0 ? 3.f : -3.f)), base));
+}
+
+// What has streamed into a site so far: density and momentum, species side by side.
+struct Sum3 {
+    float2 r, x, y, z;
+};
+
+// Adds population f of velocity (CX, CY, CZ).
+template <int CX, int CY, int CZ>
+__device__ __forceinline__ void gain(Sum3& S, float2 f) {
+    S.r = vadd(S.r, f);
+    if constexpr (CX != 0) S.x = CX > 0 ? vadd(S.x, f) : vsub(S.x, f);
+    if constexpr (CY != 0) S.y = CY > 0 ? vadd(S.y, f) : vsub(S.y, f);
+    if constexpr (CZ != 0) S.z = CZ > 0 ? vadd(S.z, f) : vsub(S.z, f);
+}
+
+// One site of a neighbouring column: what its populations need.
+struct Col3 {
+    float2 base, rho, ux, uy, uz;
+};
+template <int CX, int CY, int CZ>
+__device__ __forceinline__ void stream_in(Sum3& S, const Col3& c) {
+    constexpr float w = CX == 0 && CY == 0 && CZ == 0 ? 1.f / 3.f : (CX * CX + CY * CY + CZ * CZ == 1 ? 1.f / 18.f : 1.f / 36.f);
+    if constexpr (CX == 0 && CY == 0 && CZ == 0) {
+        gain<0, 0, 0>(S, vmul(vsplat(w), c.base));
+    } else {
+        // c.u up to the sign of its first component, which relaxed_pop takes
+        constexpr int sg = CX ? CX : (CY ? CY : CZ);
+        float2 cu = CX ? c.ux : (CY ? c.uy : c.uz);
+        if constexpr (CX != 0 && CY != 0) cu = CY * sg > 0 ? vadd(cu, c.uy) : vsub(cu, c.uy);
+        if constexpr ((CX != 0 || CY != 0) && CZ != 0) cu = CZ * sg > 0 ? vadd(cu, c.uz) : vsub(cu, c.uz);
+        gain<CX, CY, CZ>(S, relaxed_pop(w, c.base, c.rho, cu, sg));
+    }
+}
+// The population (CX, CY, CZ) coming back from a wall: the site's own opposite one, with Ladd's term.
+template <int CX, int CY, int CZ>
+__device__ __forceinline__ void wall_in(Sum3& S, const Col3& c, float uw) {
+    constexpr float w = CX * CX + CY * CY + CZ * CZ == 1 ? 1.f / 18.f : 1.f / 36.f;
+    float2 cu = c.uz;  // of the opposite velocity, up to the sign of its z component
+    if constexpr (CX != 0) cu = CX * CZ > 0 ? vadd(cu, c.ux) : vsub(cu, c.ux);
+    if constexpr (CY != 0) cu = CY * CZ > 0 ? vadd(cu, c.uy) : vsub(cu, c.uy);
+    float2 f = relaxed_pop(w, c.base, c.rho, cu, -CZ);
+    if constexpr (CX != 0) f = vfma(vsplat(6.f * CX * w), vmul(c.rho, vsplat(uw)), f);
+    gain<CX, CY, CZ>(S, f);
+}
+
+// The streaming pass.  A thread owns a column (x, y) of `chunk` layers and walks up it, one source
+// layer at a time: each layer's nine columns around it are read once (37 pairs) and give to the
+// three layers they stream to, so a site costs 37 (chunk + 2) / chunk reads instead of 67.  The
+// order of the additions (from below, from the same layer, from above) is the same whatever the
+// chunk.  With TOT the block's FP64 partials of the state's totals too (as k3_density's).
+// Bound by instruction issue and L1 (about 240 instructions and 300 B of reads per site) with the
+// whole state in L2 at 128^3.
+template <int NS, bool TOT>
+__global__ void __launch_bounds__(128, 4)
+    k3_stream(const Mom3 M, int dc, float* __restrict__ vol, const Step3<float> C, int chunk, double* __restrict__ part) {
+    pdl_enter();
+    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y;
+    const bool live = x < C.nx && y < C.ny;
+    const int z0 = blockIdx.z * chunk, z1 = min(z0 + chunk, C.nz);
+    double tot[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    if (live) {
+        const int xm = x == 0 ? C.nx - 1 : x - 1, xp = x == C.nx - 1 ? 0 : x + 1;
+        // rows within a layer, whose sites number less than 2^31
+        const int r0 = y * C.pitch, rm = (y == 0 ? C.ny - 1 : y - 1) * C.pitch, rp = (y == C.ny - 1 ? 0 : y + 1) * C.pitch;
+        const long long lay = (long long)C.ny * C.pitch;
+        const float2* const D = dc ? M.d[1] : M.d[0];
+        float2* const Dn = dc ? M.d[0] : M.d[1];
+        const float2 rref = make_float2(C.rho_ref[0], C.rho_ref[1]);
+        float2* const P = reinterpret_cast<float2*>(vol);
+        int xs[2 * GX + 1], ys[2 * GY + 1], zs_[2 * GZ + 1];
+        const int nxl = ghost_list(x, C.nx, GX, false, xs);
+        const int nyl = ghost_list(y, C.ny, GY, false, ys);
+        const bool edge = nxl > 1 || nyl > 1;
+        const Sum3 none = {vsplat(0.f), vsplat(0.f), vsplat(0.f), vsplat(0.f)};
+        // layers zs - 1 (complete after this source layer), zs, zs + 1
+        Sum3 below = none, here = none, above = none;
+        const bool walls = C.zbc != 0;
+        for (int zs = z0 - 1; zs <= z1; ++zs) {
+            const bool in = zs >= 0 && zs < C.nz;
+            if (in || !walls) {
+                const long long o = lay * (in ? zs : (zs < 0 ? zs + C.nz : zs - C.nz));
+                const float2 *const pb = M.base + o, *const pd = D + o, *const px = M.ux + o, *const py = M.uy + o,
+                                   *const pz = M.uz + o;
+#define LBM3_COL(name, off, X, Y, Z)  \
+    Col3 name;                        \
+    {                                 \
+        const int k_ = (off);         \
+        name.base = pb[k_];           \
+        name.rho = vadd(rref, pd[k_]); \
+        if (X) name.ux = px[k_];      \
+        if (Y) name.uy = py[k_];      \
+        if (Z) name.uz = pz[k_];      \
+    }
+                {
+                    LBM3_COL(c, r0 + x, true, true, true)
+                    stream_in<0, 0, -1>(below, c);
+                    stream_in<0, 0, 0>(here, c);
+                    stream_in<0, 0, 1>(above, c);
+                    if (walls && zs == 0) {  // `here` is the bottom layer: nothing came from below
+                        Sum3 own = none;
+                        wall_in<0, 0, 1>(own, c, C.wall_u[0]);
+                        wall_in<1, 0, 1>(own, c, C.wall_u[0]);
+                        wall_in<-1, 0, 1>(own, c, C.wall_u[0]);
+                        wall_in<0, 1, 1>(own, c, C.wall_u[0]);
+                        wall_in<0, -1, 1>(own, c, C.wall_u[0]);
+                        here.r = vadd(here.r, own.r);
+                        here.x = vadd(here.x, own.x);
+                        here.y = vadd(here.y, own.y);
+                        here.z = vadd(here.z, own.z);
+                    }
+                    if (walls && zs == C.nz - 1) {  // `here` is the top layer: nothing will come from above
+                        wall_in<0, 0, -1>(here, c, C.wall_u[1]);
+                        wall_in<1, 0, -1>(here, c, C.wall_u[1]);
+                        wall_in<-1, 0, -1>(here, c, C.wall_u[1]);
+                        wall_in<0, 1, -1>(here, c, C.wall_u[1]);
+                        wall_in<0, -1, -1>(here, c, C.wall_u[1]);
+                    }
+                }
+                {
+                    LBM3_COL(c, r0 + xm, true, false, true)
+                    stream_in<1, 0, -1>(below, c);
+                    stream_in<1, 0, 0>(here, c);
+                    stream_in<1, 0, 1>(above, c);
+                }
+                {
+                    LBM3_COL(c, r0 + xp, true, false, true)
+                    stream_in<-1, 0, -1>(below, c);
+                    stream_in<-1, 0, 0>(here, c);
+                    stream_in<-1, 0, 1>(above, c);
+                }
+                {
+                    LBM3_COL(c, rm + x, false, true, true)
+                    stream_in<0, 1, -1>(below, c);
+                    stream_in<0, 1, 0>(here, c);
+                    stream_in<0, 1, 1>(above, c);
+                }
+                {
+                    LBM3_COL(c, rp + x, false, true, true)
+                    stream_in<0, -1, -1>(below, c);
+                    stream_in<0, -1, 0>(here, c);
+                    stream_in<0, -1, 1>(above, c);
+                }
+                if (zs >= z0 && zs < z1) {  // the diagonals stay in their layer
+                    {
+                        LBM3_COL(c, rm + xm, true, true, false)
+                        stream_in<1, 1, 0>(here, c);
+                    }
+                    {
+                        LBM3_COL(c, rp + xp, true, true, false)
+                        stream_in<-1, -1, 0>(here, c);
+                    }
+                    {
+                        LBM3_COL(c, rp + xm, true, true, false)
+                        stream_in<1, -1, 0>(here, c);
+                    }
+                    {
+                        LBM3_COL(c, rm + xp, true, true, false)
+                        stream_in<-1, 1, 0>(here, c);
+                    }
+                }
+#undef LBM3_COL
+            }
+            const int z = zs - 1;  // complete
+            if (z >= z0) {
+                const long long i = lay * z + r0 + x;
+                Dn[i] = below.r;
+                const float jx = below.x.x + below.x.y, jy = below.y.x + below.y.y, jz = below.z.x + below.z.y;
+                M.jx[i] = jx;
+                M.jy[i] = jy;
+                M.jz[i] = jz;
+                const float2 rho = vadd(rref, below.r);
+                float2 psi = make_float2(psi3(C, 0, rho.x), NS == 2 ? psi3(C, 1, rho.y) : 0.f);
+                if constexpr (TOT) {
+                    tot[0] += (double)below.r.x;
+                    if (NS == 2) tot[1] += (double)below.r.y;
+                    tot[2] += (double)jx;
+                    tot[3] += (double)jy;
+                    tot[4] += (double)jz;
+                }
+                float2* const own = P + ((long long)(z + GZ) * C.gy + (y + GY)) * C.gpitch + (x + GX);
+                own[0] = psi;
+                own[C.gvol] = rho;
+                if (edge || z < GZ || z >= C.nz - GZ) {  // and where ghosts repeat the site
+                    const int nzl = ghost_list(z, C.nz, GZ, walls, zs_);
+                    for (int c = 0; c < nzl; ++c)
+                        for (int b = 0; b < nyl; ++b)
+                            for (int a = c == 0 && b == 0 ? 1 : 0; a < nxl; ++a) {
+                                const long long k = ((long long)zs_[c] * C.gy + ys[b]) * C.gpitch + xs[a];
+                                P[k] = psi;
+                                P[C.gvol + k] = rho;
+                            }
+                }
+            }
+            below = here;
+            here = above;
+            above = none;
+        }
+    }
+    if constexpr (TOT) {
+        __shared__ double red[5][128];
+        const int t = threadIdx.y * 32 + threadIdx.x;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) red[q][t] = tot[q];
+        __syncthreads();
+        for (int h = 64; h > 0; h >>= 1) {
+            if (t < h)
+                for (int q = 0; q < 5; ++q) red[q][t] += red[q][t + h];
+            __syncthreads();
+        }
+        const long long blk = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        if (t < 5) part[blk * 5 + t] = red[t][0];
+    }
+}
+
+// The site update of the relaxing pass (k3_step, K3_RELAX): from the force, the streamed-in density
+// and momentum, the species' velocities and base.
+template <int NS>
+__device__ __forceinline__ void relax3(const Step3<float>& C, const Mom3& M, const float (&F)[2][3], float2 rho,
+                                       long long i, float jx, float jy, float jz, float2 d, int* __restrict__ flag) {
+    bool bad = !(rho.x > 0.f) || !(rho.x < 1e30f);
+    if (NS == 2) bad = bad || !(rho.y > 0.f) || !(rho.y < 1e30f);
+    if (bad) atomicOr(flag, 1);
+    const float iden = 1.f / (NS == 2 ? sadd(rho.x, rho.y) : rho.x);
+    const float2 ir = make_float2(1.f / rho.x, NS == 2 ? 1.f / rho.y : 0.f);
+    const float2 fx = make_float2(sfma(rho.x, C.g, F[0][0]), NS == 2 ? sfma(rho.y, C.g, F[1][0]) : 0.f);
+    const float2 fy = make_float2(F[0][1], NS == 2 ? F[1][1] : 0.f), fz = make_float2(F[0][2], NS == 2 ? F[1][2] : 0.f);
+    const float px = smul(jx, iden), py = smul(jy, iden), pz = smul(jz, iden);
+    float2 ux = vfma(fx, ir, vsplat(px)), uy = vfma(fy, ir, vsplat(py)), uz = vfma(fz, ir, vsplat(pz));
+    if (NS == 1) ux.y = uy.y = uz.y = 0.f;
+    const float2 u15 = vmul(vsplat(1.5f), vfma(ux, ux, vfma(uy, uy, vmul(uz, uz))));
+    M.base[i] = vsub(d, vmul(rho, u15));
+    M.ux[i] = ux;
+    M.uy[i] = uy;
+    M.uz[i] = uz;
+}
+
+// Populations of the state after streaming, from the moments, into f: what streams into each site,
+// population by population (k3_stream's arithmetic).
+template <int NS>
+__global__ void __launch_bounds__(128) k3_expand(const Mom3 M, int dc, float* __restrict__ f, const Step3<float> C) {
+    const int x = blockIdx.x * 128 + threadIdx.x;
+    if (x >= C.nx) return;
+    const float2 rref = make_float2(C.rho_ref[0], C.rho_ref[1]);
+    for (int z = blockIdx.z; z < C.nz; z += gridDim.z)
+        for (int y = blockIdx.y; y < C.ny; y += gridDim.y) {
+            const long long i = ((long long)z * C.ny + y) * C.pitch + x;
+#pragma unroll
+            for (int l = 0; l < 19; ++l) {
+                const int cx = c3x(l), cy = c3y(l), cz = c3z(l);
+                int xs = x - cx, ys = y - cy, zs = z - cz;
+                xs = xs < 0 ? xs + C.nx : (xs >= C.nx ? xs - C.nx : xs);
+                ys = ys < 0 ? ys + C.ny : (ys >= C.ny ? ys - C.ny : ys);
+                const bool wall = C.zbc && (zs < 0 || zs >= C.nz);
+                zs = zs < 0 ? zs + C.nz : (zs >= C.nz ? zs - C.nz : zs);
+                const long long k = wall ? i : ((long long)zs * C.ny + ys) * C.pitch + xs;
+                const float2 base = M.base[k], rho = vadd(rref, (dc ? M.d[1] : M.d[0])[k]);
+                const float2 ux = M.ux[k], uy = M.uy[k], uz = M.uz[k];
+                float2 v;
+                if (l == 0) {
+                    v = vmul(vsplat(w19<float>(0)), base);
+                } else if (!wall) {  // as stream_in
+                    const int sg = cx ? cx : (cy ? cy : cz);
+                    float2 cu = cx ? ux : (cy ? uy : uz);
+                    if (cx && cy) cu = cy * sg > 0 ? vadd(cu, uy) : vsub(cu, uy);
+                    if ((cx || cy) && cz) cu = cz * sg > 0 ? vadd(cu, uz) : vsub(cu, uz);
+                    v = relaxed_pop(w19<float>(l), base, rho, cu, sg);
+                } else {  // as wall_in
+                    float2 cu = uz;
+                    if (cx) cu = cx * cz > 0 ? vadd(cu, ux) : vsub(cu, ux);
+                    if (cy) cu = cy * cz > 0 ? vadd(cu, uy) : vsub(cu, uy);
+                    v = relaxed_pop(w19<float>(l), base, rho, cu, -cz);
+                    if (cx) v = vfma(vsplat(6.f * cx * w19<float>(l)), vmul(rho, vsplat(cz > 0 ? C.wall_u[0] : C.wall_u[1])), v);
+                }
+                f[l * C.plane + i] = v.x;
+                if (NS == 2) f[(19 + l) * C.plane + i] = v.y;
+            }
+        }
+}
+
 // FP32 tiles of 256 threads: 3 CTAs per SM (80 registers, 16 bytes of spills), measured faster than
 // 2 CTAs at 110 registers without spills -- the kernel waits on memory and more warps hide it.
 template <typename T, int MODE, int NS, int TY, int TZ>
 __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
-                                  Tile3<T>::TX* TY* TZ > 256 ? 1 : (sizeof(T) == 4 ? 3 : 512 / (Tile3<T>::TX * TY * TZ)))
+                                  Tile3<T>::TX* TY* TZ > 256 ? (MODE == K3_RELAX ? 2 : 1)
+                                                             : (sizeof(T) == 4 ? (MODE == K3_RELAX ? 4 : 3)
+                                                                               : 512 / (Tile3<T>::TX * TY * TZ)))
     k3_step(const __grid_constant__ CUtensorMap vmap, const T* __restrict__ fin, T* __restrict__ fout,
-            const Step3<T> C, int* __restrict__ flag, double* __restrict__ fields) {
+            const Step3<T> C, int* __restrict__ flag, double* __restrict__ fields, const Mom3 M, int dn) {
     constexpr int TX = Tile3<T>::TX;
     extern __shared__ __align__(1024) unsigned char smem3[];
     Smem3<T, TY, TZ>& S = *reinterpret_cast<Smem3<T, TY, TZ>*>(smem3);
@@ -716,12 +1046,22 @@ __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
     // own populations from HBM while the box is on its way
     const long long i = ((long long)z * C.ny + y) * C.pitch + x;
     // (FP64, short of registers, loads them after the force: its other warps cover the wait)
-    T f[NS][19];
+    // K3_RELAX: the streamed-in density and momentum instead
+    T f[MODE == K3_RELAX ? 1 : NS][19];
+    float jx = 0.f, jy = 0.f, jz = 0.f;
+    float2 d = make_float2(0.f, 0.f);
     const auto load = [&]() {
+        if constexpr (MODE == K3_RELAX) {
+            d = (dn ? M.d[1] : M.d[0])[i];
+            jx = M.jx[i];
+            jy = M.jy[i];
+            jz = M.jz[i];
+        } else {
 #pragma unroll
-        for (int s = 0; s < NS; ++s)
+            for (int s = 0; s < NS; ++s)
 #pragma unroll
-            for (int l = 0; l < 19; ++l) f[s][l] = fin[(s * 19 + l) * C.plane + i];
+                for (int l = 0; l < 19; ++l) f[s][l] = fin[(s * 19 + l) * C.plane + i];
+        }
     };
     if (sizeof(T) == 4 && live) load();
     __syncthreads();  // the barrier is initialised before anyone waits on it
@@ -770,7 +1110,10 @@ __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
         C, [&](int dx, int dy, int dz) { return S.box[0][bz + dz][by + dy][bx + dx]; },
         [&](int dx, int dy, int dz) { return S.box[1][bz + dz][by + dy][bx + dx]; }, F);
     if (sizeof(T) == 8) load();
-    site3<T, NS, MODE>(C, f, F, x, y, z, i, fout, flag, fields);
+    if constexpr (MODE == K3_RELAX)
+        relax3<NS>(C, M, F, S.box[1][bz][by][bx], i, jx, jy, jz, d, flag);
+    else
+        site3<T, NS, MODE>(C, f, F, x, y, z, i, fout, flag, fields);
 }
 
 // ---- equilibrium at rest, totals ---------------------------------------------------------------
@@ -790,7 +1133,7 @@ __global__ void k3_init(T* __restrict__ f, const double* __restrict__ rho, const
 
 template <typename T, int MODE, int NS, int TY, int TZ>
 cudaError_t launch_step3(const CUtensorMap& map, const T* fin, T* fout, const Step3<T>& C, int* flag, double* fields,
-                         cudaStream_t st) {
+                         const Mom3& M, int dn, cudaStream_t st) {
     const size_t smem = sizeof(Smem3<T, TY, TZ>);
     static bool attr = false;  // per template instance
     if (!attr) {
@@ -801,17 +1144,18 @@ cudaError_t launch_step3(const CUtensorMap& map, const T* fin, T* fout, const St
     }
     constexpr int TX = Tile3<T>::TX;
     const dim3 grid((C.nx + TX - 1) / TX, (C.ny + TY - 1) / TY, (C.nz + TZ - 1) / TZ);
-    return launch_pdl(k3_step<T, MODE, NS, TY, TZ>, grid, dim3(TX, TY, TZ), smem, st, map, fin, fout, C, flag, fields);
+    return launch_pdl(k3_step<T, MODE, NS, TY, TZ>, grid, dim3(TX, TY, TZ), smem, st, map, fin, fout, C, flag, fields, M,
+                      dn);
 }
 
 template <typename T, int MODE, int NS>
 cudaError_t launch_shape(int shape, const CUtensorMap& map, const T* fin, T* fout, const Step3<T>& C, int* flag,
-                         double* fields, cudaStream_t st) {
+                         double* fields, const Mom3& M, int dn, cudaStream_t st) {
     switch (shape) {
-        case 0: return launch_step3<T, MODE, NS, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, st);
-        case 1: return launch_step3<T, MODE, NS, Tile3<T>::ty(1), Tile3<T>::tz(1)>(map, fin, fout, C, flag, fields, st);
-        case 2: return launch_step3<T, MODE, NS, Tile3<T>::ty(2), Tile3<T>::tz(2)>(map, fin, fout, C, flag, fields, st);
-        case 3: return launch_step3<T, MODE, NS, Tile3<T>::ty(3), Tile3<T>::tz(3)>(map, fin, fout, C, flag, fields, st);
+        case 0: return launch_step3<T, MODE, NS, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st);
+        case 1: return launch_step3<T, MODE, NS, Tile3<T>::ty(1), Tile3<T>::tz(1)>(map, fin, fout, C, flag, fields, M, dn, st);
+        case 2: return launch_step3<T, MODE, NS, Tile3<T>::ty(2), Tile3<T>::tz(2)>(map, fin, fout, C, flag, fields, M, dn, st);
+        case 3: return launch_step3<T, MODE, NS, Tile3<T>::ty(3), Tile3<T>::tz(3)>(map, fin, fout, C, flag, fields, M, dn, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -819,12 +1163,17 @@ cudaError_t launch_shape(int shape, const CUtensorMap& map, const T* fin, T* fou
 // the step pass in the chosen tile shape; the fields pass (lbm3_get_fields) in shape 0
 template <typename T>
 cudaError_t launch_step3_any(int mode, int ns, int shape, const CUtensorMap& map, const T* fin, T* fout,
-                             const Step3<T>& C, int* flag, double* fields, cudaStream_t st) {
+                             const Step3<T>& C, int* flag, double* fields, const Mom3& M, int dn, cudaStream_t st) {
+    if constexpr (sizeof(T) == 4) {
+        if (mode == K3_RELAX)
+            return ns == 2 ? launch_shape<T, K3_RELAX, 2>(shape, map, fin, fout, C, flag, fields, M, dn, st)
+                           : launch_shape<T, K3_RELAX, 1>(shape, map, fin, fout, C, flag, fields, M, dn, st);
+    }
     if (mode == K3_WRITE)
-        return ns == 2 ? launch_shape<T, K3_WRITE, 2>(shape, map, fin, fout, C, flag, fields, st)
-                       : launch_shape<T, K3_WRITE, 1>(shape, map, fin, fout, C, flag, fields, st);
-    return ns == 2 ? launch_step3<T, K3_FIELDS, 2, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, st)
-                   : launch_step3<T, K3_FIELDS, 1, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, st);
+        return ns == 2 ? launch_shape<T, K3_WRITE, 2>(shape, map, fin, fout, C, flag, fields, M, dn, st)
+                       : launch_shape<T, K3_WRITE, 1>(shape, map, fin, fout, C, flag, fields, M, dn, st);
+    return ns == 2 ? launch_step3<T, K3_FIELDS, 2, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st)
+                   : launch_step3<T, K3_FIELDS, 1, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st);
 }
 
 }  // namespace lbm3
@@ -848,6 +1197,11 @@ struct lbm3_ctx {
     void* vol = nullptr;               // psi and rho volumes: [2][gz][gy][gpitch] pairs
     alignas(64) unsigned char map[NSHAPE][128] = {};  // TMA descriptors of vol, per tile shape
     int shape = 0;                     // tile shape of the step pass (lbm3_autotune)
+    // FP32 at tau = 1: the state is held as moments (Mom3), which live in f[cur ^ 1], and f[cur] is
+    // stale; mom: that is so now; dc: which copy of the densities is current; chunk: k3_stream's
+    bool mom = false;
+    int dc = 0;
+    int chunk = 8;
     int* flag = nullptr;
     double* staging = nullptr;         // lbm3_get_fields / lbm3_set_fields from the host
     size_t staging_bytes = 0;
@@ -969,6 +1323,8 @@ static void release3(lbm3_ctx* c) {
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
 }
 
+static dim3 stream_grid3(const lbm3_ctx* c);
+
 static int make_vol_map(lbm3_ctx* c, int shape) {
     const auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(lbm::tensor_map_encoder());
     if (!encode) return 1;
@@ -1053,7 +1409,12 @@ extern "C" int lbm3_create(lbm3_ctx** out, const lbm3_desc* d) {
         c->tot_grid[2] = gz;
         c->nblk_den = gx * gy * gz;
     }
-    CKC3(cudaMalloc(&c->part, (size_t)c->nblk_den * 5 * sizeof(double)));
+    // k3_stream: chunks of 8 layers while they fill the GPU, shorter ones on small lattices
+    while (c->chunk > 1 && (long long)((nx + 31) / 32) * ((ny + 3) / 4) * ((nz + c->chunk - 1) / c->chunk) < 4LL * nsm)
+        c->chunk /= 2;
+    const dim3 sg = stream_grid3(c);
+    const size_t parts = std::max<size_t>(c->nblk_den, (size_t)sg.x * sg.y * sg.z);
+    CKC3(cudaMalloc(&c->part, parts * 5 * sizeof(double)));
     CKC3(cudaMalloc(&c->tot, 5 * sizeof(double)));
     CKC3(cudaMalloc(&c->dcheck, lbm::DCHECK_DOUBLES * sizeof(double)));
     for (int k = 0; k < NSHAPE; ++k)
@@ -1076,6 +1437,8 @@ extern "C" void lbm3_destroy(lbm3_ctx* c) {
 
 extern "C" const char* lbm3_last_error(const lbm3_ctx* c) { return c ? c->err.c_str() : g3_create_error.c_str(); }
 
+static cudaError_t expand3(lbm3_ctx* c);
+
 extern "C" int lbm3_set_params(lbm3_ctx* c, const lbm_params* p) {
     if (!c) return LBM_EINVAL;
     if (!p) return fail3(c, LBM_EINVAL, "params is NULL");
@@ -1083,8 +1446,19 @@ extern "C" int lbm3_set_params(lbm3_ctx* c, const lbm_params* p) {
         return fail3(c, LBM_EINVAL, "invalid parameters: %s", lbm_last_error(nullptr));
     if (p->weight_preset != LBM_WEIGHTS_PAPER) return fail3(c, LBM_EINVAL, "the 3-D step has the paper's weights only");
     if (p->psi_wall != LBM_WALL_MIRROR) return fail3(c, LBM_EINVAL, "the 3-D step has the mirror wall reading only");
+    const lbm_params was = c->p;
     c->p = *p;
     c->have_params = true;
+    // moments hold the state only under the relaxation times (all 1) and wall velocities it was formed
+    // with (a population leaving through a wall is reflected by the step that sends it): under others
+    // it goes on as the populations those give
+    const bool keep = p->tau[0] == 1.0 && (c->d.n_species == 1 || p->tau[1] == 1.0) &&
+                      (c->d.z_boundary == LBM_PERIODIC || (p->wall_u[0] == was.wall_u[0] && p->wall_u[1] == was.wall_u[1]));
+    if (c->mom && !keep) {
+        CK3(cudaSetDevice(c->d.device));
+        CK3(expand3(c));  // with the constants of the steps taken
+        c->mom = false;
+    }
     refresh3(c);
     return LBM_OK;
 }
@@ -1138,6 +1512,7 @@ extern "C" int lbm3_set_fields(lbm3_ctx* c, const double* rho, int where) {
     CK3(cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
     CK3(cudaStreamSynchronize(c->stream));
     c->cur = 0;
+    c->mom = false;
     c->step = 0;
     c->have_fields = true;
     return LBM_OK;
@@ -1145,39 +1520,115 @@ extern "C" int lbm3_set_fields(lbm3_ctx* c, const double* rho, int where) {
 
 // the density pass over f[cur] into the volumes; totals: its block partials of the totals of
 // f[cur] summed into out (5 doubles, device memory) as well
-static cudaError_t density3(lbm3_ctx* c, double* totals = nullptr) {
+static Mom3 moments3(const lbm3_ctx* c) {
+    float* p = static_cast<float*>(c->f[c->cur ^ 1]);  // 15 planes of the 19 or 38
+    const long long n = c->plane;
+    Mom3 M;
+    float2** pair[] = {&M.d[0], &M.d[1], &M.base, &M.ux, &M.uy, &M.uz};
+    for (int k = 0; k < 6; ++k) *pair[k] = reinterpret_cast<float2*>(p + 2 * k * n);
+    M.jx = p + 12 * n;
+    M.jy = p + 13 * n;
+    M.jz = p + 14 * n;
+    return M;
+}
+
+// Whether a step relaxes every population fully to its equilibrium (and the context holds FP32).
+static bool relaxed3(const lbm3_ctx* c) {
+    return c->d.precision == LBM_FP32 && c->c32.omega[0] == 1.0f && (c->d.n_species == 1 || c->c32.omega[1] == 1.0f);
+}
+
+static dim3 stream_grid3(const lbm3_ctx* c) {
+    return dim3((c->d.nx + 31) / 32, (c->d.ny + 3) / 4, (c->d.nz + c->chunk - 1) / c->chunk);
+}
+
+// The populations of the state held as moments into f[cur]; the state stays what it is.
+static cudaError_t expand3(lbm3_ctx* c) {
+    const dim3 grid((c->d.nx + 127) / 128, c->d.ny, c->d.nz);
+    const Mom3 M = moments3(c);
+    if (c->d.n_species == 2)
+        k3_expand<2><<<grid, 128, 0, c->stream>>>(M, c->dc, (float*)c->f[c->cur], c->c32);
+    else
+        k3_expand<1><<<grid, 128, 0, c->stream>>>(M, c->dc, (float*)c->f[c->cur], c->c32);
+    return cudaGetLastError();
+}
+
+// The density and momentum that stream into every site of a state held as moments (and psi and rho
+// into the volumes), with the totals' partials.
+static cudaError_t stream3(lbm3_ctx* c, bool totals) {
+    const dim3 grid = stream_grid3(c), block(32, 4);
+    const Mom3 M = moments3(c);
+    float* vol = (float*)c->vol;
+    if (c->d.n_species == 2)
+        return totals ? launch_pdl(k3_stream<2, true>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk, c->part)
+                      : launch_pdl(k3_stream<2, false>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk,
+                                   (double*)nullptr);
+    return totals ? launch_pdl(k3_stream<1, true>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk, c->part)
+                  : launch_pdl(k3_stream<1, false>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk,
+                               (double*)nullptr);
+}
+
+// read: for a read of the state's densities only (no collision follows)
+static cudaError_t density3(lbm3_ctx* c, double* totals = nullptr, bool read = false) {
     const dim3 grid = totals ? dim3(c->tot_grid[0], c->tot_grid[1], c->tot_grid[2])
                              : dim3((c->d.nx + 127) / 128, c->d.ny, c->d.nz);
     const dim3 block(128);
     cudaError_t e;
     if (c->d.precision == LBM_FP64)
         e = totals ? launch_pdl(lbm3::k3_density<double, true>, grid, block, 0, c->stream, (const double*)c->f[c->cur],
-                                (double*)c->vol, c->c64, c->part)
+                                (double*)c->vol, c->c64, c->part, (float2*)nullptr, (float*)nullptr)
                    : launch_pdl(lbm3::k3_density<double, false>, grid, block, 0, c->stream,
-                                (const double*)c->f[c->cur], (double*)c->vol, c->c64, (double*)nullptr);
-    else
+                                (const double*)c->f[c->cur], (double*)c->vol, c->c64, (double*)nullptr,
+                                (float2*)nullptr, (float*)nullptr);
+    else if (c->mom && !read) {
+        e = stream3(c, totals != nullptr);
+    } else if (relaxed3(c) && !read) {  // populations, on the way to moments
+        const Mom3 M = moments3(c);
+        e = totals ? launch_pdl(lbm3::k3_density<float, true, true>, grid, block, 0, c->stream,
+                                (const float*)c->f[c->cur], (float*)c->vol, c->c32, c->part, M.d[c->dc ^ 1], M.jx)
+                   : launch_pdl(lbm3::k3_density<float, false, true>, grid, block, 0, c->stream,
+                                (const float*)c->f[c->cur], (float*)c->vol, c->c32, (double*)nullptr, M.d[c->dc ^ 1],
+                                M.jx);
+    } else {
         e = totals ? launch_pdl(lbm3::k3_density<float, true>, grid, block, 0, c->stream, (const float*)c->f[c->cur],
-                                (float*)c->vol, c->c32, c->part)
+                                (float*)c->vol, c->c32, c->part, (float2*)nullptr, (float*)nullptr)
                    : launch_pdl(lbm3::k3_density<float, false>, grid, block, 0, c->stream, (const float*)c->f[c->cur],
-                                (float*)c->vol, c->c32, (double*)nullptr);
+                                (float*)c->vol, c->c32, (double*)nullptr, (float2*)nullptr, (float*)nullptr);
+    }
     if (e != cudaSuccess || !totals) return e;
+    const dim3 sg = stream_grid3(c);
+    const int nblk = c->mom && !read ? (int)(sg.x * sg.y * sg.z) : c->nblk_den;
     // the reference densities the FP32 deviations are taken from (zero in FP64, and for an absent
     // species), once per site
     const double n = (double)c->n;
     const double r0 = c->d.precision == LBM_FP64 ? 0.0 : (double)c->c32.rho_ref[0];
     const double r1 = c->d.precision == LBM_FP64 ? 0.0 : (double)c->c32.rho_ref[1];
-    lbm3::k3_totals_sum<<<1, 256, 0, c->stream>>>(c->part, c->nblk_den, n * r0, n * r1, totals);
+    lbm3::k3_totals_sum<<<1, 256, 0, c->stream>>>(c->part, nblk, n * r0, n * r1, totals);
     return cudaGetLastError();
 }
 
+// The collide pass of a step (K3_WRITE, after density3: it makes the new state the current one), or
+// K3_FIELDS.
 static cudaError_t collide3(lbm3_ctx* c, int mode, double* fields) {
+    const bool relax = mode == K3_WRITE && relaxed3(c);
     const int shape = mode == K3_WRITE ? c->shape : 0;
     const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(c->map[shape]);
+    cudaError_t e;
     if (c->d.precision == LBM_FP64)
-        return launch_step3_any<double>(mode, c->d.n_species, shape, map, (const double*)c->f[c->cur],
-                                        (double*)c->f[c->cur ^ 1], c->c64, c->flag, fields, c->stream);
-    return launch_step3_any<float>(mode, c->d.n_species, shape, map, (const float*)c->f[c->cur],
-                                   (float*)c->f[c->cur ^ 1], c->c32, c->flag, fields, c->stream);
+        e = launch_step3_any<double>(mode, c->d.n_species, shape, map, (const double*)c->f[c->cur],
+                                     (double*)c->f[c->cur ^ 1], c->c64, c->flag, fields, Mom3{}, 0, c->stream);
+    else
+        e = launch_step3_any<float>(relax ? K3_RELAX : mode, c->d.n_species, shape, map, (const float*)c->f[c->cur],
+                                    (float*)c->f[c->cur ^ 1], c->c32, c->flag, fields, moments3(c), c->dc ^ 1,
+                                    c->stream);
+    if (e == cudaSuccess && mode == K3_WRITE) {
+        if (relax) {
+            c->mom = true;
+            c->dc ^= 1;
+        } else {
+            c->cur ^= 1;
+        }
+    }
+    return e;
 }
 
 // one step: the density pass and the collide pass (bracketed by events while profiling)
@@ -1201,7 +1652,6 @@ static int one_step3(lbm3_ctx* c) {
     }
     CK3(collide3(c, K3_WRITE, nullptr));
     if (e) CK3(cudaEventRecord(e[3], c->stream));
-    c->cur ^= 1;
     c->step += 1;
     return LBM_OK;
 }
@@ -1244,7 +1694,6 @@ extern "C" int lbm3_step_totals(lbm3_ctx* c, int nsteps, double* dst, long long 
     for (int k = 0; k < nsteps; ++k) {
         if (k == 0) CK3(density3(c));
         CK3(collide3(c, K3_WRITE, nullptr));
-        c->cur ^= 1;
         c->step += 1;
         CK3(density3(c, out + (long long)k * (stride / (long long)sizeof(double))));
     }
@@ -1290,7 +1739,8 @@ extern "C" int lbm3_get_fields(lbm3_ctx* c, double* rho, double* u, double* f, i
     const size_t per = (size_t)(ns + 3 + 19 * ns);
     int rc = staging3(c, per * n * sizeof(double));
     if (rc) return rc;
-    CK3(density3(c));
+    if (c->mom) CK3(expand3(c));
+    CK3(density3(c, nullptr, true));
     CK3(collide3(c, K3_FIELDS, c->staging));
     const cudaMemcpyKind kind = where == LBM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     if (rho) CK3(cudaMemcpyAsync(rho, c->staging, (size_t)ns * n * sizeof(double), kind, c->stream));
@@ -1350,12 +1800,15 @@ extern "C" int lbm3_autotune(lbm3_ctx* c, int steps, int* chosen, double* ms) {
     if (steps < 1 || steps > 10000) return fail3(c, LBM_EINVAL, "steps must be in 1 .. 10000");
     if (!c->have_fields) return fail3(c, LBM_EINVAL, "lbm3_set_fields has not been called");
     CK3(cudaSetDevice(c->d.device));
-    // the state is kept aside and put back: the shapes change the schedule, not the arithmetic
-    const size_t fbytes = (size_t)c->d.n_species * 19 * c->plane * c->esize;
+    // the state is kept aside and put back: the shapes change the schedule, not the arithmetic (held as
+    // moments it is 15 planes of the other buffer)
+    const int cur0 = c->cur, shape0 = c->shape, dc0 = c->dc;
+    const bool mom0 = c->mom;
+    void* const at = c->f[mom0 ? cur0 ^ 1 : cur0];
+    const size_t fbytes = (mom0 ? (size_t)15 : (size_t)c->d.n_species * 19) * c->plane * c->esize;
     void* saved = nullptr;
     CK3(cudaMalloc(&saved, fbytes));
-    cudaError_t e = cudaMemcpyAsync(saved, c->f[c->cur], fbytes, cudaMemcpyDeviceToDevice, c->stream);
-    const int cur0 = c->cur, shape0 = c->shape;
+    cudaError_t e = cudaMemcpyAsync(saved, at, fbytes, cudaMemcpyDeviceToDevice, c->stream);
     const long long step0 = c->step;
     cudaEvent_t a = nullptr, b = nullptr;
     if (e == cudaSuccess) e = cudaEventCreate(&a);
@@ -1364,12 +1817,12 @@ extern "C" int lbm3_autotune(lbm3_ctx* c, int steps, int* chosen, double* ms) {
     int best = 0;
     for (int k = 0; k < NSHAPE && e == cudaSuccess; ++k) {
         c->shape = k;
-        e = collide3(c, K3_WRITE, nullptr);  // one untimed pass (module load, caches)
+        e = density3(c);  // one untimed step (module load, caches)
+        if (e == cudaSuccess) e = collide3(c, K3_WRITE, nullptr);
         if (e == cudaSuccess) e = cudaEventRecord(a, c->stream);
         for (int i = 0; i < steps && e == cudaSuccess; ++i) {
             e = density3(c);
             if (e == cudaSuccess) e = collide3(c, K3_WRITE, nullptr);
-            c->cur ^= 1;
         }
         if (e == cudaSuccess) e = cudaEventRecord(b, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(b);
@@ -1378,13 +1831,17 @@ extern "C" int lbm3_autotune(lbm3_ctx* c, int steps, int* chosen, double* ms) {
         t[k] = (double)v / steps;
         if (t[k] < t[best]) best = k;
         c->cur = cur0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(c->f[c->cur], saved, fbytes, cudaMemcpyDeviceToDevice, c->stream);
+        c->mom = mom0;
+        c->dc = dc0;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(at, saved, fbytes, cudaMemcpyDeviceToDevice, c->stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (a) cudaEventDestroy(a);
     if (b) cudaEventDestroy(b);
     cudaFree(saved);
     c->cur = cur0;
+    c->mom = mom0;
+    c->dc = dc0;
     c->step = step0;
     c->shape = e == cudaSuccess ? best : shape0;
     CK3(e);
