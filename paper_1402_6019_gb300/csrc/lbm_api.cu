@@ -437,6 +437,10 @@ extern "C" int lbm_create(lbm_ctx** out, const lbm_desc* d) {
         const int modes[5] = {M_WRITE, M_WRITE | M_OBS | per, M_OBS | per, M_FIELDS, M_WRITE | M_RECORD};
         for (int m : modes)
             for (int st = 1; st <= 2; ++st) {
+                if (d->precision == LBM_FP64 && st == 2) {  // one depth
+                    c->pull_grid[m][1][0] = c->pull_grid[m][0][0];
+                    break;
+                }
                 const int nb = d->precision == LBM_FP64 ? pull_blocks_per_sm<double>(ns, m, st, narrow)
                                                         : pull_blocks_per_sm<float>(ns, m, st, 32);
                 if (nb < 1) return bail(fail(c, LBM_ECUDA, "occupancy query of the pull kernel failed"));

@@ -349,6 +349,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
     const int rot = !WALL && ninst == 1 && ntz > 2 ? ntiles - ntx : 0;  // work order (describe)
     // work items of the folded reduction: blocks of rows, then blocks of columns
     const int nrb = (nz + RB_THREADS / 32 - 1) / (RB_THREADS / 32);
+    // (more CTAs than tiles and items together: each item has a CTA of its own)
     const int nfold = Rd.enabled ? nrb + (nx + RB_THREADS / 32 - 1) / (RB_THREADS / 32) : 0;
 
     // threads with a ring position (ring_position), RPW per warp; the observing builds keep it in
@@ -382,6 +383,13 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
     // buffers or the counters.
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    const bool own_items = nfold > 0 && (int)gridDim.x >= ntiles + nfold;
+    if (own_items && (int)blockIdx.x >= ntiles) {
+        reduce_block<T, SH::NW>((int)blockIdx.x - ntiles, Rd.part_row, Rd.part_col, O.flag, Rd.nxpart, Rd.nzpart, nx, nz,
+                                C.zbc, nrb, Rd.out, Rd.avg, Rd.bpart, Rd.bavg, Rd.accumulate, T(Rd.inx), T(Rd.inz),
+                                S.wsc, ninst > 1 ? inst : nullptr, ninst);
+        return;
+    }
     if (tid == 0) {
         if (blockIdx.x == 0) {  // the next launch's counters (this launch's were zeroed by the last)
             ctr_next[0] = 0u;
@@ -399,7 +407,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
             more = S.ti[sl].t < ntiles;
             if (more && sl == 0) issue_load(S, &tin, S.ti[0].x0, S.ti[0].prow0 + S.ti[0].z0, 0);
         }
-        if (more) upcoming = min(nstat + (int)atomicAdd(ctr, 1u), ntiles);
+        if (more && nstat < ntiles) upcoming = min(nstat + (int)atomicAdd(ctr, 1u), ntiles);
     }
     __syncthreads();
     // thread 0: the reduction's counter as last seen (no draw), during the CTA's last tiles
@@ -854,7 +862,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
             static_cast<T*>(O.part_col)[((long long)prev_x * ntz + prev_jg) * NQC + tz] = v;
         }
     }
-    if (nfold > 0 && !failed) {
+    if (nfold > 0 && !own_items && !failed) {
         // the previous pass's reduction: work items from the second counter until they run out
         for (;;) {
             if (tid == 0) S.fold_item = fold_seen < nfold ? (int)atomicAdd(ctr + 1, 1u) : nfold;
@@ -897,8 +905,10 @@ cudaError_t launch_mode(const void* tin, T* fout, const StepConst<T>& C, const O
                         T* rec) {
     const int ntx = (C.nx + Shape<SHP>::W - 1) / Shape<SHP>::W;
     const long long ntiles = (long long)ntx * B.ntz;
-    int grid = (int)(ntiles < grid_max ? ntiles : grid_max);
-    if (Rd.enabled && grid < 1) grid = 1;
+    // small lattices: the previous pass's reduction runs beside the tiles, on CTAs of its own, where it
+    // would otherwise follow them (a draw, a round of loads and two barriers: 2 us of a 7 us launch)
+    const long long items = Rd.enabled ? reduce_blocks(C.nx, C.nz) : 0;
+    int grid = (int)(ntiles + items <= grid_max ? ntiles + items : (ntiles < grid_max ? ntiles : grid_max));
     PairConst K{};
     if constexpr (kPair<T, NS>) fill_pair_const(K, C);
     // launched with programmatic stream serialisation: it may start while the kernel before it
