@@ -55,20 +55,6 @@ __global__ void k_init(int ns, T* __restrict__ f, const double* __restrict__ rho
     }
 }
 
-// Where the gather of the pull layout reads population l of site (x, z) (as pull_slot), taking
-// x - c_l and, without walls, z - c_l from the ghost columns and rows, which hold the periodic
-// images of the current state: no wrapping.  For reads only (a write must go to the wrapped slot).
-template <typename T>
-__device__ __forceinline__ long long pull_src(const StepConst<T>& C, int x, int z, int nz, int prow0, int l, int& ls) {
-    const int zs = z - cz(l);
-    if (C.zbc && (zs < 0 || zs >= nz)) {
-        ls = opp(l);
-        return (long long)(prow0 + z + PULL_GZ) * C.pitch + x + PULL_GX;
-    }
-    ls = l;
-    return (long long)(prow0 + zs + PULL_GZ) * C.pitch + (x - cx(l) + PULL_GX);
-}
-
 // W_l rho_ref of each species' rest, axis and diagonal populations, and as two floats hi + lo.
 struct ExportBase {
     double base[6];
@@ -92,44 +78,59 @@ __device__ __forceinline__ O plain_value(T v, double base, float hi, float lo) {
 }
 
 // The post-streaming populations as plain values, [ns][9][nz][nx]: the stored value of (x, l) in
-// the push layout, the gather of the pull layout.  Blocks of 32 columns x 8 EXPORT_ROWS rows of one
-// population (blockIdx.z = s * 9 + l), a thread EXPORT_ROWS rows 8 apart: with one value a thread the
-// 1.2 M blocks of a 4096 x 4096 lattice took their turns, not the bytes, 1180 us.
-constexpr int EXPORT_ROWS = 8;
+// the push layout, the gather of the pull layout (pull_slot's, with x - c_l and, without walls,
+// z - c_l taken from the ghosts, which hold the periodic images: no wrapping).  Blocks of 32 columns x
+// EXPORT_Z rows of one population (blockIdx.z = s * 9 + l), a thread EXPORT_ROWS rows 8 apart, all
+// read before they are written.  Bound by instruction issue: at 4096 x 4096 one value a thread took
+// 1180 us, eight with the slot worked out for each 840, and each row's lattice searched for by every
+// thread 1200 at 48 channels of 13.4 M sites; here a row costs its wall test and one
+// multiply-add, and a batch's rows are looked up once per block.
+constexpr int EXPORT_ROWS = 8, EXPORT_Z = 8 * EXPORT_ROWS;
 template <typename T, typename O>
 __global__ void __launch_bounds__(256) k_export(int ns, const T* __restrict__ f, O* __restrict__ out,
                                                 const StepConst<T> C, const __grid_constant__ ExportBase B,
                                                 const InstGeom* __restrict__ inst, int ninst) {
-    const long long n = (long long)C.nx * C.nz;
+    // a batch's rows: padded row, and bit 0 / 1: next to its lattice's bottom / top wall
+    __shared__ int prow[EXPORT_Z];
+    __shared__ unsigned char edge[EXPORT_Z];
     const int s = blockIdx.z / 9, l = blockIdx.z % 9;
-    const int x = blockIdx.x * 32 + threadIdx.x, z0 = blockIdx.y * (8 * EXPORT_ROWS) + threadIdx.y;
+    const int x = blockIdx.x * 32 + threadIdx.x, zb = blockIdx.y * EXPORT_Z;
+    const bool batch = inst && ninst > 1;
+    if (batch) {
+        const int t = threadIdx.y * 32 + threadIdx.x;
+        if (t < EXPORT_Z && zb + t < C.nz) {
+            const InstGeom& I = inst[inst_of_row(inst, ninst, zb + t)];
+            const int z = zb + t - I.zrow0;
+            prow[t] = I.prow0 + z + PULL_GZ;
+            edge[t] = (unsigned char)((z == 0 ? 1 : 0) | (z == I.nz - 1 ? 2 : 0));
+        }
+        __syncthreads();
+    }
     if (x >= C.nx) return;
     const int k = s * 3 + (l == 0 ? 0 : (l <= 4 ? 1 : 2));
     const double base = B.base[k];
     const float hi = B.hi[k], lo = B.lo[k];
+    const int c = cz(l);
+    const int beyond = C.zbc ? (c > 0 ? 1 : (c < 0 ? 2 : 0)) : 0;  // the edge this population comes back from
+    // where a row's values start: streamed in (one row over), or reflected at a wall
+    const T* const from = f + (s * 9 + l) * C.plane + (inst ? x + PULL_GX - cx(l) : x);
+    const T* const back = f + (s * 9 + opp(l)) * C.plane + (x + PULL_GX);
     T v[EXPORT_ROWS];
 #pragma unroll
     for (int r = 0; r < EXPORT_ROWS; ++r) {
-        const int zg = z0 + 8 * r;
-        if (zg >= C.nz) break;
-        long long o = (long long)zg * C.pitch + x;
-        int ls = l;
+        const int t = threadIdx.y + 8 * r, zg = min(zb + t, C.nz - 1);
+        const T* p = from + (long long)zg * C.pitch;
         if (inst) {
-            if (ninst > 1) {
-                const int q = inst_of_row(inst, ninst, zg);
-                o = pull_src(C, x, zg - inst[q].zrow0, inst[q].nz, inst[q].prow0, l, ls);
-            } else {  // one lattice: its rows start at padded row PULL_GZ
-                o = pull_src(C, x, zg, C.nz, 0, l, ls);
-            }
+            const int row = batch ? prow[zg - zb] : zg + PULL_GZ;
+            const int e = batch ? edge[zg - zb] : (zg == 0 ? 1 : 0) | (zg == C.nz - 1 ? 2 : 0);
+            p = (e & beyond) ? back + (long long)row * C.pitch : from + (long long)(row - c) * C.pitch;
         }
-        v[r] = f[(s * 9 + ls) * C.plane + o];
+        v[r] = *p;
     }
-    O* const to = out + (s * 9 + l) * n + x;
+    O* to = out + ((long long)(s * 9 + l) * C.nz + zb + threadIdx.y) * C.nx + x;
 #pragma unroll
-    for (int r = 0; r < EXPORT_ROWS; ++r) {
-        const int zg = z0 + 8 * r;
-        if (zg < C.nz) to[(long long)zg * C.nx] = plain_value<T, O>(v[r], base, hi, lo);
-    }
+    for (int r = 0; r < EXPORT_ROWS; ++r, to += 8LL * C.nx)
+        if (zb + (int)threadIdx.y + 8 * r < C.nz) *to = plain_value<T, O>(v[r], base, hi, lo);
 }
 
 // The inverse of k_export: plain FP64 post-streaming values in, stored values out.
@@ -277,7 +278,7 @@ cudaError_t launch_init(int ns, T* f, const double* rho, const double* u, const 
 
 template <typename T, typename O>
 cudaError_t launch_export(int ns, const T* f, O* out, const StepConst<T>& C, const Batch* B, cudaStream_t st) {
-    const dim3 grid((C.nx + 31) / 32, (C.nz + 8 * EXPORT_ROWS - 1) / (8 * EXPORT_ROWS), 9 * ns);
+    const dim3 grid((C.nx + 31) / 32, (C.nz + EXPORT_Z - 1) / EXPORT_Z, 9 * ns);
     ExportBase E;
     for (int k = 0; k < 6; ++k) {
         const int l[3] = {0, 1, 5};
