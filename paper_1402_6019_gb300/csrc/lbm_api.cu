@@ -111,6 +111,8 @@ struct lbm_ctx {
     size_t ev_used = 0;
     std::vector<cudaEvent_t> aev;  // adjoint: three pairs per step, around its kernels
     size_t aev_used = 0;
+    cudaStream_t side = nullptr;   // lbm_adjoint_sweep: the sweep's stream beside the recording's
+    cudaEvent_t sev[4] = {};       // its events: states recorded [0, 1], states swept back [2, 3], by buffer
     unsigned serial = 0;           // this context's number among the contexts of the process
     unsigned snap_seq = 0;         // snapshots written so far
     std::map<const void*, SnapTail> snaps;  // tails of this context's latest snapshots, by address
@@ -269,6 +271,9 @@ static void release(lbm_ctx* c) {
     c->aev.clear();
     for (cudaEvent_t& e : c->tev)
         if (e) cudaEventDestroy(e);
+    for (cudaEvent_t& e : c->sev)
+        if (e) cudaEventDestroy(e);
+    if (c->side) cudaStreamDestroy(c->side);
     void* ptrs[] = {c->f_raw[0],   c->f_raw[1], c->part_row[0], c->part_row[1], c->part_col[0],
                     c->part_col[1], c->sched,   c->ticket,      c->flag,        c->out,
                     c->avg,         c->staging, c->fexport,     c->gfield,      c->inst_d,
@@ -1546,6 +1551,54 @@ extern "C" int lbm_adjoint_steps(lbm_ctx* c, int nsteps, const void* states, voi
                                      (double*)lam, (double*)lam, grad);
     return adjoint_steps<float>(c, A, nsteps, (const float*)states, (const float*)lam, (float*)c->adj_lam,
                                 (float*)lam, (float*)lam, grad);
+}
+
+extern "C" int lbm_adjoint_sweep(lbm_ctx* c, int nseg, const void* const* snaps, const int* nsteps, void* seg,
+                                 void* seg2, void* lam, double* grad, int precision) {
+    if (!c) return LBM_EINVAL;
+    if (nseg < 0 || !lam || !grad || (nseg > 0 && (!snaps || !nsteps || !seg))) return fail(c, LBM_EINVAL, "bad argument");
+    for (int k = 0; k < nseg; ++k)
+        if (!snaps[k] || nsteps[k] < 0) return fail(c, LBM_EINVAL, "snaps[%d] is NULL or nsteps[%d] < 0", k, k);
+    CK(cudaSetDevice(c->d.device));
+    // one after the other: one buffer, one segment, or kernels timed by events on the stream
+    if (!seg2 || nseg < 2 || c->profiling) {
+        for (int k = nseg - 1; k >= 0; --k) {
+            if (int r = lbm_restore_own(c, snaps[k])) return r;
+            if (int r = lbm_record_states(c, nsteps[k], seg, precision)) return r;
+            if (int r = lbm_adjoint_steps(c, nsteps[k], seg, lam, grad, precision)) return r;
+        }
+        return LBM_OK;
+    }
+    if (!c->side) CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+    for (cudaEvent_t& e : c->sev)
+        if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    void* const buf[2] = {seg, seg2};
+    cudaStream_t const main = c->stream;
+    int rc = LBM_OK;
+    auto ck = [&](cudaError_t e) {
+        if (rc == LBM_OK && e != cudaSuccess) rc = fail(c, LBM_ECUDA, "lbm_adjoint_sweep: %s", cudaGetErrorString(e));
+    };
+    // segment k uses buffer b; it is recorded on the context's stream once segment k + 2 has been
+    // swept out of that buffer, and swept back on the side stream, which so follows main throughout
+    bool swept[2] = {false, false};
+    for (int k = nseg - 1, b = 0; k >= 0 && rc == LBM_OK; --k, b ^= 1) {
+        if (swept[b]) ck(cudaStreamWaitEvent(main, c->sev[2 + b], 0));
+        if (rc == LBM_OK) rc = lbm_restore_own(c, snaps[k]);
+        if (rc == LBM_OK) rc = lbm_record_states(c, nsteps[k], buf[b], precision);
+        ck(cudaEventRecord(c->sev[b], main));
+        ck(cudaStreamWaitEvent(c->side, c->sev[b], 0));
+        if (rc != LBM_OK) break;
+        c->stream = c->side;  // the adjoint calls neither read nor change the context's own state
+        rc = lbm_adjoint_steps(c, nsteps[k], buf[b], lam, grad, precision);
+        c->stream = main;
+        ck(cudaEventRecord(c->sev[2 + b], c->side));
+        swept[b] = true;
+    }
+    // what follows on the context's stream waits for the sweep, also after an error
+    const cudaError_t e1 = cudaEventRecord(c->sev[2], c->side), e2 = cudaStreamWaitEvent(main, c->sev[2], 0);
+    ck(e1);
+    ck(e2);
+    return rc;
 }
 
 extern "C" int lbm_adjoint_objective(lbm_ctx* c, const void* f, const double* target_u, const double* target_rho,

@@ -104,6 +104,8 @@ SIGNATURES = {
     "lbm_record_states": (ctypes.c_int, [_VP, ctypes.c_int, _VP, ctypes.c_int]),
     "lbm_adjoint_step": (ctypes.c_int, [_VP, _VP, _VP, _VP, _VP, ctypes.c_int]),
     "lbm_adjoint_steps": (ctypes.c_int, [_VP, ctypes.c_int, _VP, _VP, _VP, ctypes.c_int]),
+    "lbm_adjoint_sweep": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.POINTER(_VP), ctypes.POINTER(ctypes.c_int), _VP, _VP,
+                                         _VP, _VP, ctypes.c_int]),
     "lbm_adjoint_objective": (ctypes.c_int, [_VP, _VP, _VP, _VP, _VP, _VP, ctypes.c_int]),
     "lbm_adjoint_initial": (ctypes.c_int, [_VP, _VP, _VP, ctypes.c_int]),
     "lbm3_default_desc": (None, [ctypes.POINTER(lbm3_desc)]),
@@ -360,6 +362,15 @@ def lbm_adjoint_step(h, f, lam_next, lam, grad):
 def lbm_adjoint_steps(h, nsteps, states, lam, grad):
     """lam (in place): dJ/df after the recorded steps -> dJ/df before them; grad += dJ/dtheta."""
     _check(load().lbm_adjoint_steps(h, int(nsteps), _dev(states), _dev(lam), _dev(grad), _prec(states, lam)), h)
+
+
+def lbm_adjoint_sweep(h, snaps, nsteps, seg, seg2, lam, grad):
+    """The backward sweep of a checkpointed run from its snapshots; seg, seg2 (or None): CUDA tensors
+    for the largest segment's states; lam and grad as in lbm_adjoint_steps (asynchronous)."""
+    n = len(snaps)
+    ptrs = (_VP * n)(*[s.data_ptr() for s in snaps])
+    counts = (ctypes.c_int * n)(*[int(k) for k in nsteps])
+    _check(load().lbm_adjoint_sweep(h, n, ptrs, counts, _dev(seg), _dev(seg2), _dev(lam), _dev(grad), _prec(seg, lam)), h)
 
 
 def lbm_adjoint_objective(h, f, target_u, target_rho, J, dJdf=None):
