@@ -353,32 +353,30 @@ __global__ void __launch_bounds__(128, TOT || MOM || sizeof(T) == 8 ? 8 : 16)
     }
 }
 
-// out = mass A, mass B, momentum x, y, z: the sum of part[b][q] over the nblk blocks (thread t adds
-// blocks t, t + 256, ... in order, then a fixed tree over the threads; FP64, the same bits on every
-// call), plus base[q] (the sites times rho_ref,s for the masses).
-__global__ void __launch_bounds__(256)
+// out = mass A, mass B, momentum x, y, z: the sum of part[b][q] over the nblk blocks (64 threads per
+// quantity, thread t adding blocks t, t + 64, ... in order, then a fixed tree; FP64, the same bits on
+// every call), plus base[q] (the sites times rho_ref,s for the masses).
+__global__ void __launch_bounds__(320)
     k3_totals_sum(const double* __restrict__ part, int nblk, double base0, double base1, double* __restrict__ out) {
-    __shared__ double red[5][256];
-    double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nblk; b += 256)
-        for (int q = 0; q < 5; ++q) a[q] += part[b * 5 + q];
-    for (int q = 0; q < 5; ++q) red[q][threadIdx.x] = a[q];
+    __shared__ double red[10];
+    pdl_enter();
+    const int q = threadIdx.x / 64, t = threadIdx.x % 64;
+    double a = 0.0;
+#pragma unroll 4
+    for (int b = t; b < nblk; b += 64) a += part[b * 5 + q];
+    for (int h = 16; h > 0; h >>= 1) a += __shfl_xor_sync(0xffffffffu, a, h);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = a;
     __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h)
-            for (int q = 0; q < 5; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + h];
-        __syncthreads();
-    }
     if (threadIdx.x < 5) {
         const double base = threadIdx.x == 0 ? base0 : (threadIdx.x == 1 ? base1 : 0.0);
-        out[threadIdx.x] = red[threadIdx.x][0] + base;
+        out[threadIdx.x] = (red[2 * threadIdx.x] + red[2 * threadIdx.x + 1]) + base;
     }
 }
 
 // ---- k3_step -----------------------------------------------------------------------------
 
-// K3_RELAX (FP32, tau = 1): the pass over moments
-enum { K3_WRITE = 1, K3_FIELDS = 2, K3_RELAX = 4 };
+// (FP32, tau = 1) K3_RELAX: the pass over moments; K3_LOOK: rho and u of a state held as moments
+enum { K3_WRITE = 1, K3_FIELDS = 2, K3_RELAX = 4, K3_LOOK = 8 };
 
 template <typename T, int TY, int TZ>
 struct Smem3 {
@@ -532,6 +530,11 @@ __device__ __forceinline__ void force3(const Step3<T>& C, const PSF& ps, const R
 #undef RH
 }
 
+// Where the fields of a state go (device memory, FP64; null: not wanted).
+struct Fields3 {
+    double *rho, *u, *f;
+};
+
 // The moments of the site's populations f, the body force along x, the common velocity of R5;
 // then (K3_FIELDS) rho_s, u and the plain populations into `fields`, or (K3_WRITE) the
 // shifted-velocity BGK of Sec. II and the push of the new populations to x + c_l.  Every scalar
@@ -540,7 +543,7 @@ __device__ __forceinline__ void force3(const Step3<T>& C, const PSF& ps, const R
 template <typename T, int NS, int MODE>
 __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T (&F)[2][3], int x, int y, int z,
                                       long long i, T* __restrict__ fout, int* __restrict__ flag,
-                                      double* __restrict__ fields) {
+                                      const Fields3& fields) {
     using V = typename PairOf<T>::V;
     // ---- moments, body force, common velocity ----
     T rho[NS], ir[NS], jx[NS], jy[NS], jz[NS], drho[NS];
@@ -587,14 +590,18 @@ __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T
             mys += jy[s] + T(0.5) * F[s][1];
             mzs += jz[s] + T(0.5) * F[s][2];
             rt += rho[s];
-            fields[s * n + k] = (double)rho[s];
+            if (fields.rho) fields.rho[s * n + k] = (double)rho[s];
+            if (fields.f) {
 #pragma unroll
-            for (int l = 0; l < 19; ++l)
-                fields[(NS + 3 + s * 19 + l) * n + k] = wide3(f[s][l]) + w19<double>(l) * (double)C.rho_ref[s];
+                for (int l = 0; l < 19; ++l)
+                    fields.f[(s * 19 + l) * n + k] = wide3(f[s][l]) + w19<double>(l) * (double)C.rho_ref[s];
+            }
         }
-        fields[(NS + 0) * n + k] = (double)(mxs / rt);
-        fields[(NS + 1) * n + k] = (double)(mys / rt);
-        fields[(NS + 2) * n + k] = (double)(mzs / rt);
+        if (fields.u) {
+            fields.u[k] = (double)(mxs / rt);
+            fields.u[n + k] = (double)(mys / rt);
+            fields.u[2 * n + k] = (double)(mzs / rt);
+        }
     }
 
     if constexpr ((MODE & K3_WRITE) != 0) {
@@ -729,23 +736,36 @@ struct Mom3 {
     float *jx, *jy, *jz;
 };
 
-// cu: c.u, or with sg = -1 its negative: (-cu) (3 - 9/2 cu) = cu (9/2 cu - 3) to the bit.
-__device__ __forceinline__ float2 relaxed_pop(float w, float2 base, float2 rho, float2 cu, int sg) {
-    return vmul(vsplat(w), vfma(vmul(rho, cu), vfma(vsplat(4.5f), cu, vsplat(sg > 0 ? 3.f : -3.f)), base));
+// That population over w_l; cu: c.u, or with sg = -1 its negative: (-cu) (3 - 9/2 cu) = cu (9/2 cu - 3)
+// to the bit.
+__device__ __forceinline__ float2 relaxed_pop(float2 base, float2 rho, float2 cu, int sg) {
+    return vfma(vmul(rho, cu), vfma(vsplat(4.5f), cu, vsplat(sg > 0 ? 3.f : -3.f)), base);
 }
 
-// What has streamed into a site so far: density and momentum, species side by side.
+// What has streamed into a site so far: density and momentum, species side by side, times 36 (the
+// weights 12, 2 and 1 are exact, and a site is scaled once).
 struct Sum3 {
     float2 r, x, y, z;
 };
 
-// Adds population f of velocity (CX, CY, CZ).
+// v / 36 to the last rounding (1/36 in FP32 alone is 7e-9 too large: the same growth every step).
+__device__ __forceinline__ float2 over36(float2 v) {
+    constexpr float hi = (float)(1.0 / 36.0), lo = (float)(1.0 / 36.0 - (double)hi);
+    return vfma(v, vsplat(hi), vmul(v, vsplat(lo)));
+}
+
+// Adds population 36 w g of velocity (CX, CY, CZ), w = 1/18 (axes: W2 = 2) or 1/36 (edges: 1).
 template <int CX, int CY, int CZ>
-__device__ __forceinline__ void gain(Sum3& S, float2 f) {
-    S.r = vadd(S.r, f);
-    if constexpr (CX != 0) S.x = CX > 0 ? vadd(S.x, f) : vsub(S.x, f);
-    if constexpr (CY != 0) S.y = CY > 0 ? vadd(S.y, f) : vsub(S.y, f);
-    if constexpr (CZ != 0) S.z = CZ > 0 ? vadd(S.z, f) : vsub(S.z, f);
+__device__ __forceinline__ void gain(Sum3& S, float2 g) {
+    constexpr float W2 = CX * CX + CY * CY + CZ * CZ == 1 ? 2.f : 1.f;
+    const auto add = [&](float2 a, float sign) {
+        if (W2 == 1.f) return sign > 0 ? vadd(a, g) : vsub(a, g);
+        return vfma(vsplat(sign * W2), g, a);
+    };
+    S.r = add(S.r, 1.f);
+    if constexpr (CX != 0) S.x = add(S.x, (float)CX);
+    if constexpr (CY != 0) S.y = add(S.y, (float)CY);
+    if constexpr (CZ != 0) S.z = add(S.z, (float)CZ);
 }
 
 // One site of a neighbouring column: what its populations need.
@@ -754,27 +774,25 @@ struct Col3 {
 };
 template <int CX, int CY, int CZ>
 __device__ __forceinline__ void stream_in(Sum3& S, const Col3& c) {
-    constexpr float w = CX == 0 && CY == 0 && CZ == 0 ? 1.f / 3.f : (CX * CX + CY * CY + CZ * CZ == 1 ? 1.f / 18.f : 1.f / 36.f);
     if constexpr (CX == 0 && CY == 0 && CZ == 0) {
-        gain<0, 0, 0>(S, vmul(vsplat(w), c.base));
+        S.r = vfma(vsplat(12.f), c.base, S.r);
     } else {
         // c.u up to the sign of its first component, which relaxed_pop takes
         constexpr int sg = CX ? CX : (CY ? CY : CZ);
         float2 cu = CX ? c.ux : (CY ? c.uy : c.uz);
         if constexpr (CX != 0 && CY != 0) cu = CY * sg > 0 ? vadd(cu, c.uy) : vsub(cu, c.uy);
         if constexpr ((CX != 0 || CY != 0) && CZ != 0) cu = CZ * sg > 0 ? vadd(cu, c.uz) : vsub(cu, c.uz);
-        gain<CX, CY, CZ>(S, relaxed_pop(w, c.base, c.rho, cu, sg));
+        gain<CX, CY, CZ>(S, relaxed_pop(c.base, c.rho, cu, sg));
     }
 }
 // The population (CX, CY, CZ) coming back from a wall: the site's own opposite one, with Ladd's term.
 template <int CX, int CY, int CZ>
 __device__ __forceinline__ void wall_in(Sum3& S, const Col3& c, float uw) {
-    constexpr float w = CX * CX + CY * CY + CZ * CZ == 1 ? 1.f / 18.f : 1.f / 36.f;
     float2 cu = c.uz;  // of the opposite velocity, up to the sign of its z component
     if constexpr (CX != 0) cu = CX * CZ > 0 ? vadd(cu, c.ux) : vsub(cu, c.ux);
     if constexpr (CY != 0) cu = CY * CZ > 0 ? vadd(cu, c.uy) : vsub(cu, c.uy);
-    float2 f = relaxed_pop(w, c.base, c.rho, cu, -CZ);
-    if constexpr (CX != 0) f = vfma(vsplat(6.f * CX * w), vmul(c.rho, vsplat(uw)), f);
+    float2 f = relaxed_pop(c.base, c.rho, cu, -CZ);
+    if constexpr (CX != 0) f = vfma(vsplat(6.f * CX), vmul(c.rho, vsplat(uw)), f);
     gain<CX, CY, CZ>(S, f);
 }
 
@@ -898,16 +916,17 @@ __global__ void __launch_bounds__(128, 4)
             const int z = zs - 1;  // complete
             if (z >= z0) {
                 const long long i = lay * z + r0 + x;
-                Dn[i] = below.r;
-                const float jx = below.x.x + below.x.y, jy = below.y.x + below.y.y, jz = below.z.x + below.z.y;
+                const float2 dn = over36(below.r), px = over36(below.x), py = over36(below.y), pz = over36(below.z);
+                Dn[i] = dn;
+                const float jx = px.x + px.y, jy = py.x + py.y, jz = pz.x + pz.y;
                 M.jx[i] = jx;
                 M.jy[i] = jy;
                 M.jz[i] = jz;
-                const float2 rho = vadd(rref, below.r);
+                const float2 rho = vadd(rref, dn);
                 float2 psi = make_float2(psi3(C, 0, rho.x), NS == 2 ? psi3(C, 1, rho.y) : 0.f);
                 if constexpr (TOT) {
-                    tot[0] += (double)below.r.x;
-                    if (NS == 2) tot[1] += (double)below.r.y;
+                    tot[0] += (double)dn.x;
+                    if (NS == 2) tot[1] += (double)dn.y;
                     tot[2] += (double)jx;
                     tot[3] += (double)jy;
                     tot[4] += (double)jz;
@@ -969,10 +988,30 @@ __device__ __forceinline__ void relax3(const Step3<float>& C, const Mom3& M, con
     M.uz[i] = uz;
 }
 
-// Populations of the state after streaming, from the moments, into f: what streams into each site,
-// population by population (k3_stream's arithmetic).
+// rho_s and the barycentric velocity (sum_s j_s + F_s / 2) / sum_s rho_s of a site (K3_LOOK).
 template <int NS>
-__global__ void __launch_bounds__(128) k3_expand(const Mom3 M, int dc, float* __restrict__ f, const Step3<float> C) {
+__device__ __forceinline__ void look3(const Step3<float>& C, const float (&F)[2][3], float2 rho, long long k, float jx,
+                                      float jy, float jz, const Fields3& out) {
+    const long long n = (long long)C.nx * C.ny * C.nz;
+    const float irt = 1.f / (NS == 2 ? sadd(rho.x, rho.y) : rho.x);
+    float fx = sfma(rho.x, C.g, F[0][0]), fy = F[0][1], fz = F[0][2];
+    if (NS == 2) fx = sadd(fx, sfma(rho.y, C.g, F[1][0])), fy = sadd(fy, F[1][1]), fz = sadd(fz, F[1][2]);
+    if (out.rho) {
+        out.rho[k] = wide3(rho.x);
+        if (NS == 2) out.rho[n + k] = wide3(rho.y);
+    }
+    if (out.u) {
+        out.u[k] = wide3(smul(sfma(0.5f, fx, jx), irt));
+        out.u[n + k] = wide3(smul(sfma(0.5f, fy, jy), irt));
+        out.u[2 * n + k] = wide3(smul(sfma(0.5f, fz, jz), irt));
+    }
+}
+
+// Populations of the state after streaming, from the moments, into f: what streams into each site,
+// population by population (k3_stream's terms).  O = float: the stored populations; double: the plain
+// values of lbm3_get_fields.
+template <int NS, typename O>
+__global__ void __launch_bounds__(128) k3_expand(const Mom3 M, int dc, O* __restrict__ f, const Step3<float> C) {
     const int x = blockIdx.x * 128 + threadIdx.x;
     if (x >= C.nx) return;
     const float2 rref = make_float2(C.rho_ref[0], C.rho_ref[1]);
@@ -998,16 +1037,23 @@ __global__ void __launch_bounds__(128) k3_expand(const Mom3 M, int dc, float* __
                     float2 cu = cx ? ux : (cy ? uy : uz);
                     if (cx && cy) cu = cy * sg > 0 ? vadd(cu, uy) : vsub(cu, uy);
                     if ((cx || cy) && cz) cu = cz * sg > 0 ? vadd(cu, uz) : vsub(cu, uz);
-                    v = relaxed_pop(w19<float>(l), base, rho, cu, sg);
+                    v = vmul(vsplat(w19<float>(l)), relaxed_pop(base, rho, cu, sg));
                 } else {  // as wall_in
                     float2 cu = uz;
                     if (cx) cu = cx * cz > 0 ? vadd(cu, ux) : vsub(cu, ux);
                     if (cy) cu = cy * cz > 0 ? vadd(cu, uy) : vsub(cu, uy);
-                    v = relaxed_pop(w19<float>(l), base, rho, cu, -cz);
-                    if (cx) v = vfma(vsplat(6.f * cx * w19<float>(l)), vmul(rho, vsplat(cz > 0 ? C.wall_u[0] : C.wall_u[1])), v);
+                    v = relaxed_pop(base, rho, cu, -cz);
+                    if (cx) v = vfma(vsplat(6.f * cx), vmul(rho, vsplat(cz > 0 ? C.wall_u[0] : C.wall_u[1])), v);
+                    v = vmul(vsplat(w19<float>(l)), v);
                 }
-                f[l * C.plane + i] = v.x;
-                if (NS == 2) f[(19 + l) * C.plane + i] = v.y;
+                if constexpr (sizeof(O) == 4) {
+                    f[l * C.plane + i] = v.x;
+                    if (NS == 2) f[(19 + l) * C.plane + i] = v.y;
+                } else {
+                    const long long n = (long long)C.nx * C.ny * C.nz, q = ((long long)z * C.ny + y) * C.nx + x;
+                    f[l * n + q] = lbm::widen_fx(v.x) + w19<double>(l) * (double)C.rho_ref[0];
+                    if (NS == 2) f[(19 + l) * n + q] = lbm::widen_fx(v.y) + w19<double>(l) * (double)C.rho_ref[1];
+                }
             }
         }
 }
@@ -1016,11 +1062,11 @@ __global__ void __launch_bounds__(128) k3_expand(const Mom3 M, int dc, float* __
 // 2 CTAs at 110 registers without spills -- the kernel waits on memory and more warps hide it.
 template <typename T, int MODE, int NS, int TY, int TZ>
 __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
-                                  Tile3<T>::TX* TY* TZ > 256 ? (MODE == K3_RELAX ? 2 : 1)
-                                                             : (sizeof(T) == 4 ? (MODE == K3_RELAX ? 4 : 3)
+                                  Tile3<T>::TX* TY* TZ > 256 ? (MODE >= K3_RELAX ? 2 : 1)
+                                                             : (sizeof(T) == 4 ? (MODE >= K3_RELAX ? 4 : 3)
                                                                                : 512 / (Tile3<T>::TX * TY * TZ)))
     k3_step(const __grid_constant__ CUtensorMap vmap, const T* __restrict__ fin, T* __restrict__ fout,
-            const Step3<T> C, int* __restrict__ flag, double* __restrict__ fields, const Mom3 M, int dn) {
+            const Step3<T> C, int* __restrict__ flag, const Fields3 fields, const Mom3 M, int dn) {
     constexpr int TX = Tile3<T>::TX;
     extern __shared__ __align__(1024) unsigned char smem3[];
     Smem3<T, TY, TZ>& S = *reinterpret_cast<Smem3<T, TY, TZ>*>(smem3);
@@ -1047,11 +1093,11 @@ __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
     const long long i = ((long long)z * C.ny + y) * C.pitch + x;
     // (FP64, short of registers, loads them after the force: its other warps cover the wait)
     // K3_RELAX: the streamed-in density and momentum instead
-    T f[MODE == K3_RELAX ? 1 : NS][19];
+    T f[MODE >= K3_RELAX ? 1 : NS][19];
     float jx = 0.f, jy = 0.f, jz = 0.f;
     float2 d = make_float2(0.f, 0.f);
     const auto load = [&]() {
-        if constexpr (MODE == K3_RELAX) {
+        if constexpr (MODE >= K3_RELAX) {
             d = (dn ? M.d[1] : M.d[0])[i];
             jx = M.jx[i];
             jy = M.jy[i];
@@ -1110,7 +1156,9 @@ __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
         C, [&](int dx, int dy, int dz) { return S.box[0][bz + dz][by + dy][bx + dx]; },
         [&](int dx, int dy, int dz) { return S.box[1][bz + dz][by + dy][bx + dx]; }, F);
     if (sizeof(T) == 8) load();
-    if constexpr (MODE == K3_RELAX)
+    if constexpr (MODE == K3_LOOK)
+        look3<NS>(C, F, S.box[1][bz][by][bx], ((long long)z * C.ny + y) * C.nx + x, jx, jy, jz, fields);
+    else if constexpr (MODE == K3_RELAX)
         relax3<NS>(C, M, F, S.box[1][bz][by][bx], i, jx, jy, jz, d, flag);
     else
         site3<T, NS, MODE>(C, f, F, x, y, z, i, fout, flag, fields);
@@ -1132,7 +1180,7 @@ __global__ void k3_init(T* __restrict__ f, const double* __restrict__ rho, const
 }
 
 template <typename T, int MODE, int NS, int TY, int TZ>
-cudaError_t launch_step3(const CUtensorMap& map, const T* fin, T* fout, const Step3<T>& C, int* flag, double* fields,
+cudaError_t launch_step3(const CUtensorMap& map, const T* fin, T* fout, const Step3<T>& C, int* flag, const Fields3& fields,
                          const Mom3& M, int dn, cudaStream_t st) {
     const size_t smem = sizeof(Smem3<T, TY, TZ>);
     static bool attr = false;  // per template instance
@@ -1150,7 +1198,7 @@ cudaError_t launch_step3(const CUtensorMap& map, const T* fin, T* fout, const St
 
 template <typename T, int MODE, int NS>
 cudaError_t launch_shape(int shape, const CUtensorMap& map, const T* fin, T* fout, const Step3<T>& C, int* flag,
-                         double* fields, const Mom3& M, int dn, cudaStream_t st) {
+                         const Fields3& fields, const Mom3& M, int dn, cudaStream_t st) {
     switch (shape) {
         case 0: return launch_step3<T, MODE, NS, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st);
         case 1: return launch_step3<T, MODE, NS, Tile3<T>::ty(1), Tile3<T>::tz(1)>(map, fin, fout, C, flag, fields, M, dn, st);
@@ -1163,11 +1211,14 @@ cudaError_t launch_shape(int shape, const CUtensorMap& map, const T* fin, T* fou
 // the step pass in the chosen tile shape; the fields pass (lbm3_get_fields) in shape 0
 template <typename T>
 cudaError_t launch_step3_any(int mode, int ns, int shape, const CUtensorMap& map, const T* fin, T* fout,
-                             const Step3<T>& C, int* flag, double* fields, const Mom3& M, int dn, cudaStream_t st) {
+                             const Step3<T>& C, int* flag, const Fields3& fields, const Mom3& M, int dn, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
         if (mode == K3_RELAX)
             return ns == 2 ? launch_shape<T, K3_RELAX, 2>(shape, map, fin, fout, C, flag, fields, M, dn, st)
                            : launch_shape<T, K3_RELAX, 1>(shape, map, fin, fout, C, flag, fields, M, dn, st);
+        if (mode == K3_LOOK)
+            return ns == 2 ? launch_step3<T, K3_LOOK, 2, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st)
+                           : launch_step3<T, K3_LOOK, 1, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st);
     }
     if (mode == K3_WRITE)
         return ns == 2 ? launch_shape<T, K3_WRITE, 2>(shape, map, fin, fout, C, flag, fields, M, dn, st)
@@ -1201,7 +1252,7 @@ struct lbm3_ctx {
     // stale; mom: that is so now; dc: which copy of the densities is current; chunk: k3_stream's
     bool mom = false;
     int dc = 0;
-    int chunk = 8;
+    int chunk = 1;
     int* flag = nullptr;
     double* staging = nullptr;         // lbm3_get_fields / lbm3_set_fields from the host
     size_t staging_bytes = 0;
@@ -1409,9 +1460,16 @@ extern "C" int lbm3_create(lbm3_ctx** out, const lbm3_desc* d) {
         c->tot_grid[2] = gz;
         c->nblk_den = gx * gy * gz;
     }
-    // k3_stream: chunks of 8 layers while they fill the GPU, shorter ones on small lattices
-    while (c->chunk > 1 && (long long)((nx + 31) / 32) * ((ny + 3) / 4) * ((nz + c->chunk - 1) / c->chunk) < 4LL * nsm)
-        c->chunk /= 2;
+    // k3_stream: a block reads chunk + 2 layers, 4 blocks run on an SM: the chunk whose waves of
+    // blocks read the fewest layers one after the other
+    {
+        const long long columns = (long long)((nx + 31) / 32) * ((ny + 3) / 4), slots = 4LL * nsm;
+        long long best = -1;
+        for (int k = 1; k <= 64; ++k) {
+            const long long blocks = columns * ((nz + k - 1) / k), cost = (blocks + slots - 1) / slots * (k + 2);
+            if (best < 0 || cost < best) best = cost, c->chunk = k;
+        }
+    }
     const dim3 sg = stream_grid3(c);
     const size_t parts = std::max<size_t>(c->nblk_den, (size_t)sg.x * sg.y * sg.z);
     CKC3(cudaMalloc(&c->part, parts * 5 * sizeof(double)));
@@ -1437,7 +1495,7 @@ extern "C" void lbm3_destroy(lbm3_ctx* c) {
 
 extern "C" const char* lbm3_last_error(const lbm3_ctx* c) { return c ? c->err.c_str() : g3_create_error.c_str(); }
 
-static cudaError_t expand3(lbm3_ctx* c);
+static cudaError_t expand3(lbm3_ctx* c, double* out = nullptr);
 
 extern "C" int lbm3_set_params(lbm3_ctx* c, const lbm_params* p) {
     if (!c) return LBM_EINVAL;
@@ -1541,14 +1599,23 @@ static dim3 stream_grid3(const lbm3_ctx* c) {
     return dim3((c->d.nx + 31) / 32, (c->d.ny + 3) / 4, (c->d.nz + c->chunk - 1) / c->chunk);
 }
 
-// The populations of the state held as moments into f[cur]; the state stays what it is.
-static cudaError_t expand3(lbm3_ctx* c) {
+// The populations of the state held as moments into f[cur], or (out) as plain values into the caller's
+// device memory; the state stays what it is.
+static cudaError_t expand3(lbm3_ctx* c, double* out) {
     const dim3 grid((c->d.nx + 127) / 128, c->d.ny, c->d.nz);
     const Mom3 M = moments3(c);
-    if (c->d.n_species == 2)
-        k3_expand<2><<<grid, 128, 0, c->stream>>>(M, c->dc, (float*)c->f[c->cur], c->c32);
-    else
-        k3_expand<1><<<grid, 128, 0, c->stream>>>(M, c->dc, (float*)c->f[c->cur], c->c32);
+    float* const f = (float*)c->f[c->cur];
+    if (c->d.n_species == 2) {
+        if (out)
+            k3_expand<2, double><<<grid, 128, 0, c->stream>>>(M, c->dc, out, c->c32);
+        else
+            k3_expand<2, float><<<grid, 128, 0, c->stream>>>(M, c->dc, f, c->c32);
+    } else {
+        if (out)
+            k3_expand<1, double><<<grid, 128, 0, c->stream>>>(M, c->dc, out, c->c32);
+        else
+            k3_expand<1, float><<<grid, 128, 0, c->stream>>>(M, c->dc, f, c->c32);
+    }
     return cudaGetLastError();
 }
 
@@ -1602,13 +1669,13 @@ static cudaError_t density3(lbm3_ctx* c, double* totals = nullptr, bool read = f
     const double n = (double)c->n;
     const double r0 = c->d.precision == LBM_FP64 ? 0.0 : (double)c->c32.rho_ref[0];
     const double r1 = c->d.precision == LBM_FP64 ? 0.0 : (double)c->c32.rho_ref[1];
-    lbm3::k3_totals_sum<<<1, 256, 0, c->stream>>>(c->part, nblk, n * r0, n * r1, totals);
-    return cudaGetLastError();
+    return launch_pdl(lbm3::k3_totals_sum, dim3(1), dim3(320), 0, c->stream, (const double*)c->part, nblk, n * r0, n * r1,
+                      totals);
 }
 
 // The collide pass of a step (K3_WRITE, after density3: it makes the new state the current one), or
 // K3_FIELDS.
-static cudaError_t collide3(lbm3_ctx* c, int mode, double* fields) {
+static cudaError_t collide3(lbm3_ctx* c, int mode, const Fields3& fields = Fields3{}) {
     const bool relax = mode == K3_WRITE && relaxed3(c);
     const int shape = mode == K3_WRITE ? c->shape : 0;
     const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(c->map[shape]);
@@ -1650,7 +1717,7 @@ static int one_step3(lbm3_ctx* c) {
         CK3(cudaEventRecord(e[1], c->stream));
         CK3(cudaEventRecord(e[2], c->stream));
     }
-    CK3(collide3(c, K3_WRITE, nullptr));
+    CK3(collide3(c, K3_WRITE));
     if (e) CK3(cudaEventRecord(e[3], c->stream));
     c->step += 1;
     return LBM_OK;
@@ -1693,7 +1760,7 @@ extern "C" int lbm3_step_totals(lbm3_ctx* c, int nsteps, double* dst, long long 
     // too (so the populations are read once per step for both); the first step needs its own
     for (int k = 0; k < nsteps; ++k) {
         if (k == 0) CK3(density3(c));
-        CK3(collide3(c, K3_WRITE, nullptr));
+        CK3(collide3(c, K3_WRITE));
         c->step += 1;
         CK3(density3(c, out + (long long)k * (stride / (long long)sizeof(double))));
     }
@@ -1729,6 +1796,16 @@ extern "C" int lbm3_synchronize(lbm3_ctx* c) {
     return LBM_OK;
 }
 
+// Whether a kernel may write doubles at p: null, or aligned device memory of the context's device.
+static bool writable3(const lbm3_ctx* c, const void* p) {
+    if (!p) return true;
+    cudaPointerAttributes a{};
+    const cudaError_t e = cudaPointerGetAttributes(&a, p);
+    cudaGetLastError();  // an unknown pointer may leave an error behind
+    return e == cudaSuccess && a.type == cudaMemoryTypeDevice && a.device == c->d.device &&
+           reinterpret_cast<size_t>(p) % sizeof(double) == 0;
+}
+
 extern "C" int lbm3_get_fields(lbm3_ctx* c, double* rho, double* u, double* f, int where) {
     if (!c) return LBM_EINVAL;
     if (where != LBM_HOST && where != LBM_DEVICE) return fail3(c, LBM_EINVAL, "where must be LBM_HOST or LBM_DEVICE");
@@ -1736,18 +1813,35 @@ extern "C" int lbm3_get_fields(lbm3_ctx* c, double* rho, double* u, double* f, i
     CK3(cudaSetDevice(c->d.device));
     const int ns = c->d.n_species;
     const long long n = c->n;
-    const size_t per = (size_t)(ns + 3 + 19 * ns);
-    int rc = staging3(c, per * n * sizeof(double));
-    if (rc) return rc;
-    if (c->mom) CK3(expand3(c));
-    CK3(density3(c, nullptr, true));
-    CK3(collide3(c, K3_FIELDS, c->staging));
-    const cudaMemcpyKind kind = where == LBM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-    if (rho) CK3(cudaMemcpyAsync(rho, c->staging, (size_t)ns * n * sizeof(double), kind, c->stream));
-    if (u) CK3(cudaMemcpyAsync(u, c->staging + (size_t)ns * n, (size_t)3 * n * sizeof(double), kind, c->stream));
-    if (f)
-        CK3(cudaMemcpyAsync(f, c->staging + (size_t)(ns + 3) * n, (size_t)19 * ns * n * sizeof(double), kind,
-                            c->stream));
+    // straight into the caller's device memory, or through the staging buffer (host memory, and
+    // pointers that a kernel may not write)
+    const size_t nrho = (size_t)ns * n, nu = (size_t)3 * n, nf = (size_t)19 * ns * n;
+    Fields3 at{rho, u, f};
+    const bool direct = where == LBM_DEVICE && writable3(c, rho) && writable3(c, u) && writable3(c, f);
+    if (!direct) {
+        const int rc = staging3(c, ((rho ? nrho : 0) + (u ? nu : 0) + (f ? nf : 0)) * sizeof(double));
+        if (rc) return rc;
+        double* p = c->staging;
+        if (rho) at.rho = p, p += nrho;
+        if (u) at.u = p, p += nu;
+        if (f) at.f = p;
+    }
+    if (c->mom) {  // held as moments: no populations but those asked for
+        if (at.f) CK3(expand3(c, at.f));
+        if (at.rho || at.u) {
+            CK3(density3(c));
+            CK3(collide3(c, K3_LOOK, at));
+        }
+    } else {
+        CK3(density3(c, nullptr, true));
+        CK3(collide3(c, K3_FIELDS, at));
+    }
+    if (!direct) {
+        const cudaMemcpyKind kind = where == LBM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+        if (rho) CK3(cudaMemcpyAsync(rho, at.rho, nrho * sizeof(double), kind, c->stream));
+        if (u) CK3(cudaMemcpyAsync(u, at.u, nu * sizeof(double), kind, c->stream));
+        if (f) CK3(cudaMemcpyAsync(f, at.f, nf * sizeof(double), kind, c->stream));
+    }
     return lbm3_synchronize(c);
 }
 
@@ -1818,11 +1912,11 @@ extern "C" int lbm3_autotune(lbm3_ctx* c, int steps, int* chosen, double* ms) {
     for (int k = 0; k < NSHAPE && e == cudaSuccess; ++k) {
         c->shape = k;
         e = density3(c);  // one untimed step (module load, caches)
-        if (e == cudaSuccess) e = collide3(c, K3_WRITE, nullptr);
+        if (e == cudaSuccess) e = collide3(c, K3_WRITE);
         if (e == cudaSuccess) e = cudaEventRecord(a, c->stream);
         for (int i = 0; i < steps && e == cudaSuccess; ++i) {
             e = density3(c);
-            if (e == cudaSuccess) e = collide3(c, K3_WRITE, nullptr);
+            if (e == cudaSuccess) e = collide3(c, K3_WRITE);
         }
         if (e == cudaSuccess) e = cudaEventRecord(b, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(b);
