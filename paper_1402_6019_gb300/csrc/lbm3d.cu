@@ -768,6 +768,15 @@ __device__ __forceinline__ void gain(Sum3& S, float2 g) {
     if constexpr (CZ != 0) S.z = add(S.z, (float)CZ);
 }
 
+constexpr int AHEAD = 2;
+__device__ __forceinline__ void prefetch5(const Mom3& M, const float2* D, long long k) {
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(M.base + k));
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(D + k));
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(M.ux + k));
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(M.uy + k));
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(M.uz + k));
+}
+
 // One site of a neighbouring column: what its populations need.
 struct Col3 {
     float2 base, rho, ux, uy, uz;
@@ -830,6 +839,13 @@ __global__ void __launch_bounds__(128, 4)
         const bool walls = C.zbc != 0;
         for (int zs = z0 - 1; zs <= z1; ++zs) {
             const bool in = zs >= 0 && zs < C.nz;
+            if (zs + AHEAD < min(z1 + 1, C.nz)) {  // the block's part of a later layer into L1, its halo by its edge threads
+                const long long o = lay * (zs + AHEAD);
+                const int k = r0 + x;
+                prefetch5(M, D, o + k);
+                if (threadIdx.y == 0) prefetch5(M, D, o + rm + x);
+                if (threadIdx.y == 3) prefetch5(M, D, o + rp + x);
+            }
             if (in || !walls) {
                 const long long o = lay * (in ? zs : (zs < 0 ? zs + C.nz : zs - C.nz));
                 const float2 *const pb = M.base + o, *const pd = D + o, *const px = M.ux + o, *const py = M.uy + o,
