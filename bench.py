@@ -258,7 +258,7 @@ def _traffic(kernel_src_hash, workload, precision, kernel):
 _CORE = ("lbm_core.cuh", "lbm_pair.cuh", "lbm_reduce.cuh")
 KERNEL_SOURCE = {"pull": ("lbm_pull.cu",) + _CORE, "fused": ("lbm_tile.cu",) + _CORE,
                  "twopass": ("lbm_twopass.cu",) + _CORE, "sweep": ("lbm_fused.cu",) + _CORE,
-                 "k3_step": ("lbm3d.cu",), "k3_density": ("lbm3d.cu",)}
+                 "k3_step": ("lbm3d.cu",), "k3_density": ("lbm3d.cu",), "k3_stream": ("lbm3d.cu",)}
 
 
 def kernel_source_hash(kernel):
@@ -570,10 +570,12 @@ def run_adjoint(a, w):
 
 
 # the 3-D step (D3Q19, two species): the method reads and writes each population once (304 B per
-# site-update in FP32); the collide pass k3_step itself reads the site's populations and the
-# psi / rho pairs and writes the pushed populations (152 + 16 + 152 = 320 B), the density pass
-# reads the populations and writes the pairs (168 B)
-BYTES3 = {"fp32": {"step": 304, "k3_step": 320, "k3_density": 168},
+# site-update in FP32).  FP64 moves populations: the collide pass k3_step reads the site's and the psi /
+# rho pairs and writes the pushed ones, the density pass reads them and writes the pairs.  FP32 at
+# tau = 1 (this workload) holds the state as moments: k3_stream reads the densities, base and
+# velocities (40 B) and writes the new densities, the momentum and the pairs (8 + 12 + 16 B), the
+# collide pass reads those (36 B) and writes base and velocities (32 B).
+BYTES3 = {"fp32": {"step": 304, "k3_step": 68, "k3_stream": 76},
           "fp64": {"step": 608, "k3_step": 640, "k3_density": 336}}
 
 
@@ -667,7 +669,8 @@ def run_3d(a, w):
     peak, peak_kind = _peaks()
     B = BYTES3[a.precision]
     kd, kc = d_ms / max(nstep, 1), c_ms / max(nstep, 1)
-    top, kms = ("k3_step", kc) if kc >= kd else ("k3_density", kd)
+    first = "k3_stream" if a.precision == "fp32" else "k3_density"
+    top, kms = ("k3_step", kc) if kc >= kd else (first, kd)
     achieved = B[top] * sites / (kms * 1e-3) / 1e9
     traffic = _traffic(kernel_source_hash(top), a.workload, a.precision, top)
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
@@ -676,7 +679,7 @@ def run_3d(a, w):
                 "peak_source": peak_kind,
                 "kernel": f"lbm3::{top}<T, ...>", "kernel_ms": round(kms, 5),
                 "algorithmic_bytes_per_site": B[top],
-                "kernels_ms": {"k3_density": round(kd, 5), "k3_step": round(kc, 5)},
+                "kernels_ms": {first: round(kd, 5), "k3_step": round(kc, 5)},
                 "step_frac": round(B["step"] * value * 1e6 / 1e9 / peak, 4),
                 "step_bytes_per_site": B["step"],
                 "timing": "kernel durations from CUDA events around each kernel in a second pass over the same "
@@ -723,7 +726,8 @@ def run_3d(a, w):
         "vs_baseline": None, "dtype": "f32" if a.precision == "fp32" else "f64", "data": "synthetic",
         "config": {"workload": a.workload, "nx": nx, "ny": ny, "nz": nz, "n_species": ns, "precision": a.precision,
                    "lattice": "D3Q19", "parallelism": f"replicas{world}" if world > 1 else "single",
-                   "tile_shape": ["32x4x2", "32x2x4", "32x8x1", "32x4x4"][shape],
+                   "tile_shape": (["32x4x2", "32x2x4", "32x8x1", "32x4x4"] if a.precision == "fp32"
+                                  else ["16x8x1", "16x4x2", "16x2x4", "16x8x2"])[shape],
                    "autotune_ms_per_step": [round(t, 5) for t in tune_ms],
                    "l2": f"one lattice of {2 * 19 * ns * sites * (4 if a.precision == 'fp32' else 8) / 2**20:.0f} "
                          f"MiB of populations (both copies) > {L2_BYTES / 2**20:.0f} MiB L2; no flush"},
