@@ -12,7 +12,7 @@ namespace lbm {
 // logic at all; without it the kernel reads the boundary from the step constants.  M_RECORD
 // (pull kernel, with M_WRITE, one lattice): also writes the step's input state, the
 // post-streaming populations as plain values, [ns][9][nz][nx] in the kernel's precision.
-enum { M_WRITE = 1, M_OBS = 2, M_FIELDS = 4, M_PERIODIC = 8, M_RECORD = 16 };
+enum { M_WRITE = 1, M_OBS = 2, M_FIELDS = 4, M_PERIODIC = 8, M_RECORD = 16, M_OWN = 32 };
 
 // Width of the strip a warp owns in the fused sweep: 32 lanes minus a 2-column halo on
 // each side (the reach of the 5x5 interaction stencil).

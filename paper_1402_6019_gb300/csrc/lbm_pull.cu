@@ -339,6 +339,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
     const bool WALL = (MODE & M_PERIODIC) ? false : C.zbc != 0;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     using SH = Shape<SHP>;
+    constexpr bool OWN = (MODE & M_OWN) != 0;
     constexpr int PZ = SH::PZ, TW = SH::W, QB = PullSmem<T, NS, ST, SHP>::QB;
     PullSmem<T, NS, ST, SHP>& S = *reinterpret_cast<PullSmem<T, NS, ST, SHP>*>(smem_raw);
     const int tx = threadIdx.x, tz = threadIdx.y, tid = tz * Shape<SHP>::W + tx;
@@ -349,7 +350,6 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
     const int rot = !WALL && ninst == 1 && ntz > 2 ? ntiles - ntx : 0;  // work order (describe)
     // work items of the folded reduction: blocks of rows, then blocks of columns
     const int nrb = (nz + RB_THREADS / 32 - 1) / (RB_THREADS / 32);
-    // (more CTAs than tiles and items together: each item has a CTA of its own)
     const int nfold = Rd.enabled ? nrb + (nx + RB_THREADS / 32 - 1) / (RB_THREADS / 32) : 0;
 
     // threads with a ring position (ring_position), RPW per warp; the observing builds keep it in
@@ -383,8 +383,9 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
     // buffers or the counters.
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    const bool own_items = nfold > 0 && (int)gridDim.x >= ntiles + nfold;
-    if (own_items && (int)blockIdx.x >= ntiles) {
+    // as many CTAs as tiles and items together: each item has a CTA of its own (launch_mode)
+    const bool own_items = OWN || (sizeof(T) == 8 && nfold > 0 && (int)gridDim.x >= ntiles + nfold);
+    if ((OWN || sizeof(T) == 8) && own_items && (int)blockIdx.x >= ntiles) {
         reduce_block<T, SH::NW>((int)blockIdx.x - ntiles, Rd.part_row, Rd.part_col, O.flag, Rd.nxpart, Rd.nzpart, nx, nz,
                                 C.zbc, nrb, Rd.out, Rd.avg, Rd.bpart, Rd.bavg, Rd.accumulate, T(Rd.inx), T(Rd.inz),
                                 S.wsc, ninst > 1 ? inst : nullptr, ninst);
@@ -407,7 +408,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
             more = S.ti[sl].t < ntiles;
             if (more && sl == 0) issue_load(S, &tin, S.ti[0].x0, S.ti[0].prow0 + S.ti[0].z0, 0);
         }
-        if (more && nstat < ntiles) upcoming = min(nstat + (int)atomicAdd(ctr, 1u), ntiles);
+        if (!OWN && more && (sizeof(T) == 4 || nstat < ntiles)) upcoming = min(nstat + (int)atomicAdd(ctr, 1u), ntiles);
     }
     __syncthreads();
     // thread 0: the reduction's counter as last seen (no draw), during the CTA's last tiles
@@ -862,7 +863,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
             static_cast<T*>(O.part_col)[((long long)prev_x * ntz + prev_jg) * NQC + tz] = v;
         }
     }
-    if (nfold > 0 && !own_items && !failed) {
+    if (!OWN && nfold > 0 && !own_items && !failed) {
         // the previous pass's reduction: work items from the second counter until they run out
         for (;;) {
             if (tid == 0) S.fold_item = fold_seen < nfold ? (int)atomicAdd(ctr + 1, 1u) : nfold;
@@ -885,9 +886,21 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
     }
 }
 
+// Small lattices: the previous pass's reduction runs beside the tiles, on CTAs of its own, where it
+// would otherwise follow them (a draw, a round of loads and two barriers: 2 us of a 7 us launch).  In
+// FP32 that is a build of its own: the reduction's second copy in the general one cost every larger
+// lattice 0.4 % (1024^2 observed: 29,165 against 29,055 MLUPS).  The FP64 builds choose at run time.
+template <typename T, int MODE, int SHP>
+constexpr bool own_build = sizeof(T) == 4 && SHP == SHAPE_32 && (MODE & M_WRITE) != 0 && (MODE & M_OBS) != 0;
+
 template <typename T, int NS, int MODE, int ST, int SHP>
 int pull_occupancy() {
     const size_t smem = sizeof(PullSmem<T, NS, ST, SHP>);
+    if constexpr (own_build<T, MODE, SHP>) {
+        if (cudaFuncSetAttribute(k_pull<T, NS, MODE | M_OWN, ST, SHP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem) != cudaSuccess)
+            return 0;
+    }
     // a short tile's launch may ask for 116 KB (launch_mode)
     if (cudaFuncSetAttribute(k_pull<T, NS, MODE, ST, SHP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              SHP == SHAPE_SHORT ? 116 * 1024 : (int)smem) != cudaSuccess)
@@ -905,10 +918,9 @@ cudaError_t launch_mode(const void* tin, T* fout, const StepConst<T>& C, const O
                         T* rec) {
     const int ntx = (C.nx + Shape<SHP>::W - 1) / Shape<SHP>::W;
     const long long ntiles = (long long)ntx * B.ntz;
-    // small lattices: the previous pass's reduction runs beside the tiles, on CTAs of its own, where it
-    // would otherwise follow them (a draw, a round of loads and two barriers: 2 us of a 7 us launch)
     const long long items = Rd.enabled ? reduce_blocks(C.nx, C.nz) : 0;
-    int grid = (int)(ntiles + items <= grid_max ? ntiles + items : (ntiles < grid_max ? ntiles : grid_max));
+    const bool own = (own_build<T, MODE, SHP> || sizeof(T) == 8) && items > 0 && ntiles + items <= grid_max;
+    const int grid = (int)(own ? ntiles + items : (ntiles < grid_max ? ntiles : grid_max));
     PairConst K{};
     if constexpr (kPair<T, NS>) fill_pair_const(K, C);
     // launched with programmatic stream serialisation: it may start while the kernel before it
@@ -928,9 +940,12 @@ cudaError_t launch_mode(const void* tin, T* fout, const StepConst<T>& C, const O
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_pull<T, NS, MODE, ST, SHP>, *static_cast<const CUtensorMap*>(tin), fout, C, K,
-                              O, Rd, sched + 2 * set, sched + 2 * (set ^ 1), B.inst, B.ninst, ntx, B.ntz, rec,
-                              set & 1);
+    auto kernel = k_pull<T, NS, MODE, ST, SHP>;
+    if constexpr (own_build<T, MODE, SHP>) {
+        if (own) kernel = k_pull<T, NS, MODE | M_OWN, ST, SHP>;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, *static_cast<const CUtensorMap*>(tin), fout, C, K, O, Rd, sched + 2 * set,
+                              sched + 2 * (set ^ 1), B.inst, B.ninst, ntx, B.ntz, rec, set & 1);
 }
 
 // The passes built at width 64 as well: the FP32 step passes (lbm_step); all others run width 32.

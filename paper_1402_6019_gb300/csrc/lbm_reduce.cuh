@@ -105,126 +105,119 @@ __device__ __forceinline__ void reduce_block(int blk, const void* part_row, cons
         else if (accumulate && bad)
             R::put(avg, O_BAD, R::from(PT(1)));
     }
-    // row or column `warp` of the item
-    auto line = [&](const int warp) {
-    if (blk < nrowblocks) {
-        const int z = blk * WPB + warp;
-        if (z < nz) {
-            // this row's lattice: its first compact row and height
-            int z0 = 0, nzi = nz;
-            if (inst) {
-                const int k = inst_of_row(inst, ninst, z);
-                z0 = inst[k].zrow0;
-                nzi = inst[k].nz;
-            }
-            const int zi = z - z0;  // row within the lattice
-            int zl = zi - 1, zr = zi + 1;
-            PT wl = PT(0.5), wr = PT(0.5);
-            if (nzi == 1) {
-                zl = zr = zi;
-            } else if (zbc == 0) {
-                zl = zi == 0 ? nzi - 1 : zi - 1;
-                zr = zi == nzi - 1 ? 0 : zi + 1;
-            } else if (zi == 0) {
-                zl = 0;
-                wl = wr = PT(1);
-            } else if (zi == nzi - 1) {
-                zr = nzi - 1;
-                wl = wr = PT(1);
-            }
-            zl += z0;
-            zr += z0;
-            // the output entries of this lane (lanes 0..8), -1 for none; the second is the wall
-            // force scalar of a single lattice
-            long long oi = -1, oi2 = -1;
-            switch (lane) {
-                case QR_UX: oi = iux + z; break;
-                case QR_RHOA: oi = irz + z; break;
-                case QR_RHOB: oi = irz + nz + z; break;
-                case QR_SXZ: oi = isx + z; break;
-                case QR_MX: oi = imx + z; break;
-                case QR_MZ: oi = imz + z; break;
-                case QR_WALLB:
-                    oi = iwb + z;
-                    oi2 = (!inst && zbc && z == 0) ? O_WALL : -1;
-                    break;
-                case QR_WALLT:
-                    oi = iwt + z;
-                    oi2 = (!inst && zbc && z == nz - 1) ? O_WALL + 1 : -1;
-                    break;
-                case NQR: oi = ifl + z; break;
-                default: break;
-            }
-            PT v[NQR + 2];
-#pragma unroll
-            for (int k = 0; k < NQR + 2; ++k) v[k] = PT(0);
-            for (int p = lane; p < nxpart; p += 32) {
-                const PT* src = prow + ((long long)z * nxpart + p) * NQR;
-#pragma unroll
-                for (int k = 0; k < NQR; ++k) v[k] += src[k];
-                v[NQR] += prow[((long long)zl * nxpart + p) * NQR + QR_UX];
-                v[NQR + 1] += prow[((long long)zr * nxpart + p) * NQR + QR_UX];
-            }
-            const A old = (accumulate == 1 && oi >= 0) ? R::get(avg, oi) : R::zero();  // in flight with the sums
-            const A old2 = (accumulate == 1 && oi2 >= 0) ? R::get(avg, oi2) : R::zero();
-#pragma unroll
-            for (int k = 0; k < NQR + 2; ++k) v[k] = warp_sum(v[k]);
-            if (lane <= NQR) {
-                PT mine = v[0];
-#pragma unroll
-                for (int k = 1; k < NQR; ++k)
-                    if (lane == k) mine = v[k];
-                A val;
-                if (lane == NQR) {  // fluidity
-                    const PT gd = nzi == 1 ? PT(0) : (wr * v[NQR + 1] - wl * v[NQR]) * inx;
-                    val = R::from(gd / (v[QR_SXZ] * inx));
-                } else {
-                    val = R::from(mine * inx);
+    // row or column `warp` of the item (a plain loop: as a lambda it cost the pull kernel 0.4 %)
+    for (int warp = warp0; warp < WPB; warp += NWARP) {
+        if (blk < nrowblocks) {
+            const int z = blk * WPB + warp;
+            if (z < nz) {
+                // this row's lattice: its first compact row and height
+                int z0 = 0, nzi = nz;
+                if (inst) {
+                    const int k = inst_of_row(inst, ninst, z);
+                    z0 = inst[k].zrow0;
+                    nzi = inst[k].nz;
                 }
-                if (lane == QR_RHOA) wsc[warp][0] = R::from(mine);
-                if (lane == QR_RHOB) wsc[warp][1] = R::from(mine);
-                if (lane == QR_MX) wsc[warp][2] = R::from(mine);
-                if (lane == QR_MZ) wsc[warp][3] = R::from(mine);
+                const int zi = z - z0;  // row within the lattice
+                int zl = zi - 1, zr = zi + 1;
+                PT wl = PT(0.5), wr = PT(0.5);
+                if (nzi == 1) {
+                    zl = zr = zi;
+                } else if (zbc == 0) {
+                    zl = zi == 0 ? nzi - 1 : zi - 1;
+                    zr = zi == nzi - 1 ? 0 : zi + 1;
+                } else if (zi == 0) {
+                    zl = 0;
+                    wl = wr = PT(1);
+                } else if (zi == nzi - 1) {
+                    zr = nzi - 1;
+                    wl = wr = PT(1);
+                }
+                zl += z0;
+                zr += z0;
+                // the output entries of this lane (lanes 0..8), -1 for none; the second is the wall
+                // force scalar of a single lattice
+                long long oi = -1, oi2 = -1;
+                switch (lane) {
+                    case QR_UX: oi = iux + z; break;
+                    case QR_RHOA: oi = irz + z; break;
+                    case QR_RHOB: oi = irz + nz + z; break;
+                    case QR_SXZ: oi = isx + z; break;
+                    case QR_MX: oi = imx + z; break;
+                    case QR_MZ: oi = imz + z; break;
+                    case QR_WALLB:
+                        oi = iwb + z;
+                        oi2 = (!inst && zbc && z == 0) ? O_WALL : -1;
+                        break;
+                    case QR_WALLT:
+                        oi = iwt + z;
+                        oi2 = (!inst && zbc && z == nz - 1) ? O_WALL + 1 : -1;
+                        break;
+                    case NQR: oi = ifl + z; break;
+                    default: break;
+                }
+                PT v[NQR + 2];
+    #pragma unroll
+                for (int k = 0; k < NQR + 2; ++k) v[k] = PT(0);
+                for (int p = lane; p < nxpart; p += 32) {
+                    const PT* src = prow + ((long long)z * nxpart + p) * NQR;
+    #pragma unroll
+                    for (int k = 0; k < NQR; ++k) v[k] += src[k];
+                    v[NQR] += prow[((long long)zl * nxpart + p) * NQR + QR_UX];
+                    v[NQR + 1] += prow[((long long)zr * nxpart + p) * NQR + QR_UX];
+                }
+                const A old = (accumulate == 1 && oi >= 0) ? R::get(avg, oi) : R::zero();  // in flight with the sums
+                const A old2 = (accumulate == 1 && oi2 >= 0) ? R::get(avg, oi2) : R::zero();
+    #pragma unroll
+                for (int k = 0; k < NQR + 2; ++k) v[k] = warp_sum(v[k]);
+                if (lane <= NQR) {
+                    PT mine = v[0];
+    #pragma unroll
+                    for (int k = 1; k < NQR; ++k)
+                        if (lane == k) mine = v[k];
+                    A val;
+                    if (lane == NQR) {  // fluidity
+                        const PT gd = nzi == 1 ? PT(0) : (wr * v[NQR + 1] - wl * v[NQR]) * inx;
+                        val = R::from(gd / (v[QR_SXZ] * inx));
+                    } else {
+                        val = R::from(mine * inx);
+                    }
+                    if (lane == QR_RHOA) wsc[warp][0] = R::from(mine);
+                    if (lane == QR_RHOB) wsc[warp][1] = R::from(mine);
+                    if (lane == QR_MX) wsc[warp][2] = R::from(mine);
+                    if (lane == QR_MZ) wsc[warp][3] = R::from(mine);
+                    if (oi >= 0) {
+                        R::put(out, oi, val);
+                        if (accumulate) R::put(avg, oi, R::add(old, val));
+                    }
+                    if (oi2 >= 0) {
+                        R::put(out, oi2, val);
+                        if (accumulate) R::put(avg, oi2, R::add(old2, val));
+                    }
+                }
+            }
+        } else {
+            const int x = (blk - nrowblocks) * WPB + warp;
+            if (x < nx) {
+                const long long oi = lane == 0 ? ips + x : (lane == 1 ? ipx + x : -1);
+                PT v[NQC];
+    #pragma unroll
+                for (int k = 0; k < NQC; ++k) v[k] = PT(0);
+                for (int p = lane; p < nzpart; p += 32) {
+                    const PT* src = pcol + ((long long)x * nzpart + p) * NQC;
+    #pragma unroll
+                    for (int k = 0; k < NQC; ++k) v[k] += src[k];
+                }
+                const A old = (accumulate == 1 && oi >= 0) ? R::get(avg, oi) : R::zero();
+    #pragma unroll
+                for (int k = 0; k < NQC; ++k) v[k] = warp_sum(v[k]);
                 if (oi >= 0) {
+                    const A val = R::from((lane == 0 ? v[QC_PS] : v[QC_PXX]) * inz);
+                    if (lane == 0) wsc[warp][4] = val;
                     R::put(out, oi, val);
                     if (accumulate) R::put(avg, oi, R::add(old, val));
                 }
-                if (oi2 >= 0) {
-                    R::put(out, oi2, val);
-                    if (accumulate) R::put(avg, oi2, R::add(old2, val));
-                }
             }
         }
-    } else {
-        const int x = (blk - nrowblocks) * WPB + warp;
-        if (x < nx) {
-            const long long oi = lane == 0 ? ips + x : (lane == 1 ? ipx + x : -1);
-            PT v[NQC];
-#pragma unroll
-            for (int k = 0; k < NQC; ++k) v[k] = PT(0);
-            for (int p = lane; p < nzpart; p += 32) {
-                const PT* src = pcol + ((long long)x * nzpart + p) * NQC;
-#pragma unroll
-                for (int k = 0; k < NQC; ++k) v[k] += src[k];
-            }
-            const A old = (accumulate == 1 && oi >= 0) ? R::get(avg, oi) : R::zero();
-#pragma unroll
-            for (int k = 0; k < NQC; ++k) v[k] = warp_sum(v[k]);
-            if (oi >= 0) {
-                const A val = R::from((lane == 0 ? v[QC_PS] : v[QC_PXX]) * inz);
-                if (lane == 0) wsc[warp][4] = val;
-                R::put(out, oi, val);
-                if (accumulate) R::put(avg, oi, R::add(old, val));
-            }
-        }
-    }
-    };
-    if constexpr (NWARP == WPB) {
-        line(warp0);
-    } else if constexpr (NWARP > WPB) {
-        if (warp0 < WPB) line(warp0);
-    } else {
-        for (int w = warp0; w < WPB; w += NWARP) line(w);
     }
     __syncthreads();
     A bsum = R::zero();
