@@ -38,10 +38,10 @@ sys.path.insert(0, ROOT)
 
 BYTES_PER_SITE = {("fp32", 2): 144, ("fp64", 2): 288, ("fp32", 1): 72, ("fp64", 1): 144}
 # The FP64 step (two species, observables every step) is bound by the FP64 pipe: FP64 flops per
-# site-update counted by ncu (242 DFMA, 244 DADD, 119 DMUL; profiles/k_pull_emulsion_1024_fp64.md)
-# against 2 DFMA per SM per cycle x 152 SMs x 2 flops x 2.07 GHz
-FP64_FLOPS_PER_SITE = 847
-FP64_INSTR_PER_SITE = 605  # the same counts as instructions: each occupies the FP64 pipe once
+# site-update counted by ncu (96 DFMA, 121 DADD, 70 DMUL; psi and its sums run on the integer pipes;
+# profiles/k_pull_emulsion_1024_fp64.md) against 2 DFMA per SM per cycle x 152 SMs x 2 flops x 2.07 GHz
+FP64_FLOPS_PER_SITE = 383
+FP64_INSTR_PER_SITE = 287  # the same counts as instructions: each occupies the FP64 pipe once
 FP64_PEAK_TFLOPS = 304 * 2 * 2.07e9 / 1e12
 L2_FLUSH_BYTES = 256 << 20
 L2_BYTES = 126 << 20          # L2 of a GB300 (nvidia-smi / device properties: 126.5 MiB)
@@ -255,10 +255,10 @@ def _traffic(kernel_src_hash, workload, precision, kernel):
     return e.get("dram_bytes_per_launch")
 
 
-_CORE = ("lbm_core.cuh", "lbm_pair.cuh", "lbm_reduce.cuh")
+_CORE = ("lbm_core.cuh", "lbm_fixed.cuh", "lbm_pair.cuh", "lbm_reduce.cuh")
 KERNEL_SOURCE = {"pull": ("lbm_pull.cu",) + _CORE, "fused": ("lbm_tile.cu",) + _CORE,
                  "twopass": ("lbm_twopass.cu",) + _CORE, "sweep": ("lbm_fused.cu",) + _CORE,
-                 "k3_step": ("lbm3d.cu",), "k3_density": ("lbm3d.cu",), "k3_stream": ("lbm3d.cu",)}
+                 **dict.fromkeys(("k3_step", "k3_density", "k3_stream"), ("lbm3d.cu", "lbm_fixed.cuh"))}
 
 
 def kernel_source_hash(kernel):

@@ -25,7 +25,7 @@
 //  * k3_stream evaluates, at every site, the 19 equilibria that stream in from the neighbours'
 //    moments, and writes their density and momentum (and the psi / rho volumes);
 //  * k3_step in its K3_RELAX form takes the force from the volumes and writes the new density and velocity.
-// About 170 B per site-update, and half the instructions.  Populations are formed where they are asked
+// 144 B per site-update, and half the instructions.  Populations are formed where they are asked
 // for (k3_expand).
 #include <cuda.h>
 #include <cudaTypedefs.h>
