@@ -982,14 +982,20 @@ __global__ void __launch_bounds__(128, 4)
     }
 }
 
+// Whether a density of the site is <= 0, NaN or Inf.
+template <int NS>
+__device__ __forceinline__ bool bad_density(float2 rho) {
+    bool bad = !(rho.x > 0.f) || !(rho.x < 1e30f);
+    if (NS == 2) bad = bad || !(rho.y > 0.f) || !(rho.y < 1e30f);
+    return bad;
+}
+
 // The site update of the relaxing pass (k3_step, K3_RELAX): from the force, the streamed-in density
 // and momentum, the species' velocities and base.
 template <int NS>
 __device__ __forceinline__ void relax3(const Step3<float>& C, const Mom3& M, const float (&F)[2][3], float2 rho,
                                        long long i, float jx, float jy, float jz, float2 d, int* __restrict__ flag) {
-    bool bad = !(rho.x > 0.f) || !(rho.x < 1e30f);
-    if (NS == 2) bad = bad || !(rho.y > 0.f) || !(rho.y < 1e30f);
-    if (bad) atomicOr(flag, 1);
+    if (bad_density<NS>(rho)) atomicOr(flag, 1);
     const float iden = 1.f / (NS == 2 ? sadd(rho.x, rho.y) : rho.x);
     const float2 ir = make_float2(1.f / rho.x, NS == 2 ? 1.f / rho.y : 0.f);
     const float2 fx = make_float2(sfma(rho.x, C.g, F[0][0]), NS == 2 ? sfma(rho.y, C.g, F[1][0]) : 0.f);
@@ -1004,10 +1010,12 @@ __device__ __forceinline__ void relax3(const Step3<float>& C, const Mom3& M, con
     M.uz[i] = uz;
 }
 
-// rho_s and the barycentric velocity (sum_s j_s + F_s / 2) / sum_s rho_s of a site (K3_LOOK).
+// rho_s and the barycentric velocity (sum_s j_s + F_s / 2) / sum_s rho_s of a site (K3_LOOK), and, as
+// every read of a state, the test of its densities.
 template <int NS>
 __device__ __forceinline__ void look3(const Step3<float>& C, const float (&F)[2][3], float2 rho, long long k, float jx,
-                                      float jy, float jz, const Fields3& out) {
+                                      float jy, float jz, int* __restrict__ flag, const Fields3& out) {
+    if (bad_density<NS>(rho)) atomicOr(flag, 1);
     const long long n = (long long)C.nx * C.ny * C.nz;
     const float irt = 1.f / (NS == 2 ? sadd(rho.x, rho.y) : rho.x);
     float fx = sfma(rho.x, C.g, F[0][0]), fy = F[0][1], fz = F[0][2];
@@ -1173,7 +1181,8 @@ __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
         [&](int dx, int dy, int dz) { return S.box[1][bz + dz][by + dy][bx + dx]; }, F);
     if (sizeof(T) == 8) load();
     if constexpr (MODE == K3_LOOK)
-        look3<NS>(C, F, S.box[1][bz][by][bx], ((long long)z * C.ny + y) * C.nx + x, jx, jy, jz, fields);
+        look3<NS>(C, F, S.box[1][bz][by][bx], ((long long)z * C.ny + y) * C.nx + x, jx, jy, jz, flag,
+                 fields);
     else if constexpr (MODE == K3_RELAX)
         relax3<NS>(C, M, F, S.box[1][bz][by][bx], i, jx, jy, jz, d, flag);
     else
@@ -1842,12 +1851,10 @@ extern "C" int lbm3_get_fields(lbm3_ctx* c, double* rho, double* u, double* f, i
         if (u) at.u = p, p += nu;
         if (f) at.f = p;
     }
-    if (c->mom) {  // held as moments: no populations but those asked for
+    if (c->mom) {  // held as moments: no populations but those asked for; the densities are always looked at
         if (at.f) CK3(expand3(c, at.f));
-        if (at.rho || at.u) {
-            CK3(density3(c));
-            CK3(collide3(c, K3_LOOK, at));
-        }
+        CK3(density3(c));
+        CK3(collide3(c, K3_LOOK, at));
     } else {
         CK3(density3(c, nullptr, true));
         CK3(collide3(c, K3_FIELDS, at));
