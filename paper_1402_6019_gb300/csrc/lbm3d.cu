@@ -252,9 +252,18 @@ __device__ __forceinline__ int ghost_list(int v, int n, int g, bool mirror, int*
     return k;
 }
 
+// A block of the density pass: 128 sites of a row; with the totals in FP32 32 columns of 4 rows, whose
+// threads a narrow lattice keeps busy too (step_totals of one species at 32 x 32 x 128: 673 us for 24
+// steps, 859 with rows of 128; at 128^3 2,527 and 2,550).  In FP64, bound by the FP64 pipe, the
+// smaller blocks share small lattices out more evenly (32^3: 1,927 us for 24 steps, 2,038 in 32 x 4).
+template <typename T, bool TOT>
+struct DensityBlock {
+    static constexpr int X = TOT && sizeof(T) == 4 ? 32 : 128, Y = 128 / X;
+};
+
 // The density pass: each site's sums over its 19 populations per species give rho_s and psi_s,
-// written with their ghost images into the two volumes.  One thread per site: x from the block
-// (128 sites of a row), y and z from the grid, looping when the grid is smaller than the lattice
+// written with their ghost images into the two volumes.  One thread per site: x and the row within
+// the block (DensityBlock), y and z from the grid, looping when the grid is smaller than the lattice
 // (the plain pass launches one block per row segment, so each loop runs once).  TOT: the block's
 // FP64 partials of the totals of the state go to part[block] as well -- the sums over its sites of
 // each species' density deviation sum_l f_l and of the lattice momentum: a site's sums (its two
@@ -270,11 +279,12 @@ __global__ void __launch_bounds__(128, TOT || MOM || sizeof(T) == 8 ? 8 : 16)
                float2* __restrict__ dn = nullptr, float* __restrict__ jt = nullptr) {
     using V = typename PairOf<T>::V;
     pdl_enter();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    using B = DensityBlock<T, TOT>;
+    const int x = blockIdx.x * B::X + threadIdx.x % B::X;
     double mass0 = 0.0, mass1 = 0.0, momx = 0.0, momy = 0.0, momz = 0.0;
     V* const P = reinterpret_cast<V*>(vol);
     for (int z = blockIdx.z; z < C.nz; z += gridDim.z)
-        for (int y = blockIdx.y; y < C.ny; y += gridDim.y) {
+        for (int y = blockIdx.y * B::Y + threadIdx.x / B::X; y < C.ny; y += gridDim.y * B::Y) {
             if (x >= C.nx) continue;
             const long long i = ((long long)z * C.ny + y) * C.pitch + x;
             T rho[2] = {T(0), T(0)}, psi[2] = {T(0), T(0)};
@@ -1472,13 +1482,18 @@ extern "C" int lbm3_create(lbm3_ctx** out, const lbm3_desc* d) {
     CKC3(cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
     int nsm = 0;
     CKC3(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, d->device));
-    {  // the density pass with totals: about 8 CTAs per SM, each looping over as many rows (not one
-       // over two and the next over one), or a CTA per row segment while there are few
-        const int gx = (nx + 127) / 128, target = (long long)gx * ny * nz <= 16 * nsm ? 16 * nsm : 8 * nsm;
-        int gy = std::max(1, std::min(ny, target / gx));
+    {  // the density pass with totals: no more than the 8 CTAs that run on an SM, each looping over as many
+       // rows (not one over two and the next over one); in FP64 also a CTA per row segment while those
+       // are at most 16 per SM (FP32 there, 48^3: 963 us for 24 steps, 861 looping)
+        const bool f32 = c->esize == 4;
+        const int bx = f32 ? DensityBlock<float, true>::X : DensityBlock<double, true>::X;
+        const int by = f32 ? DensityBlock<float, true>::Y : DensityBlock<double, true>::Y;
+        const int gx = (nx + bx - 1) / bx, rows = (ny + by - 1) / by;
+        const int target = !f32 && (long long)gx * rows * nz <= 16 * nsm ? 16 * nsm : 8 * nsm;
+        int gy = std::max(1, std::min(rows, target / gx));
         int gz = std::max(1, std::min(nz, target / (gx * gy)));
-        const int py = (ny + gy - 1) / gy, pz = (nz + gz - 1) / gz;
-        gy = (ny + py - 1) / py;
+        const int py = (rows + gy - 1) / gy, pz = (nz + gz - 1) / gz;
+        gy = (rows + py - 1) / py;
         gz = (nz + pz - 1) / pz;
         c->tot_grid[0] = gx;
         c->tot_grid[1] = gy;
