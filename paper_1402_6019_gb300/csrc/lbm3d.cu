@@ -19,7 +19,7 @@
 // (each population read and written once).  Populations are SoA f[s][l][z][y][x] (rows padded
 // to 32), FP32 deviations f - W_l rho_ref,s or plain FP64.
 //
-// Full relaxation (FP32, tau = 1 for every species) needs no populations: the collision leaves
+// Full relaxation (two species in FP32, tau = 1 for both; lbm3_create says which lattices) needs no populations: the collision leaves
 // f*_l = feq_l(rho_s, u_s), so the density and velocity after it (4 numbers per species, held as 5)
 // are the whole state, and a step only needs the density and momentum of what streams in.
 //  * k3_stream evaluates, at every site, the 19 equilibria that stream in from the neighbours'
@@ -739,7 +739,6 @@ __device__ __forceinline__ void site3(const Step3<T>& C, const T (&f)[NS][19], T
 //   f*_l - w_l rho_ref = w_l (base + rho c.u (3 + 9/2 c.u)).
 // d has two copies (k3_stream reads the neighbours' old one while it writes the new).  jt holds the
 // streamed-in lattice momentum, the species added (R5's common velocity needs no more at tau = 1).
-// With one species the B half is zero.
 struct Mom3 {
     float2* d[2];
     float2 *base, *ux, *uy, *uz;
@@ -822,7 +821,7 @@ __device__ __forceinline__ void wall_in(Sum3& S, const Col3& c, float uw) {
 // chunk.  With TOT the block's FP64 partials of the state's totals too (as k3_density's).
 // Bound by instruction issue and L1 (about 240 instructions and 300 B of reads per site) with the
 // whole state in L2 at 128^3.
-template <int NS, bool TOT>
+template <bool TOT>
 __global__ void __launch_bounds__(128, 4)
     k3_stream(const Mom3 M, int dc, float* __restrict__ vol, const Step3<float> C, int chunk, double* __restrict__ part) {
     pdl_enter();
@@ -949,10 +948,10 @@ __global__ void __launch_bounds__(128, 4)
                 M.jy[i] = jy;
                 M.jz[i] = jz;
                 const float2 rho = vadd(rref, dn);
-                float2 psi = make_float2(psi3(C, 0, rho.x), NS == 2 ? psi3(C, 1, rho.y) : 0.f);
+                const float2 psi = make_float2(psi3(C, 0, rho.x), psi3(C, 1, rho.y));
                 if constexpr (TOT) {
                     tot[0] += (double)dn.x;
-                    if (NS == 2) tot[1] += (double)dn.y;
+                    tot[1] += (double)dn.y;
                     tot[2] += (double)jx;
                     tot[3] += (double)jy;
                     tot[4] += (double)jz;
@@ -993,26 +992,21 @@ __global__ void __launch_bounds__(128, 4)
 }
 
 // Whether a density of the site is <= 0, NaN or Inf.
-template <int NS>
 __device__ __forceinline__ bool bad_density(float2 rho) {
-    bool bad = !(rho.x > 0.f) || !(rho.x < 1e30f);
-    if (NS == 2) bad = bad || !(rho.y > 0.f) || !(rho.y < 1e30f);
-    return bad;
+    return !(rho.x > 0.f) || !(rho.x < 1e30f) || !(rho.y > 0.f) || !(rho.y < 1e30f);
 }
 
 // The site update of the relaxing pass (k3_step, K3_RELAX): from the force, the streamed-in density
 // and momentum, the species' velocities and base.
-template <int NS>
 __device__ __forceinline__ void relax3(const Step3<float>& C, const Mom3& M, const float (&F)[2][3], float2 rho,
                                        long long i, float jx, float jy, float jz, float2 d, int* __restrict__ flag) {
-    if (bad_density<NS>(rho)) atomicOr(flag, 1);
-    const float iden = 1.f / (NS == 2 ? sadd(rho.x, rho.y) : rho.x);
-    const float2 ir = make_float2(1.f / rho.x, NS == 2 ? 1.f / rho.y : 0.f);
-    const float2 fx = make_float2(sfma(rho.x, C.g, F[0][0]), NS == 2 ? sfma(rho.y, C.g, F[1][0]) : 0.f);
-    const float2 fy = make_float2(F[0][1], NS == 2 ? F[1][1] : 0.f), fz = make_float2(F[0][2], NS == 2 ? F[1][2] : 0.f);
+    if (bad_density(rho)) atomicOr(flag, 1);
+    const float iden = 1.f / sadd(rho.x, rho.y);
+    const float2 ir = make_float2(1.f / rho.x, 1.f / rho.y);
+    const float2 fx = make_float2(sfma(rho.x, C.g, F[0][0]), sfma(rho.y, C.g, F[1][0]));
+    const float2 fy = make_float2(F[0][1], F[1][1]), fz = make_float2(F[0][2], F[1][2]);
     const float px = smul(jx, iden), py = smul(jy, iden), pz = smul(jz, iden);
-    float2 ux = vfma(fx, ir, vsplat(px)), uy = vfma(fy, ir, vsplat(py)), uz = vfma(fz, ir, vsplat(pz));
-    if (NS == 1) ux.y = uy.y = uz.y = 0.f;
+    const float2 ux = vfma(fx, ir, vsplat(px)), uy = vfma(fy, ir, vsplat(py)), uz = vfma(fz, ir, vsplat(pz));
     const float2 u15 = vmul(vsplat(1.5f), vfma(ux, ux, vfma(uy, uy, vmul(uz, uz))));
     M.base[i] = vsub(d, vmul(rho, u15));
     M.ux[i] = ux;
@@ -1022,17 +1016,16 @@ __device__ __forceinline__ void relax3(const Step3<float>& C, const Mom3& M, con
 
 // rho_s and the barycentric velocity (sum_s j_s + F_s / 2) / sum_s rho_s of a site (K3_LOOK), and, as
 // every read of a state, the test of its densities.
-template <int NS>
 __device__ __forceinline__ void look3(const Step3<float>& C, const float (&F)[2][3], float2 rho, long long k, float jx,
                                       float jy, float jz, int* __restrict__ flag, const Fields3& out) {
-    if (bad_density<NS>(rho)) atomicOr(flag, 1);
+    if (bad_density(rho)) atomicOr(flag, 1);
     const long long n = (long long)C.nx * C.ny * C.nz;
-    const float irt = 1.f / (NS == 2 ? sadd(rho.x, rho.y) : rho.x);
-    float fx = sfma(rho.x, C.g, F[0][0]), fy = F[0][1], fz = F[0][2];
-    if (NS == 2) fx = sadd(fx, sfma(rho.y, C.g, F[1][0])), fy = sadd(fy, F[1][1]), fz = sadd(fz, F[1][2]);
+    const float irt = 1.f / sadd(rho.x, rho.y);
+    const float fx = sadd(sfma(rho.x, C.g, F[0][0]), sfma(rho.y, C.g, F[1][0])), fy = sadd(F[0][1], F[1][1]),
+                fz = sadd(F[0][2], F[1][2]);
     if (out.rho) {
         out.rho[k] = wide3(rho.x);
-        if (NS == 2) out.rho[n + k] = wide3(rho.y);
+        out.rho[n + k] = wide3(rho.y);
     }
     if (out.u) {
         out.u[k] = wide3(smul(sfma(0.5f, fx, jx), irt));
@@ -1044,7 +1037,7 @@ __device__ __forceinline__ void look3(const Step3<float>& C, const float (&F)[2]
 // Populations of the state after streaming, from the moments, into f: what streams into each site,
 // population by population (k3_stream's terms).  O = float: the stored populations; double: the plain
 // values of lbm3_get_fields.
-template <int NS, typename O>
+template <typename O>
 __global__ void __launch_bounds__(128) k3_expand(const Mom3 M, int dc, O* __restrict__ f, const Step3<float> C) {
     const int x = blockIdx.x * 128 + threadIdx.x;
     if (x >= C.nx) return;
@@ -1082,11 +1075,11 @@ __global__ void __launch_bounds__(128) k3_expand(const Mom3 M, int dc, O* __rest
                 }
                 if constexpr (sizeof(O) == 4) {
                     f[l * C.plane + i] = v.x;
-                    if (NS == 2) f[(19 + l) * C.plane + i] = v.y;
+                    f[(19 + l) * C.plane + i] = v.y;
                 } else {
                     const long long n = (long long)C.nx * C.ny * C.nz, q = ((long long)z * C.ny + y) * C.nx + x;
                     f[l * n + q] = lbm::widen_fx(v.x) + w19<double>(l) * (double)C.rho_ref[0];
-                    if (NS == 2) f[(19 + l) * n + q] = lbm::widen_fx(v.y) + w19<double>(l) * (double)C.rho_ref[1];
+                    f[(19 + l) * n + q] = lbm::widen_fx(v.y) + w19<double>(l) * (double)C.rho_ref[1];
                 }
             }
         }
@@ -1191,10 +1184,9 @@ __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
         [&](int dx, int dy, int dz) { return S.box[1][bz + dz][by + dy][bx + dx]; }, F);
     if (sizeof(T) == 8) load();
     if constexpr (MODE == K3_LOOK)
-        look3<NS>(C, F, S.box[1][bz][by][bx], ((long long)z * C.ny + y) * C.nx + x, jx, jy, jz, flag,
-                 fields);
+        look3(C, F, S.box[1][bz][by][bx], ((long long)z * C.ny + y) * C.nx + x, jx, jy, jz, flag, fields);
     else if constexpr (MODE == K3_RELAX)
-        relax3<NS>(C, M, F, S.box[1][bz][by][bx], i, jx, jy, jz, d, flag);
+        relax3(C, M, F, S.box[1][bz][by][bx], i, jx, jy, jz, d, flag);
     else
         site3<T, NS, MODE>(C, f, F, x, y, z, i, fout, flag, fields);
 }
@@ -1248,12 +1240,9 @@ template <typename T>
 cudaError_t launch_step3_any(int mode, int ns, int shape, const CUtensorMap& map, const T* fin, T* fout,
                              const Step3<T>& C, int* flag, const Fields3& fields, const Mom3& M, int dn, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
-        if (mode == K3_RELAX)
-            return ns == 2 ? launch_shape<T, K3_RELAX, 2>(shape, map, fin, fout, C, flag, fields, M, dn, st)
-                           : launch_shape<T, K3_RELAX, 1>(shape, map, fin, fout, C, flag, fields, M, dn, st);
+        if (mode == K3_RELAX) return launch_shape<T, K3_RELAX, 2>(shape, map, fin, fout, C, flag, fields, M, dn, st);
         if (mode == K3_LOOK)
-            return ns == 2 ? launch_step3<T, K3_LOOK, 2, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st)
-                           : launch_step3<T, K3_LOOK, 1, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st);
+            return launch_step3<T, K3_LOOK, 2, Tile3<T>::ty(0), Tile3<T>::tz(0)>(map, fin, fout, C, flag, fields, M, dn, st);
     }
     if (mode == K3_WRITE)
         return ns == 2 ? launch_shape<T, K3_WRITE, 2>(shape, map, fin, fout, C, flag, fields, M, dn, st)
@@ -1283,9 +1272,9 @@ struct lbm3_ctx {
     void* vol = nullptr;               // psi and rho volumes: [2][gz][gy][gpitch] pairs
     alignas(64) unsigned char map[NSHAPE][128] = {};  // TMA descriptors of vol, per tile shape
     int shape = 0;                     // tile shape of the step pass (lbm3_autotune)
-    // FP32 at tau = 1: the state is held as moments (Mom3), which live in f[cur ^ 1], and f[cur] is
-    // stale; mom: that is so now; dc: which copy of the densities is current; chunk: k3_stream's
-    bool mom = false;
+    // FP32 at tau = 1: the state may be held as moments (Mom3), which live in f[cur ^ 1], and f[cur] is
+    // stale; may_mom: this lattice does; mom: that is so now; dc: which copy of the densities is current; chunk: k3_stream's
+    bool may_mom = false, mom = false;
     int dc = 0;
     int chunk = 1;
     int* flag = nullptr;
@@ -1509,6 +1498,15 @@ extern "C" int lbm3_create(lbm3_ctx** out, const lbm3_desc* d) {
             const long long blocks = columns * ((nz + k - 1) / k), cost = (blocks + slots - 1) / slots * (k + 2);
             if (best < 0 || cost < best) best = cost, c->chunk = k;
         }
+        // Which lattices are held as moments (a property of the lattice, so that the results' bits do not
+        // depend on how a run is cut into calls).  One species: none, a pair's second half would be idle
+        // (24 steps of 40^3 535 us as moments, 438 as populations; 128^3, 14 steps, 2,266 and 2,042).  Two:
+        // all but those whose blocks of one layer are a little more than run at once, where two layers a
+        // block leave a third of the slots empty and double its walk (24 steps of 36^3 533 and 508 us, 40^3
+        // 543 and 505, 160 x 24 x 24 567 and 515; below, 33^3 496 and 505; above, 128 x 32 x 32 567 and 573,
+        // 64^3 800 and 827, 96^3 1,823 and 2,374).
+        const long long layers = columns * nz;
+        c->may_mom = c->esize == 4 && ns == 2 && (layers <= slots || 2 * layers > 3 * slots);
     }
     const dim3 sg = stream_grid3(c);
     const size_t parts = std::max<size_t>(c->nblk_den, (size_t)sg.x * sg.y * sg.z);
@@ -1550,7 +1548,7 @@ extern "C" int lbm3_set_params(lbm3_ctx* c, const lbm_params* p) {
     // moments hold the state only under the relaxation times (all 1) and wall velocities it was formed
     // with (a population leaving through a wall is reflected by the step that sends it): under others
     // it goes on as the populations those give
-    const bool keep = p->tau[0] == 1.0 && (c->d.n_species == 1 || p->tau[1] == 1.0) &&
+    const bool keep = p->tau[0] == 1.0 && p->tau[1] == 1.0 &&
                       (c->d.z_boundary == LBM_PERIODIC || (p->wall_u[0] == was.wall_u[0] && p->wall_u[1] == was.wall_u[1]));
     if (c->mom && !keep) {
         CK3(cudaSetDevice(c->d.device));
@@ -1619,7 +1617,7 @@ extern "C" int lbm3_set_fields(lbm3_ctx* c, const double* rho, int where) {
 // the density pass over f[cur] into the volumes; totals: its block partials of the totals of
 // f[cur] summed into out (5 doubles, device memory) as well
 static Mom3 moments3(const lbm3_ctx* c) {
-    float* p = static_cast<float*>(c->f[c->cur ^ 1]);  // 15 planes of the 19 or 38
+    float* p = static_cast<float*>(c->f[c->cur ^ 1]);  // 15 planes of the 38
     const long long n = c->plane;
     Mom3 M;
     float2** pair[] = {&M.d[0], &M.d[1], &M.base, &M.ux, &M.uy, &M.uz};
@@ -1630,10 +1628,8 @@ static Mom3 moments3(const lbm3_ctx* c) {
     return M;
 }
 
-// Whether a step relaxes every population fully to its equilibrium (and the context holds FP32).
-static bool relaxed3(const lbm3_ctx* c) {
-    return c->d.precision == LBM_FP32 && c->c32.omega[0] == 1.0f && (c->d.n_species == 1 || c->c32.omega[1] == 1.0f);
-}
+// Whether a step relaxes every population fully to its equilibrium, on a lattice held as moments then.
+static bool relaxed3(const lbm3_ctx* c) { return c->may_mom && c->c32.omega[0] == 1.0f && c->c32.omega[1] == 1.0f; }
 
 static dim3 stream_grid3(const lbm3_ctx* c) {
     return dim3((c->d.nx + 31) / 32, (c->d.ny + 3) / 4, (c->d.nz + c->chunk - 1) / c->chunk);
@@ -1645,17 +1641,10 @@ static cudaError_t expand3(lbm3_ctx* c, double* out) {
     const dim3 grid((c->d.nx + 127) / 128, c->d.ny, c->d.nz);
     const Mom3 M = moments3(c);
     float* const f = (float*)c->f[c->cur];
-    if (c->d.n_species == 2) {
-        if (out)
-            k3_expand<2, double><<<grid, 128, 0, c->stream>>>(M, c->dc, out, c->c32);
-        else
-            k3_expand<2, float><<<grid, 128, 0, c->stream>>>(M, c->dc, f, c->c32);
-    } else {
-        if (out)
-            k3_expand<1, double><<<grid, 128, 0, c->stream>>>(M, c->dc, out, c->c32);
-        else
-            k3_expand<1, float><<<grid, 128, 0, c->stream>>>(M, c->dc, f, c->c32);
-    }
+    if (out)
+        k3_expand<double><<<grid, 128, 0, c->stream>>>(M, c->dc, out, c->c32);
+    else
+        k3_expand<float><<<grid, 128, 0, c->stream>>>(M, c->dc, f, c->c32);
     return cudaGetLastError();
 }
 
@@ -1665,12 +1654,8 @@ static cudaError_t stream3(lbm3_ctx* c, bool totals) {
     const dim3 grid = stream_grid3(c), block(32, 4);
     const Mom3 M = moments3(c);
     float* vol = (float*)c->vol;
-    if (c->d.n_species == 2)
-        return totals ? launch_pdl(k3_stream<2, true>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk, c->part)
-                      : launch_pdl(k3_stream<2, false>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk,
-                                   (double*)nullptr);
-    return totals ? launch_pdl(k3_stream<1, true>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk, c->part)
-                  : launch_pdl(k3_stream<1, false>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk,
+    return totals ? launch_pdl(k3_stream<true>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk, c->part)
+                  : launch_pdl(k3_stream<false>, grid, block, 0, c->stream, M, c->dc, vol, c->c32, c->chunk,
                                (double*)nullptr);
 }
 
