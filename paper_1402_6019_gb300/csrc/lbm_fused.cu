@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(128) k_fused(const T* __restrict__ fin, T* __r
             if (MODE & (M_WRITE | M_OBS)) {
                 const bool wall_row = C.zbc == 1 && (z == 0 || z == nz - 1);  // warp-uniform
                 if ((MODE & M_WRITE) || wall_row) {
-                    collide<T, NS>(C, f, drho, rho, ir, jx, jz, F);
+                    collide<T, NS, sizeof(T) == 8>(C, f, drho, rho, ir, jx, jz, F);
                     // streaming: f_l(x + c_l) = g_l(x), periodic in x, periodic or walls in z
                     const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
                     const long long rz0 = (long long)z * pitch;
