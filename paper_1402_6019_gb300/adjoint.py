@@ -11,8 +11,8 @@ The backward sweep needs every state f_n in reverse order.  Storing them all tak
 steps x 9 ns nx nz values, so the forward keeps an exact snapshot every `checkpoint` steps and
 the backward recomputes one segment at a time from its snapshot and sweeps it back
 (lbm_adjoint_sweep): device memory for ceil(steps / checkpoint) snapshots and `checkpoint` recorded
-states (twice that on small lattices, where the next segment is recorded meanwhile), and one
-extra forward run.
+states (twice that on small lattices where memory allows, the next segment recorded meanwhile), and
+one extra forward run.
 
 The adjoint runs in the lattice's precision unless told otherwise: an FP32 lattice records FP32
 states and sweeps an FP32 adjoint; the parameter derivatives are accumulated in FP64 either way.
@@ -26,7 +26,11 @@ import torch
 from . import lbm as L
 
 NPARAM = 8
-OVERLAP_SITES = 512 * 512  # largest lattice whose backward sweep overlaps two segments
+# Largest lattice whose backward sweep overlaps two segments: from there on a step's launches fill the
+# GPU.  Gradients of two species, one buffer / two, us (20 steps a segment): FP32 256^2, 100 steps,
+# 3,188 / 2,641; 384^2, 60 steps, 2,844 / 2,582; 512^2 3,776 / 3,720; 600^2, 40 steps, 3,493 / 3,497;
+# FP64 256^2 16,209 / 15,352, 512^2 30,923 / 30,547.
+OVERLAP_SITES = 512 * 512
 _KEYS = [("G1", 0), ("G1", 1), ("G2", 0), ("G2", 1), ("G_AB", None), ("tau", 0), ("tau", 1), ("body_force", None)]
 
 
@@ -62,6 +66,15 @@ def _handoff(device):
     torch.cuda.current_stream(device).synchronize()
 
 
+def overlaps(sites: int, segments: int, buffer_bytes: int, total_bytes: int, free_bytes) -> bool:
+    """Whether a backward sweep takes a second buffer of a segment's states: where overlapping two
+    segments pays, and the buffer is small beside the device's memory (1/64) or beside what is free of
+    it (1/4; free_bytes: a function, asked only then: it costs 50 us of host time)."""
+    if segments < 2 or sites > OVERLAP_SITES:
+        return False
+    return 64 * buffer_bytes <= total_bytes or 4 * buffer_bytes <= free_bytes()
+
+
 class Run:
     """The forward run of a gradient: snapshots every `checkpoint` steps and the final state."""
 
@@ -93,6 +106,18 @@ class Run:
         self.lat.synchronize()
         return J, g
 
+    def _second(self, seg: torch.Tensor):
+        """A second buffer like seg (the next segment's states are recorded into it while one is swept
+        back: the same results), or None."""
+        total = torch.cuda.get_device_properties(seg.device).total_memory
+        if not overlaps(self.lat.nx * self.lat.nz, len(self.snaps), seg.numel() * seg.element_size(), total,
+                        lambda: torch.cuda.mem_get_info(seg.device)[0]):
+            return None
+        try:
+            return torch.empty_like(seg)
+        except torch.cuda.OutOfMemoryError:
+            return None
+
     def backward(self, lam: torch.Tensor):
         """lam = dJ/df_steps; returns (dJ/drho_init [ns, nz, nx], dJ/dtheta [NPARAM]), FP64."""
         lat = self.lat
@@ -100,12 +125,18 @@ class Run:
         grad = torch.zeros(NPARAM, dtype=torch.float64, device=lam.device)
         shape = (min(self.checkpoint, max(self.steps, 1)),) + tuple(lam.shape)
         seg = torch.empty(shape, dtype=self.dtype, device=lam.device)
-        # a second segment's states, recorded while the first is swept back: where a step's launches do
-        # not fill the GPU (measured at 256 x 256: 552 -> 378 us per 25 steps)
-        seg2 = torch.empty_like(seg) if len(self.snaps) > 1 and lat.nx * lat.nz <= OVERLAP_SITES else None
+        seg2 = self._second(seg)
         _handoff(lam.device)
         nsteps = [min(self.checkpoint, self.steps - k * self.checkpoint) for k in range(len(self.snaps))]
-        L.lbm_adjoint_sweep(lat.h, self.snaps, nsteps, seg, seg2, lam, grad)
+        try:
+            L.lbm_adjoint_sweep(lat.h, self.snaps, nsteps, seg, seg2, lam, grad)
+        except L.LbmError as e:  # the library's own buffers, allocated before lam and grad are touched, didn't fit
+            if seg2 is None or e.code != L.LBM_ENOMEM:
+                raise
+            lat.synchronize()
+            seg2 = None
+            torch.cuda.empty_cache()
+            L.lbm_adjoint_sweep(lat.h, self.snaps, nsteps, seg, None, lam, grad)
         g_rho = torch.empty((lat.ns, lat.nz, lat.nx), dtype=torch.float64, device=lam.device)
         L.lbm_adjoint_initial(lat.h, lam, g_rho)
         lat.synchronize()

@@ -1464,12 +1464,23 @@ extern "C" int lbm_set_tile_shape(lbm_ctx* c, int width, int depth) {
 // ---------------------------------------------------------------------------------------
 // Discrete adjoint (periodic single lattice)
 // ---------------------------------------------------------------------------------------
+// One of the adjoint's device buffers, at its first use; a refusal leaves no error behind that a later
+// launch's check would read as its own.
+static int adjoint_buffer(lbm_ctx* c, void** p, size_t bytes) {
+    if (*p) return LBM_OK;
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaSuccess) return LBM_OK;
+    cudaGetLastError();
+    return fail(c, e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "adjoint buffer of %zu bytes: %s", bytes,
+                cudaGetErrorString(e));
+}
+
 static int adjoint_ready(lbm_ctx* c, AdjConst& A, int precision) {
     if (precision != LBM_FP64 && precision != LBM_FP32) return fail(c, LBM_EINVAL, "precision must be LBM_FP64 or LBM_FP32");
     if (c->d.z_boundary != LBM_PERIODIC) return fail(c, LBM_EINVAL, "the adjoint needs a periodic lattice");
     if (c->inst.size() > 1) return fail(c, LBM_EINVAL, "the adjoint is for a single lattice, not a batch");
     CK(cudaSetDevice(c->d.device));
-    if (!c->adj_scratch) CK(cudaMalloc(&c->adj_scratch, adjoint_scratch_bytes(c->d.nx, c->d.nz, c->d.n_species)));
+    if (int r = adjoint_buffer(c, &c->adj_scratch, adjoint_scratch_bytes(c->d.nx, c->d.nz, c->d.n_species))) return r;
     fill_adj_const(A, c->p, c->d.nx, c->d.nz, c->d.n_species, c->inst.empty() ? c->p.body_force : c->inst[0].g);
     return LBM_OK;
 }
@@ -1544,7 +1555,7 @@ extern "C" int lbm_adjoint_steps(lbm_ctx* c, int nsteps, const void* states, voi
     if (nsteps < 0 || !lam || !grad || (nsteps > 0 && !states)) return fail(c, LBM_EINVAL, "bad argument");
     AdjConst A;
     if (int r = adjoint_ready(c, A, precision)) return r;
-    if (!c->adj_lam) CK(cudaMalloc(&c->adj_lam, state_values(c) * sizeof(double)));
+    if (int r = adjoint_buffer(c, &c->adj_lam, state_values(c) * sizeof(double))) return r;
     // the first step writes the context's buffer, the second the caller's (read no more), ...
     if (precision == LBM_FP64)
         return adjoint_steps<double>(c, A, nsteps, (const double*)states, (const double*)lam, (double*)c->adj_lam,
