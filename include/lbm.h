@@ -371,12 +371,12 @@ int lbm_adjoint_steps(lbm_ctx *c, int nsteps, const void *states, void *lam, dou
 /* The whole backward sweep of a checkpointed run: segment k = nseg - 1 .. 0 starts from the snapshot
    snaps[k] (as lbm_restore_own takes it) and has nsteps[k] steps; its states are recorded
    (lbm_record_states) and swept back (lbm_adjoint_steps): lam and grad as there.  seg holds the
-   largest segment's states; with a second such buffer seg2 (NULL: none) the next segment's states are
-   recorded while one is swept back, on a stream of the context's own beside its stream, which
-   the call's work is ordered with as a whole: it starts after what is enqueued there and what is
-   enqueued after the call waits for it.  The results have the same bits either way; two
-   buffers pay where one step's launches do not fill the GPU.  Leaves the context's state as
-   recomputed for the first segment.  Asynchronous. */
+   largest segment's states; with a second such buffer seg2 (NULL: none; LBM_EINVAL where the two
+   overlap) the next segment's states are recorded while one is swept back, on a stream of the
+   context's own beside its stream, which the call's work is ordered with as a whole: it starts
+   after what is enqueued there and what is enqueued after the call waits for it.  The results have
+   the same bits either way; two buffers pay where one step's launches do not fill the GPU.  Leaves
+   the context's state as recomputed for the first segment.  Asynchronous. */
 int lbm_adjoint_sweep(lbm_ctx *c, int nseg, const void *const *snaps, const int *nsteps, void *seg, void *seg2,
                       void *lam, double *grad, int precision);
 

@@ -5,6 +5,7 @@
 // point returns a status; nothing throws across the ABI.
 #include <stdarg.h>
 #include <stddef.h>
+#include <stdint.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -1570,6 +1571,14 @@ extern "C" int lbm_adjoint_sweep(lbm_ctx* c, int nseg, const void* const* snaps,
     if (nseg < 0 || !lam || !grad || (nseg > 0 && (!snaps || !nsteps || !seg))) return fail(c, LBM_EINVAL, "bad argument");
     for (int k = 0; k < nseg; ++k)
         if (!snaps[k] || nsteps[k] < 0) return fail(c, LBM_EINVAL, "snaps[%d] is NULL or nsteps[%d] < 0", k, k);
+    if (precision != LBM_FP64 && precision != LBM_FP32) return fail(c, LBM_EINVAL, "precision must be LBM_FP64 or LBM_FP32");
+    if (seg2 && nseg > 0) {  // one is recorded while the other is swept back
+        size_t bytes = 0;
+        for (int k = 0; k < nseg; ++k) bytes = std::max(bytes, (size_t)nsteps[k]);
+        bytes *= state_values(c) * (precision == LBM_FP32 ? sizeof(float) : sizeof(double));
+        const uintptr_t a = reinterpret_cast<uintptr_t>(seg), b = reinterpret_cast<uintptr_t>(seg2);
+        if ((a < b ? b - a : a - b) < bytes) return fail(c, LBM_EINVAL, "seg and seg2 overlap");
+    }
     CK(cudaSetDevice(c->d.device));
     // one after the other: one buffer, one segment, or kernels timed by events on the stream
     if (!seg2 || nseg < 2 || c->profiling) {

@@ -368,9 +368,11 @@ def lbm_adjoint_sweep(h, snaps, nsteps, seg, seg2, lam, grad):
     """The backward sweep of a checkpointed run from its snapshots; seg, seg2 (or None): CUDA tensors
     for the largest segment's states; lam and grad as in lbm_adjoint_steps (asynchronous)."""
     n = len(snaps)
+    if len(nsteps) != n:
+        raise ValueError("as many step counts as snapshots are needed")
     ptrs = (_VP * n)(*[s.data_ptr() for s in snaps])
     counts = (ctypes.c_int * n)(*[int(k) for k in nsteps])
-    _check(load().lbm_adjoint_sweep(h, n, ptrs, counts, _dev(seg), _dev(seg2), _dev(lam), _dev(grad), _prec(seg, lam)), h)
+    _check(load().lbm_adjoint_sweep(h, n, ptrs, counts, _dev(seg), _dev(seg2), _dev(lam), _dev(grad), _prec(seg, seg2, lam)), h)
 
 
 def lbm_adjoint_objective(h, f, target_u, target_rho, J, dJdf=None):
