@@ -21,8 +21,8 @@
 //                  moments: lam_n; and the moments of f_{n-1} for the next step back.
 // k_adj_local and k_adj_final work on tiles of 32 x ATZ sites and stage their neighbourhood fields
 // (2 cells around the tile) in shared memory.  In FP64, bound by the FP64 pipe, antipodal links are
-// gathered shell by shell as in the forward step, psi's sums in fixed point (lbm_fixed.cuh), and lam
-// enters the collision's transpose through its six moments sum_l W_l lam_l (1, c, c c), formed of
+// gathered shell by shell as in the forward step, psi's sums in fixed point (lbm_fixed.cuh) on tiles
+// where every psi is a multiple of its unit (2^-5 and above; elsewhere in FP64), and lam enters the collision's transpose through its six moments sum_l W_l lam_l (1, c, c c), formed of
 // lam_l - lam_0.  In FP32, bound by latency, the sums stay link by link: the derivative of the body
 // force is a small difference that a run's rounding fixes to 1e-6 .. 1e-5 of itself, and other sums,
 // as exact, would land elsewhere in that range.
@@ -92,25 +92,18 @@ struct AdjC : AdjFixed<T> {
     T G_AB, g;
 };
 
-// psi as its field holds it: a value, or in FP64 with the exponential form the bits of psi on the 2^56
-// scale; psi_value the number; dpsi its derivative.
+// psi, and its derivative.
 __device__ __forceinline__ float psi_t(const AdjC<float>& A, int s, float r) {
     return A.psi_form == 1 ? r : -expm1f(-r * A.irho0[s]);
 }
 __device__ __forceinline__ double psi_t(const AdjC<double>& A, int s, double r) {
-    return A.psi_form == 1 ? r : of_bits((u64)psi_fx(r, A.ex[s]));
-}
-__device__ __forceinline__ float psi_value(const AdjC<float>&, float p) { return p; }
-__device__ __forceinline__ double psi_value(const AdjC<double>& A, double p) {
-    return A.psi_form == 1 ? p : scaled_double((i64)bits_of(p), -56);
+    return A.psi_form == 1 ? r : psi_number(r, A.irho0[s], A.ex[s]);
 }
 __device__ __forceinline__ float dpsi_t(const AdjC<float>& A, int s, float r) {
     return A.psi_form == 1 ? 1.f : expf(-r * A.irho0[s]) * A.irho0[s];
 }
 __device__ __forceinline__ double dpsi_t(const AdjC<double>& A, int s, double r) {
-    if (A.psi_form == 1) return 1.0;
-    if (!exp_fx_takes(r)) return exp(-r * A.irho0[s]) * A.irho0[s];
-    return scaled_double((i64)exp_fx(r, A.ex[s]), -62) * A.irho0[s];
+    return A.psi_form == 1 ? 1.0 : exp_number(r, A.irho0[s], A.ex[s]) * A.irho0[s];
 }
 
 // Block accumulators: FP64, or a double-float pair (hi, lo) summed with TwoSum on the FP32 pipes.
@@ -304,16 +297,39 @@ __global__ void __launch_bounds__(Tile<T>::NT) k_adj_local(const T* __restrict__
             jz[s] = B.jz[s * n + i];
         }
     }
+    bool small = false;  // a psi that the fixed-point sums would not hold exactly
+    const bool exponential = A.psi_form == 0;
     for (int k = tz * 32 + tx; k < TL::H * TL::W; k += TL::NT) {
         const int r = k / TL::W, c = k - r * TL::W;
         const int j = wrap_t(z0 - 2 + r, A.nz) * A.nx + wrap_t(x0 - 2 + c, A.nx);
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
-            ps[s][r][c] = B.psi[s * n + j];
+            T p = B.psi[s * n + j];
+            if constexpr (sizeof(T) == 8) {
+                if (exponential) {
+                    small = small || !(p >= PSI_SMALL);
+                    p = of_bits((u64)psi_bits57(p));
+                }
+            }
+            ps[s][r][c] = p;
             if (NS == 2) rh[s][r][c] = B.rho[s * n + j];
         }
     }
-    __syncthreads();
+    bool fixed = false;  // the tile holds psi's bits on the 2^57 scale (uniform)
+    if constexpr (sizeof(T) == 8) {
+        fixed = !__syncthreads_or(small) && exponential;
+        if (exponential && !fixed) {  // the numbers themselves
+            for (int k = tz * 32 + tx; k < TL::H * TL::W; k += TL::NT) {
+                const int r = k / TL::W, c = k - r * TL::W;
+                const int j = wrap_t(z0 - 2 + r, A.nz) * A.nx + wrap_t(x0 - 2 + c, A.nx);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) ps[s][r][c] = B.psi[s * n + j];
+            }
+            __syncthreads();
+        }
+    } else {
+        __syncthreads();
+    }
     T gp[NPAR] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (live) {
         // the force at the site, keeping its three sums (attraction a, repulsion p, cross b)
@@ -323,14 +339,15 @@ __global__ void __launch_bounds__(Tile<T>::NT) k_adj_local(const T* __restrict__
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
             const auto w = [&](int dx, int dz) { return ps[s][tz + 2 + dz][tx + 2 + dx]; };
-            psi[s] = psi_value(A, ps[s][tz + 2][tx + 2]);
+            psi[s] = ps[s][tz + 2][tx + 2];
             if (NS == 2)
                 rho[s] = rh[NS == 2 ? s : 0][tz + 2][tx + 2];
             else
                 rho[s] = B.rho[s * n + i];
             ax[s] = az[s] = px[s] = pz[s] = bx[s] = bz[s] = 0;
             if constexpr (sizeof(T) == 8) {
-                if (A.psi_form == 0) {  // uniform
+                if (fixed) {
+                    psi[s] = scaled_double((i64)bits_of(psi[s]), -57);
                     i64 sx[5], sz[5];
                     shell_sums([&](int dx, int dz) { return (i64)bits_of(w(dx, dz)); }, sx, sz);
                     DotFx dax, daz, dpx, dpz;
@@ -343,10 +360,10 @@ __global__ void __launch_bounds__(Tile<T>::NT) k_adj_local(const T* __restrict__
                         dpx.add(A.fr, q, sx[q]);
                         dpz.add(A.fr, q, sz[q]);
                     }
-                    ax[s] = scaled_double(dax.sum(), A.fa.e - 58);
-                    az[s] = scaled_double(daz.sum(), A.fa.e - 58);
-                    px[s] = scaled_double(dpx.sum(), A.fr.e - 58);
-                    pz[s] = scaled_double(dpz.sum(), A.fr.e - 58);
+                    ax[s] = scaled_double(dax.sum(), A.fa.e - 59);
+                    az[s] = scaled_double(daz.sum(), A.fa.e - 59);
+                    px[s] = scaled_double(dpx.sum(), A.fr.e - 59);
+                    pz[s] = scaled_double(dpz.sum(), A.fr.e - 59);
                 } else {
                     T sx[5], sz[5];
                     shell_sums(w, sx, sz);

@@ -198,7 +198,12 @@ LBM_FX unsigned mulhi32(unsigned a, unsigned b) {
 // take one-instruction products; five 64-bit products are left.  No branches: a thread's several
 // exponentials interleave.  About 80 integer instructions, against some 40 FP64 ones (640 cycles
 // of the SM's FP64 pipe per warp) for the division and the library's exponential.
-LBM_FX u64 exp_fx(double rho, const ExpFx& K) {
+//
+// exp_parts: q and n with exp(-rho / rho0) = q 2^(-62 - n), 2^61 <= q <= 2^62, and n = 64 where t is 64 or
+// more.  FINE keeps the fraction bits of t below 2^-57 too (within 2^-60 of the exponential then,
+// relatively, instead of 2^-57 of 1), for callers that need it as a number of its own.
+template <bool FINE>
+LBM_FX u64 exp_parts(double rho, const ExpFx& K, int& n) {
 #if defined(__CUDA_ARCH__)
     const u64* const table = exp2_table_dev;
 #else
@@ -209,8 +214,9 @@ LBM_FX u64 exp_fx(double rho, const ExpFx& K) {
     const u64 p = mulhi_u((b << 11) | (u64)1 << 63, K.km);  // t = p 2^(ex + ke - 1085)
     const int s = 1028 - ex - K.ke;                         // < 0: t >= 64, exp below 2^-63
     const u64 t = (s > 63 ? 0 : p >> (s & 63));
-    const int n = (int)(t >> 57);
-    const u64 R = t << 14;
+    n = s < 0 ? 64 : (int)(t >> 57);
+    u64 R = t << 14;
+    if (FINE && s >= 0) R = s < 14 ? p << (14 - s) : (s - 14 > 63 ? 0 : p >> (s - 14));
     const unsigned R32 = (unsigned)(R >> 32);
     // 1 - 2^-r = R (c1 - R (c2 - ...)), c_k = (ln 2)^k / k! 2^(-7 k) on the 2^64 scale
     unsigned w = 0xaec40u - mulhi32(R32, 0x286u);
@@ -219,12 +225,44 @@ LBM_FX u64 exp_fx(double rho, const ExpFx& K) {
     v = 0xf5fdeffc162cull - mulhi_u(R, v);
     v = 0x162e42fefa39ef3ull - mulhi_u(R, v);
     const u64 e = ((u64)1 << 63) - (mulhi_u(R, v) >> 1);  // 2^-r, 2^63 scale
-    const u64 q = mulhi_u(e, table[(t >> 50) & 127]) >> (n < 63 ? n : 63);
-    return s < 0 ? 0 : q;
+    return mulhi_u(e, table[(t >> 50) & 127]);
+}
+LBM_FX u64 exp_fx(double rho, const ExpFx& K) {
+    int n;
+    const u64 q = exp_parts<false>(rho, K, n);
+    return n < 64 ? q >> n : 0;
 }
 
 // Whether exp_fx takes rho: positive, finite, with room for the exponent arithmetic.
 LBM_FX bool exp_fx_takes(double rho) { return rho > 1e-290 && rho < 1e290; }
+
+// exp(-rho / rho0) and psi as numbers of their own, good to the last bit or two whatever their size, as the
+// library's exp and expm1 are (the fixed-point forms above are good to 2^-56 of 1): what a derivative
+// multiplies.  Those are called where the fixed-point form would be short of bits: small psi, whose
+// difference from 1 cancels, exponentials below 2^-64, and densities that exp_fx does not take.
+LBM_FX double exp_number(double rho, double inv_rho0, const ExpFx& K) {
+    if (exp_fx_takes(rho)) {
+        int n;
+        const u64 q = exp_parts<true>(rho, K, n);
+        if (n < 64) return scaled_double((i64)q, -62 - n);
+    }
+    return exp(-rho * inv_rho0);
+}
+constexpr double PSI_SMALL = 0.03125;  // 2^-5
+LBM_FX double psi_number(double rho, double inv_rho0, const ExpFx& K) {
+    if (exp_fx_takes(rho)) {
+        int n;
+        const u64 q = exp_parts<true>(rho, K, n);
+        const u64 v = ((u64)1 << 62) - (n < 64 ? q >> n : 0);
+        if (v >= (u64)1 << 57) return scaled_double((i64)v, -62);
+    }
+    return -expm1(-rho * inv_rho0);
+}
+// A psi of PSI_SMALL .. 1 on the 2^57 scale, which its FP64 value is a multiple of: exact.
+LBM_FX i64 psi_bits57(double psi) {
+    const u64 b = bits_of(psi);
+    return (i64)(((b & (((u64)1 << 52) - 1)) | (u64)1 << 52) << (((int)(b >> 52) - 1018) & 63));
+}
 
 // psi on the 2^56 scale; for a density that exp_fx does not take 1 or 0 (one that is <= 0, NaN or
 // Inf has been flagged; one below 1e-290 has psi = 0 to any precision held here)
@@ -263,7 +301,7 @@ inline void coef_fx(CoefFx<N>& F, const double* c) {
 }
 
 // sum_k c_k S_k of a few sums |S_k| < 2^60, exact in three accumulators of 29-bit limb products (each a
-// 32 x 32 -> 64 multiply-add), rounded once to the nearest: sum() 2^(e - 56) times the scale of S.
+// 32 x 32 -> 64 multiply-add), rounded once to the nearest: sum() 2^(e - 2) times the scale of S.
 // Rounding every product down instead would push each site the same way, a drift that adds up over
 // the steps; this is odd in S.  Room: with |c_k| <= 2^e and sum_k |S_k| <= 2^60.6 no accumulator
 // passes 2^62.7.
