@@ -174,6 +174,7 @@ template <>
 struct Fixed3<double> {
     lbm::ExpFx ex[2];
     lbm::CoefFx<7> kf[2];  // K_s(1, 2, 3, 4, 5, 6, 8)
+    int fixed;             // psi = 1 - exp(-rho / rho0) and every coefficient within coef_fx's range
 };
 
 template <typename T>
@@ -190,13 +191,15 @@ struct Step3 : Fixed3<T> {
     T kc[3];              // weight_norm G_AB w_cross(q), q = 1, 2 (zero for one species)
 };
 
-// psi as the volumes hold it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) the bits of psi on
-// the 2^PSI3_BITS scale.
+// psi as the volumes hold it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) (and couplings within
+// range: C.fixed) the bits of psi on the 2^PSI3_BITS scale.
 __device__ __forceinline__ float psi3(const Step3<float>& C, int s, float rho) {
     return C.psi_form == 1 ? rho : 1.0f - __expf(-rho * C.inv_rho0[s]);
 }
 __device__ __forceinline__ double psi3(const Step3<double>& C, int s, double rho) {
-    return C.psi_form == 1 ? rho : lbm::of_bits((lbm::u64)((lbm::psi_fx(rho, C.ex[s]) + 1) >> (56 - PSI3_BITS)));
+    if (C.psi_form == 1) return rho;
+    const lbm::i64 v = lbm::psi_fx(rho, C.ex[s]);
+    return C.fixed ? lbm::of_bits((lbm::u64)((v + 1) >> (56 - PSI3_BITS))) : lbm::scaled_double(v, -56);
 }
 
 __device__ __forceinline__ int wrap3(int i, int n) {
@@ -470,7 +473,7 @@ __device__ __forceinline__ void force3(const Step3<T>& C, const PSF& ps, const R
     const V zero = vsplat(T(0));
     V Fx, Fy, Fz;
     bool fixed = false;
-    if constexpr (sizeof(T) == 8) fixed = C.psi_form == 0;  // uniform
+    if constexpr (sizeof(T) == 8) fixed = C.fixed;  // uniform
     if (fixed) {
         if constexpr (sizeof(T) == 8) {
             double3 f0 = force3_fx(C.kf[0], [&](int dx, int dy, int dz) { return (lbm::i64)lbm::bits_of(PS(dx, dy, dz).x); });
@@ -1372,7 +1375,8 @@ static void fill_step3(const lbm3_ctx* c, Step3<T>& C) {
         if constexpr (sizeof(T) == 8) {
             C.ex[s] = lbm::exp_fx_const(c->p.psi_form == LBM_PSI_EXP ? c->p.rho0[ps] : 1.0);
             const double k[7] = {C.kq[s][1], C.kq[s][2], C.kq[s][3], C.kq[s][4], C.kq[s][5], C.kq[s][6], C.kq[s][8]};
-            lbm::coef_fx(C.kf[s], k);
+            const bool kept = lbm::coef_fx(C.kf[s], k);
+            C.fixed = c->p.psi_form == LBM_PSI_EXP && kept && (s == 0 || C.fixed);
         }
     }
     for (int q = 0; q < 3; ++q) C.kc[q] = c->d.n_species == 2 ? (T)(wn * c->p.G_AB * w_cross3(q)) : T(0);

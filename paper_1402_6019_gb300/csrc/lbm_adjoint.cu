@@ -82,6 +82,7 @@ struct AdjFixed<double> {
     double sa[5], sr[5], K[2][5];
     ExpFx ex[2];
     CoefFx<5> fa, fr;  // of sa and sr
+    int fixed;         // psi = 1 - exp(-rho / rho0) and the weights within coef_fx's range
 };
 
 template <typename T>
@@ -298,7 +299,8 @@ __global__ void __launch_bounds__(Tile<T>::NT) k_adj_local(const T* __restrict__
         }
     }
     bool small = false;  // a psi that the fixed-point sums would not hold exactly
-    const bool exponential = A.psi_form == 0;
+    bool bits = false;   // whether to try them at all (uniform)
+    if constexpr (sizeof(T) == 8) bits = A.fixed;
     for (int k = tz * 32 + tx; k < TL::H * TL::W; k += TL::NT) {
         const int r = k / TL::W, c = k - r * TL::W;
         const int j = wrap_t(z0 - 2 + r, A.nz) * A.nx + wrap_t(x0 - 2 + c, A.nx);
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(Tile<T>::NT) k_adj_local(const T* __restrict__
         for (int s = 0; s < NS; ++s) {
             T p = B.psi[s * n + j];
             if constexpr (sizeof(T) == 8) {
-                if (exponential) {
+                if (bits) {
                     small = small || !(p >= PSI_SMALL);
                     p = of_bits((u64)psi_bits57(p));
                 }
@@ -317,8 +319,8 @@ __global__ void __launch_bounds__(Tile<T>::NT) k_adj_local(const T* __restrict__
     }
     bool fixed = false;  // the tile holds psi's bits on the 2^57 scale (uniform)
     if constexpr (sizeof(T) == 8) {
-        fixed = !__syncthreads_or(small) && exponential;
-        if (exponential && !fixed) {  // the numbers themselves
+        fixed = !__syncthreads_or(small) && bits;
+        if (bits && !fixed) {  // the numbers themselves
             for (int k = tz * 32 + tx; k < TL::H * TL::W; k += TL::NT) {
                 const int r = k / TL::W, c = k - r * TL::W;
                 const int j = wrap_t(z0 - 2 + r, A.nz) * A.nx + wrap_t(x0 - 2 + c, A.nx);
@@ -721,8 +723,8 @@ AdjC<T> adj_const(const AdjConst& D) {
             A.sr[k] = c * D.wr[at[k]];
             for (int s = 0; s < 2; ++s) A.K[s][k] = D.G1[s] * A.sa[k] + D.G2[s] * A.sr[k];
         }
-        coef_fx(A.fa, A.sa);
-        coef_fx(A.fr, A.sr);
+        const bool kept = coef_fx(A.fa, A.sa), rep = coef_fx(A.fr, A.sr);
+        A.fixed = D.psi_form == 0 && kept && rep;
         for (int s = 0; s < 2; ++s) A.ex[s] = exp_fx_const(D.psi_form == 0 ? D.rho0[s] : 1.0);
     }
     for (int s = 0; s < 2; ++s) {

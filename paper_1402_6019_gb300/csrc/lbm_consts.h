@@ -74,8 +74,8 @@ inline void fill_step_const(StepConst<T>& C, const lbm_params& p, int nx, int nz
             C.ex[s] = exp_fx_const(p.psi_form == LBM_PSI_EXP ? p.rho0[ps] : 1.0);
             const double kf[5] = {K[1], K[2], 2.0 * K[4], K[5], 2.0 * K[8]};
             const double sf[5] = {0.5 * K[1], 0.5 * K[2], K[4], 0.25 * K[5], K[8]};
-            coef_fx(C.kf[s], kf);
-            coef_fx(C.sf[s], sf);
+            const bool kept = coef_fx(C.kf[s], kf), stress = coef_fx(C.sf[s], sf);
+            C.fixed = p.psi_form == LBM_PSI_EXP && kept && stress && (s == 0 || C.fixed);
         }
         for (int dz = -2; dz <= 2; ++dz)
             for (int dx = -2; dx <= 2; ++dx) {

@@ -283,10 +283,17 @@ struct CoefFx {
     int h[N], l[N];
     int e, pad;
 };
+// False, and all zero, for coefficients whose largest is not zero and outside 2^-900 .. 2^900 (or not
+// finite): the sums' exponents would leave FP64's range.  Those go through the FP64 forms.
 template <int N>
-inline void coef_fx(CoefFx<N>& F, const double* c) {
+inline bool coef_fx(CoefFx<N>& F, const double* c) {
+    F = CoefFx<N>{};
     double top = 0.0;
-    for (int k = 0; k < N; ++k) top = fabs(c[k]) > top ? fabs(c[k]) : top;
+    for (int k = 0; k < N; ++k) {
+        if (!isfinite(c[k])) return false;
+        top = fabs(c[k]) > top ? fabs(c[k]) : top;
+    }
+    if (top != 0.0 && (top < 0x1p-900 || top > 0x1p900)) return false;
     int e = 0;
     if (top > 0.0) (void)frexp(top, &e);  // top < 2^e
     for (int k = 0; k < N; ++k) {
@@ -297,7 +304,7 @@ inline void coef_fx(CoefFx<N>& F, const double* c) {
         F.l[k] = (int)(u & ((1 << 29) - 1));
     }
     F.e = e;
-    F.pad = 0;
+    return true;
 }
 
 // sum_k c_k S_k of a few sums |S_k| < 2^60, exact in three accumulators of 29-bit limb products (each a

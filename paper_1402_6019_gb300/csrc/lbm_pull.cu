@@ -215,11 +215,13 @@ __device__ __forceinline__ void gather_wall(const PullSmem<T, NS, ST, SHP>& S, i
         }
 }
 
-// psi as the psi/rho tile holds it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) the bits of
-// psi on the 2^56 scale (lbm_fixed.cuh), whose window sums phase B forms in integers.
+// psi as the psi/rho tile holds it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) (and couplings
+// within range: C.fixed) the bits of psi on the 2^56 scale (lbm_fixed.cuh), whose window sums phase B forms in integers.
 __device__ __forceinline__ float psi_tile(const StepConst<float>& C, int s, float rho) { return psi_of(C, s, rho); }
 __device__ __forceinline__ double psi_tile(const StepConst<double>& C, int s, double rho) {
-    return C.psi_form == 1 ? rho : of_bits((u64)psi_fx(rho, C.ex[s]));
+    if (C.psi_form == 1) return rho;
+    const i64 v = psi_fx(rho, C.ex[s]);
+    return C.fixed ? of_bits((u64)v) : scaled_double(v, -56);
 }
 
 // rho and psi at psi/rho tile position (px, pz) for a position that is not a live site of the
@@ -680,7 +682,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
 #pragma unroll
                     for (int dx = 0; dx < 5; ++dx) p[dz][dx] = Q.ps[s2][tz + dz][tx + dx];
                 if constexpr (sizeof(T) == 8) {
-                    if (C.psi_form == 0) {
+                    if (C.fixed) {
                         i64 w[5][5];
 #pragma unroll
                         for (int dz = 0; dz < 5; ++dz)

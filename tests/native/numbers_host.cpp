@@ -21,3 +21,7 @@ void number_exp(double rho, double rho0, double* out) {
 }
 long long number_bits57(double psi) { return psi_bits57(psi); }
 }
+extern "C" int coef_taken(const double* c) {
+    CoefFx<5> F;
+    return coef_fx(F, c);
+}

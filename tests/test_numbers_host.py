@@ -22,6 +22,7 @@ def numbers(tmp_path_factory):
     dp = ctypes.POINTER(ctypes.c_double)
     for f in (lib.number_psi, lib.number_exp):
         f.argtypes, f.restype = [ctypes.c_double, ctypes.c_double, dp], None
+    lib.coef_taken.argtypes, lib.coef_taken.restype = [dp], ctypes.c_int
     lib.number_bits57.argtypes, lib.number_bits57.restype = [ctypes.c_double], ctypes.c_longlong
     return lib
 
@@ -60,3 +61,11 @@ def test_a_psi_on_the_57_bit_scale_is_exact(numbers):
     for p in [2.0 ** -5, 1.0, math.nextafter(1.0, 0), math.nextafter(2.0 ** -5, 1), 0.5, math.nextafter(0.5, 0)] + \
             list(rng.uniform(2.0 ** -5, 1.0, 2000)) + list(2.0 ** rng.uniform(-5, 0, 2000)):
         assert numbers.number_bits57(p) * 2.0 ** -57 == p and math.ldexp(p, 57) == int(math.ldexp(p, 57))
+
+
+def test_couplings_beyond_the_fixed_point_range_are_refused(numbers):
+    for top, want in ((0.0, 1), (1.0, 1), (2.0 ** -900, 1), (2.0 ** -901, 0), (2.0 ** 900, 1), (2.0 ** 901, 0),
+                      (5e-324, 0), (1.7e308, 0), (math.inf, 0), (math.nan, 0)):
+        for c in ([top, 0, 0, 0, 0], [0.0, -top, 0, 0, 0], [0, 0, 0, 0, top]):
+            a = np.array(c, dtype=np.float64)
+            assert numbers.coef_taken(a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))) == want, c
