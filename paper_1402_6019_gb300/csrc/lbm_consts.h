@@ -75,7 +75,7 @@ inline void fill_step_const(StepConst<T>& C, const lbm_params& p, int nx, int nz
             const double kf[5] = {K[1], K[2], 2.0 * K[4], K[5], 2.0 * K[8]};
             const double sf[5] = {0.5 * K[1], 0.5 * K[2], K[4], 0.25 * K[5], K[8]};
             const bool kept = coef_fx(C.kf[s], kf), stress = coef_fx(C.sf[s], sf);
-            C.fixed = p.psi_form == LBM_PSI_EXP && kept && stress && (s == 0 || C.fixed);
+            if (p.psi_form == LBM_PSI_EXP) C.fixed = kept && stress && C.fixed >= 0 ? 1 : -1;
         }
         for (int dz = -2; dz <= 2; ++dz)
             for (int dx = -2; dx <= 2; ++dx) {

@@ -38,7 +38,7 @@ struct FixedConst<double> {
     ExpFx ex[2];     // psi = 1 - exp(-rho / rho0)
     CoefFx<5> kf[2];    // K(1), K(2), 2 K(4), K(5), 2 K(8) of Eq. FORCE
     CoefFx<5> sf[2];    // sq(1), sq(2), 4 sq(4), sq(5), 4 sq(8) of Appendix A
-    int fixed;          // psi = 1 - exp(-rho / rho0) and every coefficient within coef_fx's range
+    int fixed;          // psi = 1 - exp(-rho / rho0): 1, or -1 with a coefficient beyond coef_fx's range; else 0
 };
 
 // Per-step constants, passed to kernels by value (they live in the kernel-parameter

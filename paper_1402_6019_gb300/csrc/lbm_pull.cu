@@ -118,6 +118,7 @@ struct PullSmem {
     alignas(8) unsigned long long bar[ST];
     TileInfo<T> ti[NTQ];
     int fold_item;  // the reduction work item thread 0 drew for the CTA
+    int odd, numbers;  // FP64: the last iteration that may have met a density psi_fx does not take, that did
     unsigned short ring[SH::NT];  // observing builds: ring position of thread tid, rpz << 8 | rpx
 };
 
@@ -215,20 +216,41 @@ __device__ __forceinline__ void gather_wall(const PullSmem<T, NS, ST, SHP>& S, i
         }
 }
 
-// psi as the psi/rho tile holds it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) (and couplings
-// within range: C.fixed) the bits of psi on the 2^56 scale (lbm_fixed.cuh), whose window sums phase B forms in integers.
+// psi as phase A writes it into the psi/rho tile: a value, or in FP64 with psi = 1 - exp(-rho / rho0) the
+// bits of psi on the 2^56 scale (lbm_fixed.cuh), whose window sums phase B forms in integers.
 __device__ __forceinline__ float psi_tile(const StepConst<float>& C, int s, float rho) { return psi_of(C, s, rho); }
 __device__ __forceinline__ double psi_tile(const StepConst<double>& C, int s, double rho) {
-    if (C.psi_form == 1) return rho;
-    const i64 v = psi_fx(rho, C.ex[s]);
-    return C.fixed ? of_bits((u64)v) : scaled_double(v, -56);
+    return C.psi_form == 1 ? rho : of_bits((u64)psi_fx(rho, C.ex[s]));
+}
+// A density <= 0 or NaN has no such bits (0 stands there; a run may pass through such states, reported
+// but not stopped, and recover from them).  Whether this thread's share of a tile holds one that a site
+// of the lattice reads: the tile's first wx x wz positions.
+template <typename Tile>
+__device__ __noinline__ bool psi_beyond(const Tile& Q, int ns, int wx, int wz, int tid, int nt) {
+    constexpr int n = sizeof(Q.ps[0]) / sizeof(double), w = sizeof(Q.ps[0][0]) / sizeof(double);
+    bool found = false;
+    for (int s = 0; s < ns; ++s)
+        for (int k = tid; k < n; k += nt)
+            if (k % w < wx && k / w < wz && !((&Q.rh[s][0][0])[k] >= 0.0)) found = true;
+    return found;
+}
+// Such a tile's psi (and any tile's where the couplings are beyond the fixed-point range) as numbers,
+// from its densities, for the FP64 forms.
+template <typename Tile>
+__device__ __noinline__ void psi_as_numbers(Tile& Q, int ns, double rho0a, double rho0b, int tid, int nt) {
+    constexpr int n = sizeof(Q.ps[0]) / sizeof(double);
+    for (int s = 0; s < ns; ++s) {
+        const double rho0 = s == 0 ? rho0a : rho0b;
+        double *ps = &Q.ps[s][0][0], *rh = &Q.rh[s][0][0];
+        for (int k = tid; k < n; k += nt) ps[k] = 1.0 - exp(-rh[k] / rho0);
+    }
 }
 
 // rho and psi at psi/rho tile position (px, pz) for a position that is not a live site of the
 // tile: the ring, and the padding of ragged tiles.  With walls, rows beyond a wall take the
 // mirror image (or zero, Sec. IV's two readings of the ghost rows).  Positions that no live
 // site reads (far padding of ragged tiles) are set to zero.
-// side_sum returns false for those, else the sums of the populations there.
+// side_sum returns false for those (and 1s), else the sums of the populations there.
 template <typename T, int NS, int ST, int SHP>
 __device__ __forceinline__ bool side_sum(PullSmem<T, NS, ST, SHP>& S, int sl, const StepConst<T>& C, int px, int pz,
                                          int z0, int nz, bool WALL, T (&sum)[NS]) {
@@ -244,7 +266,7 @@ __device__ __forceinline__ bool side_sum(PullSmem<T, NS, ST, SHP>& S, int sl, co
     const int bz = Zs - z0 + 3, bx = px + 2;
     if (bz < 1 || bz > Shape<SHP>::BZ - 2) zero = true;
 #pragma unroll
-    for (int s = 0; s < NS; ++s) sum[s] = T(0);
+    for (int s = 0; s < NS; ++s) sum[s] = T(1);
     if (!zero) {
         T g[NS][9];
         const bool lo = WALL && Zs == 0, hi = WALL && Zs == nz - 1;
@@ -371,6 +393,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&S.bar[sl])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&tin) : "memory");
+        S.odd = S.numbers = -1;
         for (int sl = 0; sl < ST; ++sl) {
             const int t = (int)blockIdx.x + sl * (int)gridDim.x;
             if (t < nstat) describe<T, SHP>(S.ti[sl], t, ntiles, inst, ninst, ntx, rot, rev);
@@ -502,12 +525,17 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
                 has[r + 1] = false;
                 px[r + 1] = pz[r + 1] = 0;
 #pragma unroll
-                for (int s = 0; s < NS; ++s) sum[r + 1][s] = T(0);
+                for (int s = 0; s < NS; ++s) sum[r + 1][s] = T(1);  // some density; not stored
                 if (in[r + 1]) {
                     ring_position<SHP>(i, tid >> 5, px[r + 1], pz[r + 1]);
                     has[r + 1] = side_sum<T, NS, ST, SHP>(S, sl, C, px[r + 1], pz[r + 1], z0, lnz, WALL, sum[r + 1]);
                 }
             }
+#pragma unroll
+            for (int r = 0; r <= SH::RR; ++r)
+#pragma unroll
+                for (int s = 0; s < NS; ++s)  // (not > 0 and finite: its sign, or all of its exponent, set)
+                    if ((unsigned)(bits_of(C.rho_ref[s] + sum[r][s]) >> 32) - 1u >= 0x7fefffffu) S.odd = k;
             T ps[SH::RR + 1][NS];
 #pragma unroll
             for (int r = 0; r <= SH::RR; ++r)
@@ -536,6 +564,18 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
         if (__syncthreads_or(!ok)) {
             failed = true;
             break;
+        }
+        if constexpr (sizeof(T) == 8) {
+            if (S.odd == k || C.fixed < 0) {  // uniform
+                // positions past a ragged edge that no site reads hold anything
+                const TileInfo<T>& E = S.ti[k % NTQ];
+                const bool found = C.fixed < 0 || psi_beyond(S.q[qi], NS, nx + 4 - E.x0, E.lnz + 4 - E.z0, tid, SH::NT);
+                if (__syncthreads_or(found)) {
+                    psi_as_numbers(S.q[qi], NS, C.rho0[0], C.rho0[NS - 1], tid, SH::NT);
+                    if (tid == 0) S.numbers = k;
+                    __syncthreads();
+                }
+            }
         }
         if constexpr ((MODE & M_OBS) != 0) {
             const TileInfo<T>& E = S.ti[k % NTQ];
@@ -682,7 +722,7 @@ __global__ void __launch_bounds__(Shape<SHP>::NT,
 #pragma unroll
                     for (int dx = 0; dx < 5; ++dx) p[dz][dx] = Q.ps[s2][tz + dz][tx + dx];
                 if constexpr (sizeof(T) == 8) {
-                    if (C.fixed) {
+                    if (C.fixed > 0 && S.numbers != k) {  // uniform: the tile holds psi's bits
                         i64 w[5][5];
 #pragma unroll
                         for (int dz = 0; dz < 5; ++dz)
