@@ -174,7 +174,7 @@ template <>
 struct Fixed3<double> {
     lbm::ExpFx ex[2];
     lbm::CoefFx<7> kf[2];  // K_s(1, 2, 3, 4, 5, 6, 8)
-    int fixed;             // psi = 1 - exp(-rho / rho0) and every coefficient within coef_fx's range
+    int fixed;             // psi = 1 - exp(-rho / rho0): 1, or -1 with a coefficient beyond coef_fx's range; else 0
 };
 
 template <typename T>
@@ -191,15 +191,23 @@ struct Step3 : Fixed3<T> {
     T kc[3];              // weight_norm G_AB w_cross(q), q = 1, 2 (zero for one species)
 };
 
-// psi as the volumes hold it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) (and couplings within
-// range: C.fixed) the bits of psi on the 2^PSI3_BITS scale.
+// psi as the volumes hold it: a value, or in FP64 with psi = 1 - exp(-rho / rho0) the bits of psi on the
+// 2^PSI3_BITS scale.  A density <= 0 or NaN has no such bits (a run may pass through such states,
+// reported but not stopped, and recover from them): its psi stands there as a number, whose bits
+// are beyond the scale's 0 .. 2^PSI3_BITS, and psi3_number reads either.
 __device__ __forceinline__ float psi3(const Step3<float>& C, int s, float rho) {
     return C.psi_form == 1 ? rho : 1.0f - __expf(-rho * C.inv_rho0[s]);
 }
 __device__ __forceinline__ double psi3(const Step3<double>& C, int s, double rho) {
-    if (C.psi_form == 1) return rho;
-    const lbm::i64 v = lbm::psi_fx(rho, C.ex[s]);
-    return C.fixed ? lbm::of_bits((lbm::u64)((v + 1) >> (56 - PSI3_BITS))) : lbm::scaled_double(v, -56);
+    return C.psi_form == 1 ? rho : lbm::of_bits((lbm::u64)((lbm::psi_fx(rho, C.ex[s]) + 1) >> (56 - PSI3_BITS)));
+}
+__device__ __forceinline__ double psi3_number(double v) {
+    const lbm::u64 b = lbm::bits_of(v);
+    return b <= (lbm::u64)1 << PSI3_BITS ? lbm::scaled_double((lbm::i64)b, -PSI3_BITS) : v;
+}
+// Whether psi3 is to be the number: not > 0 and finite (its sign, or all of its exponent, set).
+__device__ __forceinline__ bool psi3_beyond(double rho) {
+    return (unsigned)(lbm::bits_of(rho) >> 32) - 1u >= 0x7fefffffu;
 }
 
 __device__ __forceinline__ int wrap3(int i, int n) {
@@ -275,11 +283,12 @@ struct DensityBlock {
 // 16 CTAs per SM for the plain FP32 pass (32 registers, as it ran fastest); 8 with the totals,
 // whose FP64 accumulators need up to 64 registers, and in FP64, so that neither spills
 // dn, jt (FP32, full relaxation, from populations; else null): the densities' deviations and the
-// momentum (three planes) for K3_RELAX.
+// momentum (three planes) for K3_RELAX.  odd (FP64): set where a density's psi had to be a number; it
+// stays set for the state's later steps, which take the FP64 forms then.
 template <typename T, bool TOT, bool MOM = false>
 __global__ void __launch_bounds__(128, TOT || MOM || sizeof(T) == 8 ? 8 : 16)
     k3_density(const T* __restrict__ f, T* __restrict__ vol, const Step3<T> C, double* __restrict__ part,
-               float2* __restrict__ dn = nullptr, float* __restrict__ jt = nullptr) {
+               float2* __restrict__ dn = nullptr, float* __restrict__ jt = nullptr, int* __restrict__ odd = nullptr) {
     using V = typename PairOf<T>::V;
     pdl_enter();
     using B = DensityBlock<T, TOT>;
@@ -306,6 +315,12 @@ __global__ void __launch_bounds__(128, TOT || MOM || sizeof(T) == 8 ? 8 : 16)
                 }
                 rho[s] = C.rho_ref[s] + a;
                 psi[s] = psi3(C, s, rho[s]);
+                if constexpr (sizeof(T) == 8) {
+                    if (C.fixed != 0 && psi3_beyond(rho[s])) {
+                        psi[s] = 1.0 - exp(-rho[s] / C.rho0[s]);
+                        atomicOr(odd, 1);
+                    }
+                }
                 if constexpr (TOT) {
                     if (s == 0)
                         mass0 += (double)a;
@@ -465,22 +480,28 @@ __device__ __forceinline__ double3 force3_fx(const lbm::CoefFx<7>& K, const PSF&
 // offset (dx, dy, dz) are ps(dx, dy, dz) and rh(dx, dy, dz).  LINKS: the cross force's sums link by link
 // from zero, as the two-species FP32 form on populations takes them: pairwise they are 18 additions
 // fewer, but there, short of registers, cost 3 % of a step (65 x 48 x 33: 17.9 us, 17.5 link by link).
+// fixed: psi's bits in fixed point (FP64; uniform).
 template <typename T, int NS, bool LINKS, typename PSF, typename RHF>
-__device__ __forceinline__ void force3(const Step3<T>& C, const PSF& ps, const RHF& rh, T (&F)[2][3]) {
+__device__ __forceinline__ void force3(const Step3<T>& C, bool fixed, const PSF& ps, const RHF& rh, T (&F)[2][3]) {
     using V = typename PairOf<T>::V;
-#define PS(dx, dy, dz) ps(dx, dy, dz)
+    const auto number = [&](int dx, int dy, int dz) {
+        V v = ps(dx, dy, dz);
+        if constexpr (sizeof(T) == 8) {
+            if (C.fixed != 0) v.x = psi3_number(v.x), v.y = psi3_number(v.y);
+        }
+        return v;
+    };
+#define PS(dx, dy, dz) number(dx, dy, dz)
 #define RH(dx, dy, dz) rh(dx, dy, dz)
     const V zero = vsplat(T(0));
     V Fx, Fy, Fz;
-    bool fixed = false;
-    if constexpr (sizeof(T) == 8) fixed = C.fixed;  // uniform
-    if (fixed) {
+    if (sizeof(T) == 8 && fixed) {
         if constexpr (sizeof(T) == 8) {
-            double3 f0 = force3_fx(C.kf[0], [&](int dx, int dy, int dz) { return (lbm::i64)lbm::bits_of(PS(dx, dy, dz).x); });
+            double3 f0 = force3_fx(C.kf[0], [&](int dx, int dy, int dz) { return (lbm::i64)lbm::bits_of(ps(dx, dy, dz).x); });
             Fx.x = f0.x, Fy.x = f0.y, Fz.x = f0.z;
             Fx.y = Fy.y = Fz.y = 0.0;
             if constexpr (NS == 2) {
-                f0 = force3_fx(C.kf[1], [&](int dx, int dy, int dz) { return (lbm::i64)lbm::bits_of(PS(dx, dy, dz).y); });
+                f0 = force3_fx(C.kf[1], [&](int dx, int dy, int dz) { return (lbm::i64)lbm::bits_of(ps(dx, dy, dz).y); });
                 Fx.y = f0.x, Fy.y = f0.y, Fz.y = f0.z;
             }
         }
@@ -1202,8 +1223,10 @@ __global__ void __launch_bounds__(Tile3<T>::TX* TY* TZ,
 
     const int bx = tx + GX, by = ty + GY, bz = tz + GZ;
     T F[2][3];
+    bool fixed = false;
+    if constexpr (sizeof(T) == 8) fixed = C.fixed > 0 && __ldcg(flag + 1) == 0;
     force3<T, NS, sizeof(T) == 4 && MODE == K3_WRITE>(
-        C, [&](int dx, int dy, int dz) { return S.box[0][bz + dz][by + dy][bx + dx]; },
+        C, fixed, [&](int dx, int dy, int dz) { return S.box[0][bz + dz][by + dy][bx + dx]; },
         [&](int dx, int dy, int dz) { return S.box[1][bz + dz][by + dy][bx + dx]; }, F);
     if (sizeof(T) == 8) load();
     if constexpr (MODE == K3_LOOK)
@@ -1300,7 +1323,7 @@ struct lbm3_ctx {
     bool may_mom = false, mom = false;
     int dc = 0;
     int chunk = 1;
-    int* flag = nullptr;
+    int* flag = nullptr;               // [0] what lbm3_synchronize reports, [1] k3_density's odd
     double* staging = nullptr;         // lbm3_get_fields / lbm3_set_fields from the host
     size_t staging_bytes = 0;
     double* part = nullptr;            // the density pass's block partials of the totals
@@ -1376,7 +1399,7 @@ static void fill_step3(const lbm3_ctx* c, Step3<T>& C) {
             C.ex[s] = lbm::exp_fx_const(c->p.psi_form == LBM_PSI_EXP ? c->p.rho0[ps] : 1.0);
             const double k[7] = {C.kq[s][1], C.kq[s][2], C.kq[s][3], C.kq[s][4], C.kq[s][5], C.kq[s][6], C.kq[s][8]};
             const bool kept = lbm::coef_fx(C.kf[s], k);
-            C.fixed = c->p.psi_form == LBM_PSI_EXP && kept && (s == 0 || C.fixed);
+            if (c->p.psi_form == LBM_PSI_EXP) C.fixed = kept && C.fixed >= 0 ? 1 : -1;
         }
     }
     for (int q = 0; q < 3; ++q) C.kc[q] = c->d.n_species == 2 ? (T)(wn * c->p.G_AB * w_cross3(q)) : T(0);
@@ -1491,8 +1514,8 @@ extern "C" int lbm3_create(lbm3_ctx** out, const lbm3_desc* d) {
     const size_t vbytes = (size_t)2 * c->gvol * 2 * c->esize;
     CKC3(cudaMalloc(&c->vol, vbytes));
     CKC3(cudaMemsetAsync(c->vol, 0, vbytes, c->stream));
-    CKC3(cudaMalloc(&c->flag, sizeof(int)));
-    CKC3(cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
+    CKC3(cudaMalloc(&c->flag, 2 * sizeof(int)));
+    CKC3(cudaMemsetAsync(c->flag, 0, 2 * sizeof(int), c->stream));
     int nsm = 0;
     CKC3(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, d->device));
     {  // the density pass with totals: no more than the 8 CTAs that run on an SM, each looping over as many
@@ -1629,7 +1652,7 @@ extern "C" int lbm3_set_fields(lbm3_ctx* c, const double* rho, int where) {
     else
         lbm3::k3_init<float><<<blocks, 256, 0, c->stream>>>((float*)c->f[0], c->staging, c->c32);
     CK3(cudaGetLastError());
-    CK3(cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
+    CK3(cudaMemsetAsync(c->flag, 0, 2 * sizeof(int), c->stream));
     CK3(cudaStreamSynchronize(c->stream));
     c->cur = 0;
     c->mom = false;
@@ -1691,24 +1714,24 @@ static cudaError_t density3(lbm3_ctx* c, double* totals = nullptr, bool read = f
     cudaError_t e;
     if (c->d.precision == LBM_FP64)
         e = totals ? launch_pdl(lbm3::k3_density<double, true>, grid, block, 0, c->stream, (const double*)c->f[c->cur],
-                                (double*)c->vol, c->c64, c->part, (float2*)nullptr, (float*)nullptr)
+                                (double*)c->vol, c->c64, c->part, (float2*)nullptr, (float*)nullptr, c->flag + 1)
                    : launch_pdl(lbm3::k3_density<double, false>, grid, block, 0, c->stream,
                                 (const double*)c->f[c->cur], (double*)c->vol, c->c64, (double*)nullptr,
-                                (float2*)nullptr, (float*)nullptr);
+                                (float2*)nullptr, (float*)nullptr, c->flag + 1);
     else if (c->mom && !read) {
         e = stream3(c, totals != nullptr);
     } else if (relaxed3(c) && !read) {  // populations, on the way to moments
         const Mom3 M = moments3(c);
         e = totals ? launch_pdl(lbm3::k3_density<float, true, true>, grid, block, 0, c->stream,
-                                (const float*)c->f[c->cur], (float*)c->vol, c->c32, c->part, M.d[c->dc ^ 1], M.jx)
+                                (const float*)c->f[c->cur], (float*)c->vol, c->c32, c->part, M.d[c->dc ^ 1], M.jx, (int*)nullptr)
                    : launch_pdl(lbm3::k3_density<float, false, true>, grid, block, 0, c->stream,
                                 (const float*)c->f[c->cur], (float*)c->vol, c->c32, (double*)nullptr, M.d[c->dc ^ 1],
-                                M.jx);
+                                M.jx, (int*)nullptr);
     } else {
         e = totals ? launch_pdl(lbm3::k3_density<float, true>, grid, block, 0, c->stream, (const float*)c->f[c->cur],
-                                (float*)c->vol, c->c32, c->part, (float2*)nullptr, (float*)nullptr)
+                                (float*)c->vol, c->c32, c->part, (float2*)nullptr, (float*)nullptr, (int*)nullptr)
                    : launch_pdl(lbm3::k3_density<float, false>, grid, block, 0, c->stream, (const float*)c->f[c->cur],
-                                (float*)c->vol, c->c32, (double*)nullptr, (float2*)nullptr, (float*)nullptr);
+                                (float*)c->vol, c->c32, (double*)nullptr, (float2*)nullptr, (float*)nullptr, (int*)nullptr);
     }
     if (e != cudaSuccess || !totals) return e;
     const dim3 sg = stream_grid3(c);
@@ -1986,7 +2009,7 @@ extern "C" int lbm3_autotune(lbm3_ctx* c, int steps, int* chosen, double* ms) {
     c->step = step0;
     c->shape = e == cudaSuccess ? best : shape0;
     CK3(e);
-    CK3(cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
+    CK3(cudaMemsetAsync(c->flag, 0, 2 * sizeof(int), c->stream));
     if (chosen) *chosen = best;
     if (ms)
         for (int k = 0; k < NSHAPE; ++k) ms[k] = t[k];
