@@ -64,12 +64,13 @@ struct ExportBase {
 // A stored value and its base W_l rho_ref added and rounded to O.  FP32 to FP32 stays off the FP64
 // pipe, which its two conversions and the add kept busy for three quarters of the export: the base is
 // split into two floats and added with its rounding error (two_sum), so the sum is the FP64 one
-// rounded (but for a tie in 2^-24 of the cases).
+// rounded (but for a tie in 2^-24 of the cases).  An infinite value stays what it is: its rounding error is
+// not a number.
 template <typename T, typename O>
 __device__ __forceinline__ O plain_value(T v, double base, float hi, float lo) {
     if constexpr (sizeof(T) == 4 && sizeof(O) == 4) {
         const float2 s = two_sum(hi, v);
-        return s.x + (s.y + lo);
+        return fabsf(s.x) < INFINITY ? s.x + (s.y + lo) : s.x;
     } else if constexpr (sizeof(T) == 4) {
         return (O)(widen_fx(v) + base);
     } else {
