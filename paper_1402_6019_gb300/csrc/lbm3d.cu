@@ -19,9 +19,10 @@
 // (each population read and written once).  Populations are SoA f[s][l][z][y][x] (rows padded
 // to 32), FP32 deviations f - W_l rho_ref,s or plain FP64.
 //
-// Full relaxation (two species in FP32, tau = 1 for both; lbm3_create says which lattices) needs no populations: the collision leaves
-// f*_l = feq_l(rho_s, u_s), so the density and velocity after it (4 numbers per species, held as 5)
-// are the whole state, and a step only needs the density and momentum of what streams in.
+// Full relaxation (two species in FP32, tau = 1 for both; lbm3_create says which lattices) needs no
+// populations: the collision leaves f*_l = feq_l(rho_s, u_s), so the density and velocity after it (4
+// numbers per species, held as 5) are the whole state, and a step only needs the density and
+// momentum of what streams in.
 //  * k3_stream evaluates, at every site, the 19 equilibria that stream in from the neighbours'
 //    moments, and writes their density and momentum (and the psi / rho volumes);
 //  * k3_step in its K3_RELAX form takes the force from the volumes and writes the new density and velocity.
@@ -863,8 +864,8 @@ __device__ __forceinline__ void wall_in(Sum3& S, const Col3& c, float uw) {
 // three layers they stream to, so a site costs 37 (chunk + 2) / chunk reads instead of 67.  The
 // order of the additions (from below, from the same layer, from above) is the same whatever the
 // chunk.  With TOT the block's FP64 partials of the state's totals too (as k3_density's).
-// Bound by instruction issue and L1 (about 240 instructions and 300 B of reads per site) with the
-// whole state in L2 at 128^3.
+// About 240 instructions and 300 B of L1 reads per site with the whole state in L2 at 128^3, 66.6 us a
+// step there; a block's layers are read one after the other, and the layer ahead prefetched.
 template <bool TOT>
 __global__ void __launch_bounds__(128, 4)
     k3_stream(const Mom3 M, int dc, float* __restrict__ vol, const Step3<float> C, int chunk, double* __restrict__ part) {

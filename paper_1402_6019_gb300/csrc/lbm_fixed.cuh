@@ -7,7 +7,8 @@
 // about 8, so exact sums and bounded products cost a small fraction of their FP64 forms and run
 // beside the FP64 work that is left.
 // psi = 1 - exp(-rho / rho0) lies in [0, 1] for every density > 0, which gives its sums and
-// products a range known beforehand; nothing here depends on the size of rho.
+// products a range known beforehand; nothing here depends on the size of rho.  A density <= 0 (a state
+// that a run may pass through) has no psi in that range: the steps take the FP64 forms for it.
 //
 // Precision: psi is held with 2^-56 resolution (1 - exp(-x) in FP64 has an error of up to 2^-53
 // whatever its size, that of the exponential), sums and differences are exact, the force is rounded
@@ -264,8 +265,8 @@ LBM_FX i64 psi_bits57(double psi) {
     return (i64)(((b & (((u64)1 << 52) - 1)) | (u64)1 << 52) << (((int)(b >> 52) - 1018) & 63));
 }
 
-// psi on the 2^56 scale; for a density that exp_fx does not take 1 or 0 (one that is <= 0, NaN or
-// Inf has been flagged; one below 1e-290 has psi = 0 to any precision held here)
+// psi on the 2^56 scale; for a density that exp_fx does not take 1 or 0 (callers look at one that is <= 0
+// or NaN themselves; one below 1e-290 has psi = 0 to any precision held here)
 LBM_FX i64 psi_fx(double rho, const ExpFx& K) {
     const i64 v = (i64)((((u64)1 << 62) - exp_fx(rho, K) + 32) >> 6);
     const bool big = rho >= 1e290;
